@@ -19,6 +19,7 @@ the repository's benchmark and tests.  `op` says which part a case is:
 Sizes of ragged batches come from the case (`shape_seed`), so that its work is known; everything else comes from
 the seed that `prepare` is given.
 """
+import heapq
 import math
 import random
 
@@ -166,6 +167,142 @@ def tolerance(case):
     if case["op"] == "grow":
         return {"rel": 1e-6, "max": 1e-5}
     return {"rel": 1e-2, "max": 0.1, "differ": 0.005}
+
+
+# ---- the same results in 64 bits, in plain torch and numpy ------------------------------------------------------
+def _ancestors(parents):
+    """[n, n] truth values: row i sees itself and its ancestors."""
+    see = np.eye(len(parents), dtype=bool)
+    for i, p in enumerate(parents):
+        if p >= 0:
+            see[i] |= see[p]
+    return see
+
+
+def _preorder(parents):
+    """Parent array after renumbering by a depth-first walk that takes children in index order."""
+    children = [[] for _ in parents]
+    for i, p in enumerate(parents):
+        if p >= 0:
+            children[p].append(i)
+    todo, new = [i for i, p in enumerate(parents) if p < 0][::-1], {}
+    while todo:
+        i = todo.pop()
+        new[i] = len(new)
+        todo += children[i][::-1]
+    out = np.zeros(len(parents), dtype=np.int64)
+    for i, k in new.items():
+        out[k] = new[parents[i]] if parents[i] >= 0 else -1
+    return out
+
+
+def _attention64(q, k, v, prefix_rows, tree_rows, see):
+    """One request's tree attention: the prefix, then the tree's own rows under `see`."""
+    g, rows = q.shape[1] // k.shape[1], torch.cat([prefix_rows, tree_rows])
+    out = torch.empty(q.shape, dtype=torch.float64, device=DEV)
+    hidden = torch.cat([torch.zeros((len(q), len(prefix_rows)), dtype=torch.bool, device=DEV), ~see], dim=1)
+    for h in range(q.shape[1]):
+        s = (q[:, h].double() @ k[rows, h // g].double().T) * q.shape[2] ** -0.5
+        out[:, h] = torch.softmax(s.masked_fill_(hidden, -math.inf), dim=1) @ v[rows, h // g].double()
+    return out
+
+
+def _rows_of(case, Ls, ns, seed):
+    """Per request: cache rows of the prefix tokens, cache rows of the tree."""
+    ar, got = np.arange, []
+    if case.get("layout") == "contiguous":
+        first = [sum(Ls[:r]) + sum(ns[:r]) for r in range(len(Ls))]
+        got = [(f + ar(L), f + L + ar(n)) for f, L, n in zip(first, Ls, ns)]
+    else:
+        page, inside = case["page"], case.get("layout") == "in_pages"
+        table, tree0, _ = _pages(seed, Ls, ns, page, inside)
+        for r, (L, n) in enumerate(zip(Ls, ns)):
+            t = ar(L + n)
+            at = table[r, t // page].astype(np.int64) * page + t % page
+            got.append((at[:L], at[L:] if inside else tree0[r] + ar(n)))
+    return [tuple(torch.from_numpy(x.astype(np.int64)).to(DEV) for x in pair) for pair in got]
+
+
+def _batch64(case, s, seed, Ls, ns, parents):
+    rows, offs, outs = _rows_of(case, Ls, ns, seed), np.concatenate([[0], np.cumsum(ns)]), []
+    see = [torch.from_numpy(_ancestors(parents[offs[r]:offs[r + 1]])).to(DEV) for r in range(len(ns))]
+    for q, k, v, _ in s["layers"]:
+        outs.append(torch.cat([_attention64(q[offs[r]:offs[r + 1]], k, v, *rows[r], see[r]) for r in range(len(ns))]))
+    return outs
+
+
+def _grow64(case, s):
+    """Algorithms 1 and 2 in fp64: value a node was drawn at, and value of the first draw under it."""
+    T, V, U = case["rows"], case["vocab"], s["uniforms"].cpu().numpy()
+    table, S = s["table"].cpu().numpy().astype(np.float64), case["m"] + 1
+    values, childs = np.zeros((case["n_req"], S)), np.zeros((case["n_req"], S))
+    parents = np.zeros((case["n_req"], S), dtype=np.int64)
+    for r, root in enumerate(s["root"].cpu().numpy()):
+        row, left, n = [int(root)], {}, 1
+        values[r, 0] = childs[r, 0] = 1.0
+        parents[r, 0] = -1
+
+        def sample(pos, attempt, v):
+            nonlocal n
+            p = left.setdefault(pos, table[row[pos]].copy())
+            cum = np.cumsum(p)
+            y = min(int(np.searchsorted(cum, float(U[(row[pos] * 7919 + attempt * 104729 + 17) % len(U)]) * cum[-1], side="right")), V - 1)
+            share = p[y] / cum[-1] if cum[-1] > 0 else 0.0
+            p[y] = 0.0
+            row.append(((row[pos] * 2654435761 + (y + 1) * 40503) % (1 << 32)) % T)
+            parents[r, n], values[r, n], childs[r, n] = pos, v, v * share
+            n += 1
+            return share
+
+        if case["algo"] == "greedy":
+            heap, pushed = [(-1.0, 0, 0, 0)], 1
+            while n < S and heap:
+                v, _, pos, attempt = heapq.heappop(heap)
+                share = sample(pos, attempt, -v)
+                if 1.0 - share > 0.0:
+                    heapq.heappush(heap, (v * (1.0 - share), pushed, pos, attempt + 1))
+                heapq.heappush(heap, (v * share, pushed + 1, n - 1, 0))
+                pushed += 2
+        else:
+            pos = 0
+            while pos < n and n < S:
+                v, attempt = childs[r, pos], 0
+                while v >= np.float32(case["threshold"]) and n < S:
+                    share = sample(pos, attempt, v)
+                    v, attempt = v * (1.0 - share), attempt + 1
+                    if not 1.0 - share > 0.0:
+                        break
+                left.pop(pos, None)
+                pos += 1
+    return parents, values, childs
+
+
+def exact(case, seed):
+    op = case["op"]
+    if op == "verify":              # token and node numbers
+        return None
+    s = prepare(case, seed)
+    if op == "grow":
+        _, values, childs = _grow64(case, s)
+        return [None, None, values, childs, None, None]
+    if op == "attend":
+        Ls, ns = _sizes(case)
+        parents = s["parents"].cpu().numpy()
+        if case["dfs"]:
+            parents = _preorder(parents)
+        return _batch64(case, s, seed, Ls, ns, parents) + [None] * (5 if case["dfs"] else 3)
+    if op == "loop":
+        outs, n = [], s["n"]
+        for L, parents, _, layers in s["steps"]:
+            see = torch.from_numpy(_ancestors(parents.cpu().numpy())).to(DEV)
+            at = torch.arange(L + n, device=DEV)
+            outs += [_attention64(q, k, v, at[:L], at[L:], see) for (q, _), (k, v) in zip(layers, s["caches"])]
+        return outs
+    parents, values, _ = _grow64(dict(case, algo="greedy", threshold=0.0), s)
+    outs = [None, None, values] + [None] * 8
+    for out in _batch64(case, s, seed, s["Ls"], s["ns"], parents.reshape(-1)):
+        outs += [None, None, out]   # the cache after compaction: copies of its own rows
+    return outs
 
 
 # ---- set-up --------------------------------------------------------------------------------------------------------
