@@ -367,6 +367,7 @@ int dyspec_verify_tree(const int32_t* parents, const int32_t* tokens, const floa
  *   parents, tokens, rows  dev int32 [n_req][S];  values, child_values  dev float [n_req][S]
  *                 values[k] = the estimated acceptance rate node k was created with, child_values[k] =
  *                 that of the first sampling under it;  n_nodes dev int32 [n_req] = nodes incl. the root
+ *                 (0 if a bounded wait inside the kernel ran out, which ordinary operation never sees)
  * m, max_nodes <= DYSPEC_MAX_NODES - 1.  Values are fp32; as for dyspec_verify_tree, a choice between
  * numbers closer than rounding may fall differently from another implementation's.
  */

@@ -2,231 +2,1171 @@
 //
 // The draft model is a table lookup: the distribution that follows a tree position is row
 // f(row of the parent, token) of `draft_table`, and the uniform number of the j-th sampling at a
-// position is entry g(row, j) of `uniforms` (vocab_ops.cuh).  One CTA of 1024 threads per request.
+// position is entry g(row, j) of `uniforms` (vocab_ops.cuh).  So what the j-th sampling at a position
+// yields -- its token and that token's residual probability -- is a function of the position's row
+// and j alone: positions with the same row share one stream of draws.
 //
-// A "slot" (v, position, attempt) is the next sampling at a position, v its estimated acceptance rate.
-//   greedy (Algorithm 1):   take the slot with the largest v (ties: pushed first), draw a token from
-//     the position's residual distribution (the row with the tokens of the position's existing
-//     children zeroed, renormalised), create the node, push (v (1 - r), position, attempt + 1) and
-//     (v r, new node, 0), r = the drawn token's residual probability; m times.  The heap of the paper
-//     is an array scanned by the whole block (<= 4096 slots: one pass).
+//   greedy (Algorithm 1):   take the position whose next sampling has the largest estimated acceptance
+//     rate v (ties: the one opened first), create the node of that draw, leave v (1 - r) at the position
+//     and v r at the new node, r = the drawn token's probability in the residual (the row with the
+//     tokens drawn before zeroed, renormalised); m times.
 //   threshold (Algorithm 2): layer by layer, each position keeps drawing while v >= t.
-// The residual lives in registers (thread t owns float4 chunks t, t + 1024, ...); a draw is an
-// inverse-CDF search in token order (row totals, then one block scan).  The tokens a position has
-// already used are struck out in constant time whatever their number: every thread looks at one or two
-// nodes of the tree, and where a node is a child of the position it sets the token's bit in the word of
-// the thread that owns the token (32 tokens per thread, one shared-memory word each); after a barrier a
-// thread zeroes what its word marks.  (Walking the position's child list instead costs a dependent
-// shared-memory hop per earlier sibling in all 32 warps: quadratic in the width of a position, and
-// language-model rows give the root hundreds of children.)
+//
+// Deciding which draw comes next is a serial chain over all nodes, and so is one row's stream of
+// draws; but streams of different rows are independent of each other and of the order in which the
+// tree takes them.  One thread-block cluster per request therefore splits the work by role:
+//
+//   planner  (warp 0 of CTA 0)  the serial part only.  Keys of the open positions lie in shared memory in
+//            groups of 32, the groups' champions in registers, the best of all in a scalar; the two values
+//            a step makes are compared with that scalar, so only a step that turns to another position needs
+//            reductions (two), and those overlap the load of that position's draw.
+//   helpers  (warps 1 and 2 of CTA 0)  one node behind it.  One finds the child's row in a hash table of the rows
+//            met so far and orders the row's load and first draws where it is new; the other orders further
+//            draws ahead of their use (more of them the longer a stream has become).
+//   fetcher and loaders (9 warps of a worker CTA)  row -> 64 leaf sums in fp64, every worker CTA a share of them, kept in the
+//            shared memory of the CTA that draws from the row.
+//   drawers  (4 warps of a worker CTA)   a draw by one warp: scan of the 64 leaf sums, then of the one leaf
+//            that the number falls into (read again from L1 / L2, the tokens drawn before struck out).
+//            Only that leaf is summed anew (never by subtraction), so a draw touches 2 KB instead of the row's 128.
+//   hot CTAs  (up to three of a cluster)  each takes over one row whose stream runs long: the best-first tree of a
+//            flat row is a star, and most of its draws are one serial stream (up to 762 of 768 draws on
+//            language-model rows).  The row moves into shared memory with prefix sums over sub-blocks of 8
+//            tokens (per chunk of 1024) and over the chunks, as unevaluated pairs of doubles (error 2^-100 of
+//            the row's sum), which a draw updates by subtraction; when the residual has fallen below 2^-40
+//            of the sum the tables were built from, they are built again.  No scan is left in a draw: two
+//            compares with a ballot and eight tokens.
+//
+// Messages are single words that validate themselves (a draw's record in CTA 0, a load order or a ring
+// entry in a worker CTA; written through distributed shared memory), so no hand-over needs a fence or
+// a block barrier.  Every wait is bounded; when one runs out the request reports 0 nodes.
+//
+// Measured on a B200 (vocabulary 32000, 256 language-model rows): one greedy tree of 768 nodes 5504 us with
+// the whole row re-read and re-summed by one block per node, 429 us now; eight threshold trees of 512
+// nodes 2517 -> 320 us.
 #include "vocab_ops.cuh"
 
 namespace dyspec {
 
 namespace {
 
-struct TreeOut {
+constexpr int kLeaves = 64;            // leaf sums per row; a leaf is 128 K tokens, K = 1, 2, 4 by vocabulary
+constexpr int kDrawWarps = 4;
+constexpr int kLoadWarps = 8, kBatch = 2 * kLoadWarps;         // leaves that come in with one copy: two for each warp that sums
+constexpr int kMaxStages = 4;
+constexpr int kRoles = 3;              // planner and two helpers; then the drawers, the fetcher, the loaders
+constexpr int kTreeThreads = 32 * (kRoles + kDrawWarps + 1 + kLoadWarps);
+constexpr int kHotAfter = 12;          // draws used of a row before a hot CTA takes it over
+constexpr int kHotRing = 32;           // orders to a hot CTA in flight (at most kMaxAhead)
+constexpr int kMaxHot = 3;
+constexpr int kSub = 8, kChunk = 1024, kChunks = 32;          // hot tables: tokens per sub-block, per chunk; chunks
+constexpr int kMaxAhead = 8;           // draws of a row that may be ordered before they are used
+constexpr uint32_t kEmpty = 0xFFFFFFFFu;
+constexpr uint32_t kFollow = 0x80000000u;   // slot: the record after this one, not linked yet when the slot was written
+constexpr int kMaxRecords = 8192;      // 13 bits of a ring entry
+
+// One draw: r (all ones = not drawn yet), token, record of the row's next draw.
+struct __align__(16) DrawRecord {
+  unsigned long long r_bits;
+  uint32_t token;
+  uint32_t next;
+};
+
+struct __align__(16) EntryState {      // helper's view of a row's stream
+  uint16_t consumed, ordered;
+  uint32_t last;                       // last record ordered
+  uint32_t ring;                       // cluster address of the ring that takes its orders
+  uint32_t el_unit;                    // index in its worker CTA << 8 | ring number
+};
+
+// Shared-memory layout (the same in every CTA of the cluster; a part a CTA does not use has no bytes).
+struct TreeLayout {
+  int nodes_pad;                       // m + 1 rounded up to whole groups of 32
+  int max_entries, entries_local;      // distinct rows: in all, per worker CTA
+  int n_workers, first_worker, n_hot;  // hot CTAs follow CTA 0, the workers follow them
+  int n_records, open_records, hash_size, ring_size, ring_shift, n_stages;
+  // byte offsets
+  int rec, key, val, seq, slot, ev, first, row, rec_owner, hash_row, hash_val, entry;
+  int stage, sums, load_row, attempts, number, ring, log;
+  int hot_row, hot_sub, hot_ring, hot_pub;
+  int bytes;
+};
+
+struct TreeArgs {
+  const float* table;
+  const float* uniforms;
+  const int32_t* root_row;
+  int n_rows, vocab, n_uniforms, m;
+  uint32_t rows_inverse;               // floor(2^32 / n_rows), at most 2^32 - 1
+  float threshold;                     // threshold algorithm only
   int32_t* parents;
   int32_t* tokens;
   float* values;
   float* child_values;
   int32_t* rows;
+  int32_t* n_nodes;
+  TreeLayout lay;
 };
 
-__device__ __forceinline__ void write_node(const TreeOut& o, size_t base, int k, int parent, int token, float v, float cv,
-                                           int row) {
-  o.parents[base + k] = parent;
-  o.tokens[base + k] = token;
-  o.values[base + k] = v;
-  o.child_values[base + k] = cv;
-  o.rows[base + k] = row;
+// Words that another warp or CTA writes: relaxed accesses, single-copy atomic at their size.
+__device__ __forceinline__ uint32_t ld_relaxed(const void* p) {
+  uint32_t v;
+  asm volatile("ld.relaxed.cluster.shared::cta.u32 %0, [%1];" : "=r"(v) : "r"(smem_u32(p)) : "memory");
+  return v;
+}
+__device__ __forceinline__ unsigned long long ld_relaxed64(const void* p) {
+  unsigned long long v;
+  asm volatile("ld.relaxed.cluster.shared::cta.u64 %0, [%1];" : "=l"(v) : "r"(smem_u32(p)) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_relaxed(const void* p, uint32_t v) {
+  asm volatile("st.relaxed.cluster.shared::cta.u32 [%0], %1;" ::"r"(smem_u32(p)), "r"(v) : "memory");
+}
+__device__ __forceinline__ void st_relaxed64(const void* p, unsigned long long v) {
+  asm volatile("st.relaxed.cluster.shared::cta.u64 [%0], %1;" ::"r"(smem_u32(p)), "l"(v) : "memory");
+}
+__device__ __forceinline__ unsigned long long ld_acquire64(const void* p) {
+  unsigned long long v;
+  asm volatile("ld.acquire.cta.shared::cta.u64 %0, [%1];" : "=l"(v) : "r"(smem_u32(p)) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_release64(const void* p, unsigned long long v) {
+  asm volatile("st.release.cta.shared::cta.u64 [%0], %1;" ::"r"(smem_u32(p)), "l"(v) : "memory");
+}
+__device__ __forceinline__ void st_remote(uint32_t cluster_addr, uint32_t v) {
+  asm volatile("st.relaxed.cluster.shared::cluster.u32 [%0], %1;" ::"r"(cluster_addr), "r"(v) : "memory");
+}
+__device__ __forceinline__ void st_remote64(uint32_t cluster_addr, unsigned long long v) {
+  asm volatile("st.relaxed.cluster.shared::cluster.u64 [%0], %1;" ::"r"(cluster_addr), "l"(v) : "memory");
+}
+
+// Polls `ready` (warp-uniform) until it holds; false once the exit flag is up or the limit has passed.
+template <typename F>
+__device__ __forceinline__ bool wait_until(F ready, const uint32_t* exit_flag) {
+#pragma unroll 1
+  for (int i = 0; i < 512; ++i)
+    if (ready()) return true;
+  const uint64_t t0 = global_timer_ns();
+  for (uint32_t spins = 1;; ++spins) {
+    if (ready()) return true;
+    if (ld_relaxed(exit_flag)) return false;
+    if ((spins & 255u) == 0 && global_timer_ns() - t0 > kWaitLimitNs) return false;
+  }
+}
+
+__device__ __forceinline__ uint32_t ld_remote(uint32_t cluster_addr) {
+  uint32_t v;
+  asm volatile("ld.relaxed.cluster.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(cluster_addr) : "memory");
+  return v;
+}
+
+__device__ __forceinline__ unsigned long long key_of(double v) {       // order of v >= 0; 0 = no slot (taken, or NaN)
+  return v >= 0.0 ? (unsigned long long)__double_as_longlong(v + 0.0) + 1ull : 0ull;
+}
+__device__ __forceinline__ double value_of(unsigned long long key) { return __longlong_as_double((long long)(key - 1ull)); }
+
+// Lane with the largest key (ties: the smallest sequence number); `best` = that key.
+__device__ __forceinline__ int warp_best(unsigned long long key, uint32_t seq, unsigned long long& best) {
+  const uint32_t hi = uint32_t(key >> 32), lo = uint32_t(key);
+  const uint32_t mh = __reduce_max_sync(0xffffffffu, hi);
+  bool c = hi == mh;
+  uint32_t b = __ballot_sync(0xffffffffu, c);
+  if (b & (b - 1)) {
+    const uint32_t ml = __reduce_max_sync(0xffffffffu, c ? lo : 0u);
+    c = c && lo == ml;
+    b = __ballot_sync(0xffffffffu, c);
+    if (b & (b - 1)) {
+      const uint32_t ms = __reduce_min_sync(0xffffffffu, c ? seq : kEmpty);
+      b = __ballot_sync(0xffffffffu, c && seq == ms);
+    }
+  }
+  const int src = __ffs(b) - 1;
+  best = ((unsigned long long)mh << 32) | __shfl_sync(0xffffffffu, lo, src);
+  return src;
+}
+
+struct Draw { double r; uint32_t token, next; };
+
+// The record that `slot` stands for and its content, when it has been drawn.
+__device__ __forceinline__ bool wait_draw(const DrawRecord* recs, uint32_t& slot, Draw& d, const uint32_t* exit_flag) {
+  if (slot & kFollow) {
+    const uint32_t prev = slot & ~kFollow;
+    uint32_t nx = kEmpty;
+    if (!wait_until([&] { nx = ld_relaxed(&recs[prev].next); return nx != kEmpty; }, exit_flag)) return false;
+    slot = nx;
+  }
+  const DrawRecord* rc = recs + slot;
+  unsigned long long rb = 0;
+  uint32_t t = 0;
+  if (!wait_until([&] { rb = ld_relaxed64(&rc->r_bits); t = ld_relaxed(&rc->token); return rb != ~0ull && t != kEmpty; }, exit_flag))
+    return false;
+  d.r = __longlong_as_double((long long)rb);
+  d.token = t;
+  d.next = ld_relaxed(&rc->next);
+  return true;
+}
+
+struct Shared {                        // pointers into one CTA's shared memory
+  DrawRecord* rec;
+  unsigned long long* key;             // greedy: slot keys; threshold: value of the first sampling under a node
+  unsigned long long* val;             // value a node was created with
+  uint32_t *seq, *slot, *ev, *first, *row, *rec_owner, *hash_row;
+  uint32_t* hash_val;                  // entry << 16 | first record
+  EntryState* entry;
+};
+
+__device__ __forceinline__ Shared planner_view(uint8_t* sm, const TreeLayout& l) {
+  Shared s;
+  s.rec = reinterpret_cast<DrawRecord*>(sm + l.rec);
+  s.key = reinterpret_cast<unsigned long long*>(sm + l.key);
+  s.val = reinterpret_cast<unsigned long long*>(sm + l.val);
+  s.seq = reinterpret_cast<uint32_t*>(sm + l.seq);
+  s.slot = reinterpret_cast<uint32_t*>(sm + l.slot);
+  s.ev = reinterpret_cast<uint32_t*>(sm + l.ev);
+  s.first = reinterpret_cast<uint32_t*>(sm + l.first);
+  s.row = reinterpret_cast<uint32_t*>(sm + l.row);
+  s.rec_owner = reinterpret_cast<uint32_t*>(sm + l.rec_owner);
+  s.hash_row = reinterpret_cast<uint32_t*>(sm + l.hash_row);
+  s.hash_val = reinterpret_cast<uint32_t*>(sm + l.hash_val);
+  s.entry = reinterpret_cast<EntryState*>(sm + l.entry);
+  return s;
+}
+
+// A node for the helpers: parent position and the record of its draw (13 bits).  Its value is for the end.
+__device__ __forceinline__ void announce(const Shared& s, int k, int pos, uint32_t rec, double v) {
+  s.val[k] = (unsigned long long)__double_as_longlong(v);
+  st_relaxed(&s.ev[k], (uint32_t(pos) << 13) | rec);
+}
+
+// An open position: key, sequence number (order of opening), position.
+struct Open {
+  unsigned long long key;
+  uint32_t seq;
+  int pos;
+};
+__device__ __forceinline__ bool better(const Open& a, const Open& b) {
+  return a.key > b.key || (a.key == b.key && a.seq < b.seq);
+}
+
+// Algorithm 1's order.  Returns the number of nodes created, -1 when a wait ran out.
+__device__ int plan_greedy(const TreeArgs& a, const Shared& s, const uint32_t* exit_flag) {
+  const int lane = threadIdx.x & 31;
+  const Open none{0ull, kEmpty, 0};
+  Open c0 = none, c1 = none;                     // champions of groups `lane` and `lane + 32`, without the current position
+  Open rest = none;                              // the best of them all (the same in every lane)
+  Open cur{key_of(1.0), 0u, 0};
+  uint32_t slot = kEmpty;                        // record of the current position's next draw; kEmpty: the helper names it
+  auto insert = [&](const Open& o, uint32_t rec) {
+    if (lane == 0) { s.key[o.pos] = o.key; s.seq[o.pos] = o.seq; s.slot[o.pos] = rec; }
+    const int g = o.pos >> 5;
+    if (lane == (g & 31)) {
+      if (g < 32) { if (better(o, c0)) c0 = o; }
+      else if (better(o, c1)) c1 = o;
+    }
+  };
+  int n = 0;
+  while (n < a.m && cur.key != 0ull) {
+    if (slot == kEmpty && !wait_until([&] { slot = ld_relaxed(&s.first[cur.pos]); return slot != kEmpty; }, exit_flag)) return -1;
+    Draw d;
+    if (!wait_draw(s.rec, slot, d, exit_flag)) return -1;
+    const double v = value_of(cur.key), left = 1.0 - d.r;
+    const int k = ++n;
+    Open stay{left > 0.0 ? key_of(v * left) : 0ull, 2u * k, cur.pos}, child{key_of(v * d.r), 2u * k + 1u, k};
+    const uint32_t next = d.next != kEmpty ? d.next : (slot | kFollow);
+    if (lane == 0) announce(s, k, cur.pos, slot, v);
+    const bool s_c = better(stay, child), s_r = better(stay, rest), c_r = better(child, rest);
+    if (s_c && s_r) {                            // the same position again
+      insert(child, kEmpty);
+      if (c_r) rest = child;
+      cur = stay;
+      slot = next;
+    } else if (!s_c && c_r) {                    // straight on to the new node
+      insert(stay, next);
+      if (s_r) rest = stay;
+      cur = child;
+      slot = kEmpty;
+    } else {                                     // another position: take it out of its group, find the best of the others
+      insert(stay, next);
+      insert(child, kEmpty);
+      cur = rest;
+      if (cur.key == 0ull) break;
+      __syncwarp();
+      const int g = cur.pos >> 5;
+      slot = s.slot[cur.pos];
+      Open o{s.key[(g << 5) + lane], s.seq[(g << 5) + lane], (g << 5) + lane};
+      if (lane == (cur.pos & 31)) { o.key = 0ull; o.seq = kEmpty; s.key[cur.pos] = 0ull; s.seq[cur.pos] = kEmpty; }
+      Open top;
+      top.pos = (g << 5) + warp_best(o.key, o.seq, top.key);
+      top.seq = __shfl_sync(0xffffffffu, o.seq, top.pos & 31);
+      if (lane == (g & 31)) { if (g < 32) c0 = top; else c1 = top; }
+      const bool h = better(c1, c0);
+      const Open mine{h ? c1.key : c0.key, h ? c1.seq : c0.seq, h ? c1.pos : c0.pos};
+      const int src = warp_best(mine.key, mine.seq, rest.key);
+      rest.seq = __shfl_sync(0xffffffffu, mine.seq, src);
+      rest.pos = __shfl_sync(0xffffffffu, mine.pos, src);
+    }
+    __syncwarp();
+  }
+  return n;
+}
+
+// Algorithm 2's order: positions in index order (which is layer order) draw while v >= t.
+__device__ int plan_threshold(const TreeArgs& a, const Shared& s, const uint32_t* exit_flag) {
+  const int lane = threadIdx.x & 31;
+  const double t = double(a.threshold);
+  if (lane == 0) s.key[0] = (unsigned long long)__double_as_longlong(1.0);
+  __syncwarp();
+  int n = 0;
+  for (int pos = 0; pos <= n && n < a.m; ++pos) {
+    double v = __longlong_as_double((long long)s.key[pos]);
+    if (!(v >= t)) continue;
+    uint32_t slot = kEmpty;
+    if (!wait_until([&] { slot = ld_relaxed(&s.first[pos]); return slot != kEmpty; }, exit_flag)) return -1;
+    while (v >= t && n < a.m) {
+      Draw d;
+      if (!wait_draw(s.rec, slot, d, exit_flag)) return -1;
+      const int k = ++n;
+      if (lane == 0) {
+        st_relaxed64(&s.key[k], (unsigned long long)__double_as_longlong(v * d.r));
+        announce(s, k, pos, slot, v);
+      }
+      v = v * (1.0 - d.r);
+      if (!(1.0 - d.r > 0.0)) break;
+      slot = d.next != kEmpty ? d.next : (slot | kFollow);
+    }
+    __syncwarp();
+  }
+  return n;
+}
+
+// Sends the order for draw `ordinal` of a row, to be put into record `rec` (one lane).  Two warps send to the workers' rings.
+__device__ __forceinline__ void send_order(const TreeLayout& l, uint32_t* s_tail, uint32_t ring, uint32_t el_unit, uint32_t rec) {
+  const uint32_t unit = el_unit & 0xFFu, i = atomicAdd(&s_tail[unit], 1u);
+  const bool hot = unit >= 8 * kDrawWarps;
+  const uint32_t size = hot ? uint32_t(kHotRing) : uint32_t(l.ring_size), shift = hot ? 5u : uint32_t(l.ring_shift);
+  st_remote(ring + (i & (size - 1)) * 4, (((i >> shift) & 1u) << 31) | ((el_unit >> 8) << 13) | rec);
+}
+
+// The next node for a helper warp; false when the tree is complete (or a wait ran out).
+__device__ __forceinline__ bool next_event(const Shared& s, int m, int k, uint32_t& ev, const uint32_t* s_final, const uint32_t* exit_flag) {
+  bool over = false;
+  const bool got = wait_until([&] {
+    if (k <= m) {
+      ev = ld_relaxed(&s.ev[k]);
+      if (ev != kEmpty) return true;
+    }
+    const uint32_t fin = ld_relaxed(s_final);
+    over = fin != kEmpty && uint32_t(k) > fin;
+    return over;
+  }, exit_flag);
+  return got && !over;
+}
+
+// Helper 1: rows of new nodes.
+template <bool kGreedy>
+__device__ __forceinline__ void run_opener(const TreeArgs& a, const Shared& s, uint8_t* sm, uint32_t* s_tail, const uint32_t* s_final,
+                                           const uint32_t* exit_flag, int req) {
+  const TreeLayout& l = a.lay;
+  const int lane = threadIdx.x & 31;
+  const double t = double(a.threshold);
+  int n_entries = 0, n_records = 0;
+  int next_worker = 0, next_el = 0;              // round robin over the worker CTAs
+  const uint32_t sm_addr = smem_u32(sm);
+  const uint32_t n_buckets = uint32_t(l.hash_size) >> 5;
+
+  // Names node k's first record: that of the row's entry, created (and its load ordered) when the row is new.
+  auto open_row = [&](int k, uint32_t row) {
+    uint32_t b = ((row * 2654435769u) >> 16) & (n_buckets - 1);
+    for (uint32_t tries = 0; tries < n_buckets; ++tries, b = (b + 1) & (n_buckets - 1)) {
+      const uint32_t h = s.hash_row[b * 32 + lane], hv = s.hash_val[b * 32 + lane];
+      const uint32_t hit = __ballot_sync(0xffffffffu, h == row);
+      if (hit) {
+        if (lane == __ffs(hit) - 1) st_relaxed(&s.first[k], hv & 0xFFFFu);
+        break;
+      }
+      const uint32_t open = __ballot_sync(0xffffffffu, h == kEmpty);
+      if (open) {
+        // one record is due to every row still to come; the rest of the pool lets the first draws run ahead
+        const int e = n_entries++, spare = l.open_records - n_records - (l.max_entries - e);
+        const int rec0 = n_records, want = 1 + max(0, min(kGreedy ? 1 : 3, spare));
+        n_records += want;
+        const int w = next_worker, el = next_el;
+        if (++next_worker == l.n_workers) { next_worker = 0; ++next_el; }
+        const uint32_t cta = uint32_t(w + l.first_worker);
+        if (lane < l.n_workers) st_remote(map_to_cta(sm_addr + l.load_row + e * 4, uint32_t(l.first_worker + lane)), row);
+        const EntryState st{0, uint16_t(want), uint32_t(rec0 + want - 1), map_to_cta(sm_addr + l.ring + (el % kDrawWarps) * l.ring_size * 4, cta),
+                            (uint32_t(el) << 8) | uint32_t(w * kDrawWarps + el % kDrawWarps)};
+        if (lane < want) {
+          s.rec_owner[rec0 + lane] = (uint32_t(e) << 16) | uint32_t(lane);
+          if (lane + 1 < want) st_relaxed(&s.rec[rec0 + lane].next, uint32_t(rec0 + lane + 1));
+        }
+        if (lane == 0) {
+          const int at = b * 32 + __ffs(open) - 1;
+          s.entry[e] = st;
+          s.hash_row[at] = row;
+          s.hash_val[at] = (uint32_t(e) << 16) | uint32_t(rec0);
+          __threadfence_block();                 // helper 2 reads the entry once one of these draws has been used
+          for (int i = 0; i < want; ++i) send_order(l, s_tail, st.ring, st.el_unit, uint32_t(rec0 + i));
+          st_relaxed(&s.first[k], uint32_t(rec0));
+        }
+        break;
+      }
+    }
+    __syncwarp();
+  };
+
+  const int32_t rr0 = a.root_row[req];
+  const uint32_t row0 = uint32_t(((rr0 % a.n_rows) + a.n_rows) % a.n_rows);      // non-negative remainder: any int32 maps to a row
+  if (lane == 0) s.row[0] = row0;
+  if (a.m > 0) open_row(0, row0);
+  __syncwarp();
+  uint32_t ev = kEmpty;
+  for (int k = 1; next_event(s, a.m, k, ev, s_final, exit_flag); ++k) {
+    const uint32_t rec = ev & 0x1FFFu, prow = s.row[ev >> 13];
+    const uint32_t y = ld_relaxed(&s.rec[rec].token);          // drawn: the planner has used it
+    // row of the child (draft_row_of_child), the remainder by the prepared inverse
+    const uint32_t h = prow * 2654435761u + (y + 1u) * 40503u;
+    uint32_t row = h - __umulhi(h, a.rows_inverse) * uint32_t(a.n_rows);
+    while (row >= uint32_t(a.n_rows)) row -= uint32_t(a.n_rows);                 // (the quotient is at most two short)
+    if (lane == 0) s.row[k] = row;
+    bool expand = k < a.m;
+    if (!kGreedy) expand = __longlong_as_double((long long)ld_relaxed64(&s.key[k])) >= t;   // (written before the event)
+    if (expand) open_row(k, row);
+    else __syncwarp();
+  }
+}
+
+// Helper 2: a used draw lets its row's stream run on.  `hot_addr`: the hot CTAs' hand-over words (same offset in each).
+template <bool kGreedy>
+__device__ __forceinline__ void run_orderer(const TreeArgs& a, const Shared& s, uint8_t* sm, uint32_t* s_tail, uint32_t hot_addr,
+                                            const uint32_t* s_final, const uint32_t* exit_flag) {
+  const TreeLayout& l = a.lay;
+  const int lane = threadIdx.x & 31;
+  int next_rec = l.open_records, n_hot = 0;
+  const uint32_t sm_addr = smem_u32(sm);
+  uint32_t ev = kEmpty;
+  for (int k = 1; next_event(s, a.m, k, ev, s_final, exit_flag); ++k) {
+    const uint32_t owner = s.rec_owner[ev & 0x1FFFu];
+    const int e = int(owner >> 16);
+    EntryState st = s.entry[e];
+    if ((owner & 0xFFFFu) == st.consumed) {
+      const int c = ++st.consumed;
+      if (c >= kHotAfter && n_hot < l.n_hot && (st.el_unit & 0xFFu) < 8 * kDrawWarps) {
+        // to a hot CTA: the row and the records of the draws ordered so far
+        const uint32_t cta = uint32_t(1 + n_hot), at = map_to_cta(hot_addr, cta), pos = ev >> 13;
+        uint32_t r = ld_relaxed(&s.first[pos]), mine = r;
+        for (int i = 1; i < int(st.ordered); ++i) {
+          r = ld_relaxed(&s.rec[r].next);
+          if (lane == i) mine = r;
+        }
+        if (lane < int(st.ordered)) st_remote(at + 8 + lane * 4, mine);
+        if (lane == 0) { st_remote(at + 4, st.ordered); st_remote(at, s.row[pos]); }
+        st.ring = map_to_cta(sm_addr + l.hot_ring, cta);
+        st.el_unit = uint32_t(8 * kDrawWarps + n_hot);
+        ++n_hot;
+      }
+      // one record is due to every node still to come; the rest of the pool lets streams run further ahead the longer they are
+      const int spare = max(0, l.n_records - next_rec - (a.m - k) - 1);
+      const int lead = int(st.ordered) - c;
+      const int add = max(0, max(1, min(min(2 + c, kMaxAhead), lead + spare)) - lead);
+      if (lane < add) {
+        const uint32_t rec = uint32_t(next_rec + lane);
+        s.rec_owner[rec] = (uint32_t(e) << 16) | uint32_t(st.ordered + lane);
+        st_relaxed(&s.rec[lane ? rec - 1 : st.last].next, rec);
+      }
+      if (add) {
+        st.last = uint32_t(next_rec + add - 1);
+        st.ordered = uint16_t(st.ordered + add);
+      }
+      if (lane == 0) {
+        for (int i = 0; i < add; ++i) send_order(l, s_tail, st.ring, st.el_unit, uint32_t(next_rec + i));
+        s.entry[e] = st;
+      }
+      next_rec += add;
+    }
+    __syncwarp();
+  }
+}
+
+// Row -> 64 leaf sums.  Every worker CTA sums its share of the leaves of every row (a row is then there after a quarter of
+// the time) and sends the sums to the CTA that draws from the row.  One thread brings the shares in with bulk copies, up to
+// four batches of 16 leaves ahead; 8 warps convert to fp64 (16 values a clock and SM: what bounds it) and reduce.
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+               ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
+}
+
+// Polls a barrier's phase; false once the tree is finished (or the limit has passed).
+__device__ __forceinline__ bool wait_phase(uint32_t bar, uint32_t parity, const uint32_t* exit_flag) {
+  uint64_t t0 = 0;
+  for (uint32_t spins = 0;; ++spins) {
+    if (mbar_test_wait(bar, parity)) return true;
+    if (ld_relaxed(exit_flag)) return false;
+    if ((spins & 1023u) == 0) {
+      const uint64_t now = global_timer_ns();
+      if (t0 == 0) t0 = now;
+      if (now - t0 > 4 * kWaitLimitNs) return false;
+    }
+  }
+}
+
+template <int K>
+__device__ __forceinline__ void run_fetcher(const TreeArgs& a, uint8_t* sm, int worker, unsigned long long* s_full, unsigned long long* s_empty,
+                                            const uint32_t* s_never, const uint32_t* exit_flag) {
+  const TreeLayout& l = a.lay;
+  if ((threadIdx.x & 31) != 0) return;
+  constexpr int kLeafTokens = 128 * K;
+  const uint32_t* s_row = reinterpret_cast<const uint32_t*>(sm + l.load_row);
+  const uint32_t stage0 = smem_u32(sm) + uint32_t(l.stage);
+  const int leaf0 = kLeaves * worker / l.n_workers, leaf1 = kLeaves * (worker + 1) / l.n_workers;
+  uint32_t stage = 0, round = 0, issued = 0;
+  bool go = true;
+  for (int e = 0; go && e < l.max_entries; ++e) {
+    uint32_t row = kEmpty;
+    uint64_t t0 = 0;
+    for (uint32_t spins = 0; go; ++spins) {                    // idle until a row is ordered or the tree is finished
+      row = ld_relaxed(s_row + e);
+      if (row != kEmpty) break;
+      if (ld_relaxed(exit_flag)) go = false;
+      if ((spins & 1023u) == 0) {
+        const uint64_t now = global_timer_ns();
+        if (t0 == 0) t0 = now;
+        if (now - t0 > 4 * kWaitLimitNs) go = false;
+      }
+    }
+    for (int first = leaf0; go && first < leaf1; first += kBatch) {
+      const uint32_t full = smem_u32(s_full + stage);
+      if (round > 0 && !wait_phase(smem_u32(s_empty + stage), (round - 1) & 1u, exit_flag)) { go = false; break; }
+      const int begin = first * kLeafTokens, end = min(min(first + kBatch, leaf1) * kLeafTokens, a.vocab);
+      if (end > begin) {
+        const uint32_t bytes = uint32_t(end - begin) * 4u;
+        mbar_expect_tx(full, bytes);
+        bulk_load(stage0 + stage * uint32_t(kBatch * kLeafTokens * 4), a.table + size_t(row) * a.vocab + begin, bytes, full);
+      } else {
+        mbar_arrive(full);
+      }
+      ++issued;
+      if (++stage == uint32_t(l.n_stages)) { stage = 0; ++round; }
+    }
+    if (go && e % l.n_workers == worker)
+      st_relaxed(reinterpret_cast<uint32_t*>(sm + l.number) + e / l.n_workers,
+                 __float_as_uint(__ldg(a.uniforms + draft_uniform_index(row, 0u, uint32_t(a.n_uniforms)))));
+  }
+  // no copy may be under way when the block ends
+  for (uint32_t k = 0; k < uint32_t(l.n_stages) && k < issued; ++k) {
+    if (stage == 0) { stage = uint32_t(l.n_stages); --round; }
+    --stage;
+    wait_phase(smem_u32(s_full + stage), round & 1u, s_never);
+  }
+}
+
+template <int K>
+__device__ __forceinline__ void run_loader(const TreeArgs& a, uint8_t* sm, int lw, int worker, unsigned long long* s_full, unsigned long long* s_empty,
+                                           const uint32_t* exit_flag) {
+  const TreeLayout& l = a.lay;
+  const int lane = threadIdx.x & 31, n_vec = a.vocab >> 2;
+  const uint32_t sums = smem_u32(sm) + uint32_t(l.sums);
+  const int leaf0 = kLeaves * worker / l.n_workers, leaf1 = kLeaves * (worker + 1) / l.n_workers;
+  uint32_t stage = 0, round = 0;
+  int el = 0, owner = 0;
+  for (int e = 0; e < l.max_entries; ++e) {
+    const uint32_t dst = map_to_cta(sums + uint32_t(el) * (kLeaves * 8), uint32_t(l.first_worker + owner));
+    if (++owner == l.n_workers) { owner = 0; ++el; }
+    for (int first = leaf0; first < leaf1; first += kBatch) {
+      if (!wait_phase(smem_u32(s_full + stage), round & 1u, exit_flag)) return;
+      const float4* src = reinterpret_cast<const float4*>(sm + l.stage) + stage * (kBatch * K * 32);
+      double q[2];
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {                            // leaves first + 2 lw, + 1
+        q[j] = 0.0;
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+          const int v4 = ((2 * lw + j) * K + k) * 32 + lane;
+          float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (first + 2 * lw + j < leaf1 && first * K * 32 + v4 < n_vec) x = src[v4];
+          q[j] += (double(x.x) + double(x.y)) + (double(x.z) + double(x.w));
+        }
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(s_empty + stage));
+      if (++stage == uint32_t(l.n_stages)) { stage = 0; ++round; }
+      const bool upper = lane & 16;                            // two sums over 32 lanes: halves swap, then plain steps
+      double b = upper ? q[1] : q[0];
+      b += __shfl_xor_sync(0xffffffffu, upper ? q[0] : q[1], 16);
+#pragma unroll
+      for (int o = 8; o > 0; o >>= 1) b += __shfl_xor_sync(0xffffffffu, b, o);
+      const int leaf = first + 2 * lw + (upper ? 1 : 0);
+      if ((lane & 15) == 0 && leaf < leaf1) st_remote64(dst + uint32_t(leaf) * 8, (unsigned long long)__double_as_longlong(b));
+    }
+  }
+}
+
+// Draws, one warp each, in the order in which the helpers asked for them.
+template <int K>
+__device__ __forceinline__ void run_drawer(const TreeArgs& a, uint8_t* sm, int dw, int worker, uint32_t (*s_mask)[32], uint32_t* s_log_n,
+                                           const uint32_t* exit_flag) {
+  constexpr int kLane = 4 * K, kLeaf = 32 * kLane;             // consecutive tokens of a lane, of a leaf
+  const TreeLayout& l = a.lay;
+  const int lane = threadIdx.x & 31, n_vec = a.vocab >> 2;
+  const uint32_t* ring = reinterpret_cast<const uint32_t*>(sm + l.ring) + dw * l.ring_size;
+  const uint32_t* s_row = reinterpret_cast<const uint32_t*>(sm + l.load_row);
+  unsigned long long* s_sums = reinterpret_cast<unsigned long long*>(sm + l.sums);
+  uint32_t* s_att = reinterpret_cast<uint32_t*>(sm + l.attempts);
+  uint32_t* s_log = reinterpret_cast<uint32_t*>(sm + l.log);
+  uint32_t* s_num = reinterpret_cast<uint32_t*>(sm + l.number);
+  const uint32_t rec_base = map_to_cta(smem_u32(sm) + l.rec, 0);
+  for (uint32_t i = 0;; ++i) {
+    const uint32_t at = i & uint32_t(l.ring_size - 1), phase = (i >> l.ring_shift) & 1u;
+    uint32_t msg = kEmpty;
+    uint64_t t0 = 0;
+    for (uint32_t spins = 0;; ++spins) {
+      msg = ld_relaxed(ring + at);
+      if (msg != kEmpty && (msg >> 31) == phase) break;
+      if (ld_relaxed(exit_flag)) return;
+      if ((spins & 1023u) == 0) {
+        const uint64_t now = global_timer_ns();
+        if (t0 == 0) t0 = now;
+        if (now - t0 > 4 * kWaitLimitNs) return;
+      }
+    }
+    const uint32_t el = (msg >> 13) & 0xFFFu, rec = msg & 0x1FFFu;
+    uint32_t row = kEmpty, ub = kEmpty;
+    if (!wait_until([&] { row = ld_relaxed(s_row + el * l.n_workers + worker); return row != kEmpty; }, exit_flag)) return;
+    const uint32_t att = s_att[el];
+    const float u_next = __ldg(a.uniforms + draft_uniform_index(row, att + 1, uint32_t(a.n_uniforms)));   // arrives behind this draw
+    unsigned long long* sums = s_sums + size_t(el) * kLeaves;
+    unsigned long long b0 = 0, b1 = 0;
+    if (!wait_until([&] {
+          b0 = ld_relaxed64(sums + 2 * lane);
+          b1 = ld_relaxed64(sums + 2 * lane + 1);
+          ub = ld_relaxed(s_num + el);
+          return __all_sync(0xffffffffu, b0 != ~0ull && b1 != ~0ull && ub != kEmpty) != 0;
+        }, exit_flag))
+      return;
+    const float u = __uint_as_float(ub);
+
+    // ---- the leaf: prefix sums over the 64 leaf sums, two per lane
+    const double s0 = __longlong_as_double((long long)b0), s1 = __longlong_as_double((long long)b1);
+    double incl = s0 + s1;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const double t = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += t;
+    }
+    double excl = __shfl_up_sync(0xffffffffu, incl, 1);
+    if (lane == 0) excl = 0.0;
+    const double total = __shfl_sync(0xffffffffu, incl, 31);
+    const double target = double(u) * total;
+    const uint32_t over = __ballot_sync(0xffffffffu, incl > target);
+    const bool none = over == 0u;                              // rounding (or an empty residual) left no crossing: the last token
+    const int hit = none ? 0 : __ffs(over) - 1;
+    const bool second = !(excl + s0 > target);
+    int leaf = __shfl_sync(0xffffffffu, 2 * lane + (second ? 1 : 0), hit);
+    const double before = __shfl_sync(0xffffffffu, second ? excl + s0 : excl, hit);
+    if (none) leaf = (a.vocab - 1) / kLeaf;
+
+    // ---- its tokens, those drawn before struck out
+    const float4* src = reinterpret_cast<const float4*>(a.table + size_t(row) * a.vocab);
+    float4 x[K];
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      const int v4 = (leaf * 32 + lane) * K + k;
+      x[k] = v4 < n_vec ? __ldg(src + v4) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    if (att > 0) {
+      s_mask[dw][lane] = 0u;
+      __syncwarp();
+      const uint32_t n_log = ld_relaxed(s_log_n);
+      const uint32_t want = (el << 16) | uint32_t(leaf * kLeaf);
+#pragma unroll 4
+      for (uint32_t j = lane; j < n_log; j += 32) {
+        const uint32_t off = ld_relaxed(s_log + j) - want;     // token within the leaf
+        if (off < uint32_t(kLeaf)) atomicOr(&s_mask[dw][off / kLane], 1u << (off % kLane));
+      }
+      __syncwarp();
+      const uint32_t dead = s_mask[dw][lane];
+      if (dead) {
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+          if ((dead >> (4 * k)) & 1u) x[k].x = 0.f;
+          if ((dead >> (4 * k + 1)) & 1u) x[k].y = 0.f;
+          if ((dead >> (4 * k + 2)) & 1u) x[k].z = 0.f;
+          if ((dead >> (4 * k + 3)) & 1u) x[k].w = 0.f;
+        }
+      }
+    }
+    double q[K], mine = 0.0;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      q[k] = (double(x[k].x) + double(x[k].y)) + (double(x[k].z) + double(x[k].w));
+      mine += q[k];
+    }
+    double pre = mine;                                         // inclusive prefix sums over the lanes
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const double t = __shfl_up_sync(0xffffffffu, pre, o);
+      if (lane >= o) pre += t;
+    }
+    double pex = __shfl_up_sync(0xffffffffu, pre, 1);
+    if (lane == 0) pex = 0.0;
+    const uint32_t cross = __ballot_sync(0xffffffffu, before + pre > target);
+    int owner = __ffs(cross) - 1;
+    if (none) {
+      owner = ((a.vocab - 1) % kLeaf) / kLane;
+    } else if (cross == 0u) {                                  // rounding between the two levels: the leaf's last mass
+      const uint32_t some = __ballot_sync(0xffffffffu, mine > 0.0);
+      owner = some ? 31 - __clz(some) : 0;
+    }
+    if (lane == owner) {
+      // quad, then token; where rounding leaves no crossing, the lane's last token with mass
+      double cum = before + pex, at_quad = -INFINITY;
+      int kp = -1, last = 0, pe = 0;
+#pragma unroll
+      for (int k = 0; k < K; ++k) {
+        if (kp < 0 && cum + q[k] > target) { kp = k; at_quad = cum; }
+        if (q[k] > 0.0) last = k;
+        cum += q[k];
+      }
+      if (kp < 0) kp = last;
+      if (none) kp = ((a.vocab - 1) % kLane) >> 2;
+      float4 f = x[0];
+#pragma unroll
+      for (int k = 1; k < K; ++k)
+        if (k == kp) f = x[k];
+      const double f0 = f.x, f1 = f.y, f2 = f.z, c0 = at_quad + f0, c1 = c0 + f1, c2 = c1 + f2, c3 = c2 + double(f.w);
+      if (c0 > target) pe = 0;
+      else if (c1 > target) pe = 1;
+      else if (c2 > target) pe = 2;
+      else if (c3 > target) pe = 3;
+      else pe = f.w > 0.f ? 3 : f.z > 0.f ? 2 : f.y > 0.f ? 1 : 0;
+      if (none) pe = (a.vocab - 1) & 3;
+      const int y = min(leaf * kLeaf + owner * kLane + 4 * kp + pe, a.vocab - 1);
+      const float py = pe == 0 ? f.x : pe == 1 ? f.y : pe == 2 ? f.z : f.w;
+      const double r = total > 0.0 ? double(py) / total : 0.0;
+      st_remote64(rec_base + rec * 16, (unsigned long long)__double_as_longlong(r));
+      st_remote(rec_base + rec * 16 + 8, uint32_t(y));
+      // ---- the token leaves the row
+      s_log[atomicAdd(s_log_n, 1u)] = (el << 16) | uint32_t(y);
+      s_att[el] = att + 1;
+      s_num[el] = __float_as_uint(u_next);
+      if (pe == 0) f.x = 0.f; else if (pe == 1) f.y = 0.f; else if (pe == 2) f.z = 0.f; else f.w = 0.f;
+      const double quad = (double(f.x) + double(f.y)) + (double(f.z) + double(f.w));
+      mine = 0.0;
+#pragma unroll
+      for (int k = 0; k < K; ++k) mine += k == kp ? quad : q[k];
+    }
+    __syncwarp();
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mine += __shfl_xor_sync(0xffffffffu, mine, o);
+    if (lane == 0) sums[leaf] = (unsigned long long)__double_as_longlong(mine);
+    __syncwarp();
+  }
+}
+
+// ---- hot CTA: one row's stream from a copy of the row and prefix sums in shared memory ----
+struct __align__(16) Pair { double hi, lo; };   // hi + lo, unevaluated
+struct __align__(16) Published { double sum; unsigned long long word; };   // residual sum; phase, record, token, probability
+__device__ __forceinline__ Pair add(Pair a, Pair b) {
+  const double s = a.hi + b.hi, t = s - a.hi;
+  const double e = (a.hi - (s - t)) + (b.hi - t);            // Knuth's two-sum
+  return Pair{s, e + (a.lo + b.lo)};
+}
+__device__ __forceinline__ Pair take_off(Pair a, double p) { // the sum holds p: a.hi >= p, Dekker's fast two-sum
+  const double s = a.hi - p;
+  return Pair{s, a.lo + ((a.hi - s) - p)};
+}
+__device__ __forceinline__ Pair shfl_up_pair(Pair v, int o) {
+  return Pair{__shfl_up_sync(0xffffffffu, v.hi, o), __shfl_up_sync(0xffffffffu, v.lo, o)};
+}
+__device__ __forceinline__ Pair scan(Pair v, int lane) {
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const Pair t = shfl_up_pair(v, o);
+    if (lane >= o) v = add(t, v);
+  }
+  return v;
+}
+
+// Prefix sums over the sub-blocks of chunk c (one warp; lane = 4 sub-blocks).  Sub-block 4 l + j of a chunk lies at [j][l].
+__device__ __forceinline__ void build_chunk(const float* s_row, Pair* s_sub, int c, int lane) {
+  Pair v[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    v[j] = Pair{0.0, 0.0};
+    const float* x = s_row + c * kChunk + (4 * lane + j) * kSub;
+#pragma unroll
+    for (int i = 0; i < kSub; ++i) v[j] = add(v[j], Pair{double(x[(i + lane) & (kSub - 1)]), 0.0});   // (any order; rotated: fewer bank conflicts)
+    if (j) v[j] = add(v[j - 1], v[j]);
+  }
+  const Pair upto = shfl_up_pair(scan(v[3], lane), 1);
+#pragma unroll
+  for (int j = 0; j < 4; ++j) s_sub[(c * 4 + j) * 32 + lane] = lane ? add(upto, v[j]) : v[j];
+}
+
+__device__ __forceinline__ void run_hot(const TreeArgs& a, uint8_t* sm, const uint32_t* s_hot, uint32_t* s_go, const uint32_t* exit_flag) {
+  const TreeLayout& l = a.lay;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  float* s_row = reinterpret_cast<float*>(sm + l.hot_row);
+  Pair* s_sub = reinterpret_cast<Pair*>(sm + l.hot_sub);
+  const uint32_t* ring = reinterpret_cast<const uint32_t*>(sm + l.hot_ring);
+  Published* s_pub = reinterpret_cast<Published*>(sm + l.hot_pub);
+  const uint32_t rec_base = map_to_cta(smem_u32(sm) + l.rec, 0);
+  // ---- one thread waits for a row: its number and how many draws have been ordered elsewhere (each word validates itself)
+  if (tid == 0) {
+    uint32_t row = kEmpty, n_prev = kEmpty;
+    uint64_t t0 = 0;
+    for (uint32_t spins = 0;; ++spins) {
+      row = ld_relaxed(s_hot);
+      n_prev = ld_relaxed(s_hot + 1);
+      if (row != kEmpty && n_prev != kEmpty) break;
+      if (ld_relaxed(exit_flag)) { row = kEmpty; break; }
+      if ((spins & 1023u) == 0) {
+        const uint64_t now = global_timer_ns();
+        if (t0 == 0) t0 = now;
+        if (now - t0 > 4 * kWaitLimitNs) { row = kEmpty; break; }
+      }
+    }
+    s_go[0] = row;
+    s_go[1] = n_prev;
+  }
+  __syncthreads();
+  const uint32_t row = s_go[0], n_prev = s_go[1];
+  if (row == kEmpty) return;                                   // the whole block
+  const float4* src = reinterpret_cast<const float4*>(a.table + size_t(row) * a.vocab);
+  for (int i = tid; i < kChunks * kChunk / 4; i += kTreeThreads)
+    reinterpret_cast<float4*>(s_row)[i] = i < (a.vocab >> 2) ? __ldg(src + i) : make_float4(0.f, 0.f, 0.f, 0.f);
+  bool good = true;
+  uint32_t prev = kEmpty, gone = kEmpty;                       // (a draw ordered elsewhere may still be under way)
+  if (warp == 0 && lane < int(n_prev)) {
+    good = wait_until([&] { prev = ld_relaxed(s_hot + 2 + lane); return prev != kEmpty; }, exit_flag);
+    if (good) good = wait_until([&] { gone = ld_remote(rec_base + (prev & (kMaxRecords - 1)) * 16 + 8); return gone != kEmpty; }, exit_flag);
+  }
+  __syncthreads();
+  if (gone != kEmpty) s_row[gone] = 0.f;
+  __syncthreads();
+  for (int c = warp; c < kChunks; c += kTreeThreads / 32) build_chunk(s_row, s_sub, c, lane);
+  __syncthreads();
+  if (warp == 1) {                                             // divides and sends, one draw behind the stream
+    if (lane != 0) return;
+    for (uint32_t i = 0;; ++i) {
+      const uint32_t at = i & uint32_t(kHotRing - 1), phase = (i / kHotRing) & 1u;
+      unsigned long long w = 0;
+      uint64_t t0 = 0;
+      for (uint32_t spins = 0;; ++spins) {
+        w = ld_acquire64(&s_pub[at].word);
+        if (uint32_t(w >> 63) == phase) break;
+        if (ld_relaxed(exit_flag)) return;
+        if ((spins & 1023u) == 0) {
+          const uint64_t now = global_timer_ns();
+          if (t0 == 0) t0 = now;
+          if (now - t0 > 4 * kWaitLimitNs) return;
+        }
+      }
+      const double sum = s_pub[at].sum, p = double(__uint_as_float(uint32_t(w)));
+      const double r = sum > 0.0 ? p / sum : 0.0;
+      const uint32_t rec = uint32_t(w >> 47) & 0x1FFFu;
+      st_remote64(rec_base + rec * 16, (unsigned long long)__double_as_longlong(r));
+      st_remote(rec_base + rec * 16 + 8, uint32_t(w >> 32) & 0x7FFFu);
+    }
+  }
+  if (warp != 0 || !__all_sync(0xffffffffu, good)) return;
+
+  // ---- the stream.  Lane c holds the prefix sum over chunks 0 .. c.
+  Pair upto = scan(s_sub[(lane * 4 + 3) * 32 + 31], lane);
+  Pair total{__shfl_sync(0xffffffffu, upto.hi, 31), __shfl_sync(0xffffffffu, upto.lo, 31)};
+  double built = total.hi;
+  float u_next = __ldg(a.uniforms + draft_uniform_index(row, n_prev, uint32_t(a.n_uniforms)));
+  for (uint32_t i = 0;; ++i) {
+    const uint32_t at = i & uint32_t(kHotRing - 1), phase = (i / kHotRing) & 1u;
+    const float u = u_next;
+    u_next = __ldg(a.uniforms + draft_uniform_index(row, n_prev + i + 1, uint32_t(a.n_uniforms)));
+    const double sum = total.hi + total.lo, target = double(u) * sum;
+    const double mine = upto.hi + upto.lo;
+    uint32_t msg = kEmpty;
+    uint64_t t0 = 0;
+    for (uint32_t spins = 0;; ++spins) {
+      msg = ld_relaxed(ring + at);
+      if (msg != kEmpty && (msg >> 31) == phase) break;
+      if (ld_relaxed(exit_flag)) return;
+      if ((spins & 1023u) == 0) {
+        const uint64_t now = global_timer_ns();
+        if (t0 == 0) t0 = now;
+        if (now - t0 > 4 * kWaitLimitNs) return;
+      }
+    }
+    const uint32_t rec = msg & 0x1FFFu;
+    // chunk, then sub-block, then token: the first whose prefix sum exceeds the target
+    const uint32_t in_chunk = __ballot_sync(0xffffffffu, mine > target);
+    const bool none = in_chunk == 0u;                          // rounding (or an empty residual) left no crossing: the last token
+    const int c = none ? (a.vocab - 1) / kChunk : __ffs(in_chunk) - 1;
+    const double up = __shfl_sync(0xffffffffu, mine, (c - 1) & 31), before = c ? up : 0.0;
+    Pair q[4];
+    double w[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) q[j] = s_sub[(c * 4 + j) * 32 + lane];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) w[j] = before + (q[j].hi + q[j].lo);
+    const uint32_t in_sub = __ballot_sync(0xffffffffu, w[3] > target);
+    const double left = __shfl_up_sync(0xffffffffu, w[3], 1);
+    double from = lane ? left : before;                        // prefix sum in front of this lane's crossing sub-block
+    int sub = 4 * lane;
+#pragma unroll
+    for (int j = 0; j < 3; ++j)
+      if (!(w[j] > target)) { from = w[j]; sub = 4 * lane + j + 1; }
+    const int who = in_sub ? __ffs(in_sub) - 1 : 31;
+    sub = __shfl_sync(0xffffffffu, sub, who);
+    from = __shfl_sync(0xffffffffu, from, who);
+    if (none) sub = ((a.vocab - 1) % kChunk) / kSub;
+    float* xs = s_row + c * kChunk + sub * kSub;
+    // two tokens per lane, lanes 0 .. 3 (the others repeat them): prefix sums in front of each pair
+    const int t = lane & 3;
+    const float2 x = reinterpret_cast<const float2*>(xs)[t];
+    const double d0 = x.x, d1 = x.y, both = d0 + d1;
+    double pa = __shfl_up_sync(0xffffffffu, both, 1, 4);
+    if (t < 1) pa = 0.0;
+    double pb = __shfl_up_sync(0xffffffffu, both + pa, 2, 4);
+    if (t < 2) pb = 0.0;
+    const double at_pair = from + (pb + pa);
+    const bool h0 = at_pair + d0 > target, h1 = at_pair + both > target;
+    const uint32_t b0 = __ballot_sync(0xffffffffu, h0), b1 = __ballot_sync(0xffffffffu, h1) & 0xFu;
+    int lt = __ffs(b1) - 1, pick = 2 * lt + (((b0 >> (lt & 31)) & 1u) ? 0 : 1);
+    double p = __shfl_sync(0xffffffffu, h0 ? d0 : d1, lt & 31);
+    if (none || b1 == 0u) {                                    // rounding left no crossing: the last token with mass
+      const uint32_t m = __ballot_sync(0xffffffffu, x.x > 0.f || x.y > 0.f) & 0xFu, m1 = __ballot_sync(0xffffffffu, x.y > 0.f);
+      lt = m ? 31 - __clz(m) : 0;
+      pick = 2 * lt + int((m1 >> lt) & 1u);
+      if (none) pick = (a.vocab - 1) & (kSub - 1);
+      p = double(xs[pick]);
+    }
+    const int y = min(c * kChunk + sub * kSub + pick, a.vocab - 1);
+    // the token leaves the row: every prefix sum from it on
+    __syncwarp();
+    if (lane == 0) {
+      xs[pick] = 0.f;
+      s_pub[at].sum = sum;
+      st_release64(&s_pub[at].word, ((unsigned long long)phase << 63) | ((unsigned long long)rec << 47) | ((unsigned long long)y << 32) |
+                                        (unsigned long long)__float_as_uint(float(p)));
+    }
+    total = take_off(total, p);
+    const Pair cut = take_off(upto, p);
+    if (lane >= c) upto = cut;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      q[j] = take_off(q[j], p);
+      if (4 * lane + j >= sub) s_sub[(c * 4 + j) * 32 + lane] = q[j];
+    }
+    __syncwarp();
+    if (total.hi + total.lo < built * 0x1p-40) {               // (rare: what is left is small against the tables' rounding)
+      for (int k = 0; k < kChunks; ++k) build_chunk(s_row, s_sub, k, lane);
+      __syncwarp();
+      upto = scan(s_sub[(lane * 4 + 3) * 32 + 31], lane);
+      total = Pair{__shfl_sync(0xffffffffu, upto.hi, 31), __shfl_sync(0xffffffffu, upto.lo, 31)};
+      built = total.hi;
+    }
+  }
+}
+
+template <bool kGreedy, int K>
+__global__ void __launch_bounds__(kTreeThreads, 1)
+build_tree_kernel(const __grid_constant__ TreeArgs a) {
+  extern __shared__ __align__(16) uint8_t csm[];
+  __shared__ uint32_t s_exit, s_never, s_final, s_log_n;       // (planner and helper do not listen to s_exit)
+  __shared__ uint32_t s_tail[8 * kDrawWarps + kMaxHot];
+  __shared__ uint32_t s_hot[2 + 32], s_go[2];
+  __shared__ uint32_t s_mask[kDrawWarps][32];
+  __shared__ __align__(8) unsigned long long s_full[kMaxStages], s_empty[kMaxStages];
+  const TreeLayout& l = a.lay;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint32_t rank = cluster_ctarank();
+  uint32_t n_cta;
+  asm("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(n_cta));
+  const int req = int(blockIdx.x / n_cta);
+  const bool planner_cta = rank == 0, worker_cta = int(rank) >= l.first_worker, hot_cta = !planner_cta && !worker_cta;
+
+  // ---- every word that another warp or CTA will write starts as "not there yet"
+  if (tid == 0) { s_exit = 0u; s_never = 0u; s_final = kEmpty; s_log_n = 0u; }
+  if (tid < kMaxStages) {
+    mbar_init(smem_u32(s_full + tid), 1);
+    mbar_init(smem_u32(s_empty + tid), kLoadWarps);
+    fence_barrier_init();
+  }
+  if (tid < 8 * kDrawWarps + kMaxHot) s_tail[tid] = 0u;
+  if (tid < 2 + 32) s_hot[tid] = kEmpty;
+  auto fill = [&](int off, int words, uint32_t v) {
+    uint32_t* p = reinterpret_cast<uint32_t*>(csm + off);
+    for (int i = tid; i < words; i += kTreeThreads) p[i] = v;
+  };
+  if (planner_cta) {
+    fill(l.rec, l.n_records * 4, kEmpty);
+    fill(l.key, l.nodes_pad * 2, 0u);
+    fill(l.seq, l.nodes_pad, kEmpty);
+    fill(l.ev, l.nodes_pad, kEmpty);
+    fill(l.first, l.nodes_pad, kEmpty);
+    fill(l.hash_row, l.hash_size, kEmpty);
+  }
+  if (worker_cta) {
+    fill(l.load_row, l.max_entries, kEmpty);
+    fill(l.sums, l.entries_local * kLeaves * 2, kEmpty);
+    fill(l.number, l.entries_local, kEmpty);
+    fill(l.attempts, l.entries_local, 0u);
+    fill(l.ring, kDrawWarps * l.ring_size, kEmpty);
+    fill(l.log, l.n_records, kEmpty);
+  }
+  if (hot_cta) {
+    fill(l.hot_ring, kHotRing, kEmpty);
+    fill(l.hot_pub, kHotRing * int(sizeof(Published)) / 4, kEmpty);
+  }
+  __syncthreads();
+  cluster_sync_all();
+
+  const Shared s = planner_view(csm, l);
+  if (hot_cta) {
+    run_hot(a, csm, s_hot, s_go, &s_exit);
+  } else if (warp == 0) {
+    if (planner_cta) {
+      const int n = kGreedy ? plan_greedy(a, s, &s_never) : plan_threshold(a, s, &s_never);
+      __syncwarp();
+      if (lane == 0) {
+        a.n_nodes[req] = n + 1;                                // 0: a wait ran out
+        st_relaxed(&s_final, n < 0 ? 0u : uint32_t(n));
+      }
+      for (uint32_t c = uint32_t(lane); c < n_cta; c += 32) st_remote(map_to_cta(smem_u32(&s_exit), c), 1u);
+    }
+  } else if (warp == 1) {
+    if (planner_cta) run_opener<kGreedy>(a, s, csm, s_tail, &s_final, &s_never, req);
+  } else if (warp == 2) {
+    if (planner_cta) run_orderer<kGreedy>(a, s, csm, s_tail, smem_u32(s_hot), &s_final, &s_never);
+  } else if (worker_cta) {
+    if (warp < kRoles + kDrawWarps) run_drawer<K>(a, csm, warp - kRoles, int(rank) - l.first_worker, s_mask, &s_log_n, &s_exit);
+    else if (warp == kRoles + kDrawWarps) run_fetcher<K>(a, csm, int(rank) - l.first_worker, s_full, s_empty, &s_never, &s_exit);
+    else run_loader<K>(a, csm, warp - kRoles - kDrawWarps - 1, int(rank) - l.first_worker, s_full, s_empty, &s_exit);
+  }
+  __syncwarp();
+  cluster_sync_all();                                          // nobody leaves while its shared memory may be written
+
+  if (planner_cta) {                                           // the tree, from the planner's and the helper's notes
+    const int n = int(s_final);
+    const size_t base = size_t(req) * (a.m + 1);
+    for (int k = tid; k <= n; k += kTreeThreads) {
+      const DrawRecord rc = s.rec[k ? s.ev[k] & 0x1FFFu : 0u];
+      const double v = k ? __longlong_as_double((long long)s.val[k]) : 1.0;
+      a.parents[base + k] = k ? int32_t(s.ev[k] >> 13) : -1;
+      a.tokens[base + k] = k ? int32_t(rc.token) : 0;
+      a.values[base + k] = float(v);
+      a.child_values[base + k] = k ? float(v * __longlong_as_double((long long)rc.r_bits)) : 1.f;
+      a.rows[base + k] = int32_t(s.row[k]);
+    }
+  }
+}
+
+// Cluster of C CTAs: CTA 0 plans, n_hot take over long streams, the others load and draw (one CTA does it all when C = 1).
+bool tree_layout(int nodes, int n_rows, int leaf_bytes, int C, int n_hot, TreeLayout& l) {
+  l.nodes_pad = (nodes + 1 + 31) & ~31;
+  l.max_entries = nodes + 1 < n_rows ? nodes + 1 : n_rows;
+  l.n_hot = n_hot;
+  l.first_worker = C > 1 ? 1 + n_hot : 0;
+  l.n_workers = C - l.first_worker;
+  l.entries_local = (l.max_entries + l.n_workers - 1) / l.n_workers;
+  const int per_drawer = (l.entries_local + kDrawWarps - 1) / kDrawWarps;
+  l.ring_shift = 5;
+  while ((1 << l.ring_shift) < per_drawer * kMaxAhead) ++l.ring_shift;
+  l.ring_size = 1 << l.ring_shift;
+  l.hash_size = 32;
+  while (l.hash_size < 2 * l.max_entries) l.hash_size *= 2;
+  // Records: one per row to open and one per node is what the tree can need; the rest lets draws run ahead.
+  l.n_stages = kMaxStages;
+  int open_ahead = 4, run_ahead = nodes + 4 * l.max_entries;
+  for (;;) {
+    l.open_records = l.max_entries * open_ahead;
+    l.n_records = l.open_records + nodes + 1 + run_ahead;
+    int at = 0;
+    auto take = [&](int bytes) { const int o = at; at = (at + bytes + 15) & ~15; return o; };
+    l.rec = take(l.n_records * 16);
+    l.key = take(l.nodes_pad * 8);
+    l.val = take(l.nodes_pad * 8);
+    l.seq = take(l.nodes_pad * 4);
+    l.slot = take(l.nodes_pad * 4);
+    l.ev = take(l.nodes_pad * 4);
+    l.first = take(l.nodes_pad * 4);
+    l.row = take(l.nodes_pad * 4);
+    l.rec_owner = take(l.n_records * 4);
+    l.hash_row = take(l.hash_size * 4);
+    l.hash_val = take(l.hash_size * 4);
+    l.entry = take(l.max_entries * int(sizeof(EntryState)));
+    l.bytes = at;
+    if (C > 1) at = 0;                                         // the other CTAs hold none of the above
+    l.stage = take(l.n_stages * kBatch * leaf_bytes);
+    l.sums = take(l.entries_local * kLeaves * 8);
+    l.load_row = take(l.max_entries * 4);
+    l.attempts = take(l.entries_local * 4);
+    l.number = take(l.entries_local * 4);
+    l.ring = take(kDrawWarps * l.ring_size * 4);
+    l.log = take(l.n_records * 4);
+    if (at > l.bytes) l.bytes = at;
+    at = 0;
+    l.hot_row = take(n_hot ? kChunks * kChunk * 4 : 0);
+    l.hot_sub = take(n_hot ? kChunks * kChunk / kSub * int(sizeof(Pair)) : 0);
+    l.hot_ring = take(n_hot ? kHotRing * 4 : 0);
+    l.hot_pub = take(n_hot ? kHotRing * int(sizeof(Published)) : 0);
+    if (at > l.bytes) l.bytes = at;
+    if (l.bytes <= 224 * 1024 && l.n_records <= kMaxRecords) return true;
+    if (l.n_stages > 2) l.n_stages = 2;
+    else if (run_ahead > nodes) run_ahead = nodes;
+    else if (open_ahead > 2) open_ahead = 2;
+    else if (run_ahead > 64) run_ahead /= 2;
+    else if (open_ahead > 1) open_ahead = 1;
+    else if (l.n_stages > 1) l.n_stages = 1;
+    else return false;
+  }
+}
+
+template <bool kGreedy, int K>
+cudaError_t launch_tree(const TreeArgs& a, int n_req, int C, cudaStream_t stream) {
+  static DynSmemGrant grant;
+  if (cudaError_t e = grant.ensure(build_tree_kernel<kGreedy, K>, size_t(a.lay.bytes)); e != cudaSuccess) return e;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = unsigned(C);
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(unsigned(n_req) * unsigned(C));
+  cfg.blockDim = dim3(kTreeThreads);
+  cfg.dynamicSmemBytes = size_t(a.lay.bytes);
+  cfg.stream = stream;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, build_tree_kernel<kGreedy, K>, a);
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+template <bool kGreedy>
+cudaError_t launch_tree(TreeArgs a, int n_req, cudaStream_t stream) {
+  // The largest cluster with which all requests run at once; where none does, the smallest that holds the tree.
+  const int leaf_bytes = 512 * (a.vocab <= kLeaves * 128 ? 1 : a.vocab <= kLeaves * 256 ? 2 : 4);
+  int C = 8;
+  while (C > 1 && int64_t(n_req) * C > kDefaultSMs) C /= 2;
+  for (;; C *= 2) {
+    bool fits = false;
+    for (int hot = C == 8 ? kMaxHot : C == 4 ? 1 : 0; hot >= 0 && !fits; --hot)
+      fits = (hot == 0 || a.m > 2 * kHotAfter) && tree_layout(a.m, a.n_rows, leaf_bytes, C, hot, a.lay);
+    if (fits) break;
+    if (C == 8) return cudaErrorInvalidConfiguration;          // not reached: 2047 nodes and rows fit
+  }
+  a.rows_inverse = uint32_t((1ull << 32) / uint64_t(a.n_rows) - (a.n_rows == 1 ? 1 : 0));
+  if (a.vocab <= kLeaves * 128) return launch_tree<kGreedy, 1>(a, n_req, C, stream);
+  if (a.vocab <= kLeaves * 256) return launch_tree<kGreedy, 2>(a, n_req, C, stream);
+  return launch_tree<kGreedy, 4>(a, n_req, C, stream);
 }
 
 }  // namespace
-
-__global__ void __launch_bounds__(kVThreads, 1)
-build_tree_greedy_kernel(const float* __restrict__ draft_table, int n_rows, int vocab, const float* __restrict__ uniforms,
-                         int n_uniforms, const int32_t* __restrict__ root_row, int m, TreeOut out,
-                         int32_t* __restrict__ n_nodes_out) {
-  extern __shared__ __align__(16) uint8_t csm[];
-  // slots: value, position, attempt; per node: row id, token, the position it was drawn at
-  const int max_slots = 2 * m + 2;
-  double* s_v = reinterpret_cast<double*>(csm);                     // [max_slots]   (-1 = taken); fp64 like the draws
-  int16_t* s_pos = reinterpret_cast<int16_t*>(s_v + max_slots);     // [max_slots]
-  int16_t* s_att = s_pos + max_slots;                               // [max_slots]
-  int32_t* s_row = reinterpret_cast<int32_t*>(s_att + max_slots + (max_slots & 1));   // [m + 1]
-  int32_t* s_tok = s_row + (m + 1);                                 // [m + 1]
-  int16_t* s_ppos = reinterpret_cast<int16_t*>(s_tok + (m + 1));    // [m + 1] the position (parent) a node was drawn at
-  __shared__ uint32_t s_kill[kVThreads];                            // bit 4 k + e of word t: element e of thread t's chunk k is used up
-  __shared__ VocabScratch s_vs;
-  __shared__ double s_bv[33];
-  __shared__ int s_bi[33];
-
-  const int r = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const size_t base = size_t(r) * (m + 1);
-  if (tid == 0) {
-    s_row[0] = ((root_row[r] % n_rows) + n_rows) % n_rows;        // non-negative remainder: any int32 maps to a row
-    s_tok[0] = 0;
-    s_ppos[0] = -1;
-    s_v[0] = 1.0; s_pos[0] = 0; s_att[0] = 0;
-    write_node(out, base, 0, -1, 0, 1.f, 1.f, s_row[0]);
-  }
-  __syncthreads();
-  int n_slots = 1, n_created = 0;
-
-  for (int step = 0; step < m; ++step) {
-    // ---- the slot with the largest value (ties: lowest index = pushed first)
-    double bv = -1.0;
-    int bi = 0x7fffffff;
-    for (int i = tid; i < n_slots; i += kVThreads) {
-      const double v_ = s_v[i];
-      if (v_ > bv) { bv = v_; bi = i; }                          // i increases: the first of equal values is kept
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const double tv = __shfl_xor_sync(0xffffffffu, bv, o);
-      const int ti = __shfl_xor_sync(0xffffffffu, bi, o);
-      if (tv > bv || (tv == bv && ti < bi)) { bv = tv; bi = ti; }
-    }
-    __syncthreads();
-    if (lane == 0) { s_bv[warp] = bv; s_bi[warp] = bi; }
-    __syncthreads();
-    if (warp == 0) {
-      double v_ = s_bv[lane];
-      int i_ = s_bi[lane];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const double tv = __shfl_xor_sync(0xffffffffu, v_, o);
-        const int ti = __shfl_xor_sync(0xffffffffu, i_, o);
-        if (tv > v_ || (tv == v_ && ti < i_)) { v_ = tv; i_ = ti; }
-      }
-      if (lane == 0) { s_bv[32] = v_; s_bi[32] = i_; }
-    }
-    __syncthreads();
-    if (s_bv[32] < 0.0) break;                                   // no live slot (cannot happen before m nodes exist)
-    const int slot = s_bi[32];
-    const double v = s_v[slot];
-    const int pos = s_pos[slot], attempt = s_att[slot];
-    const int prow = s_row[pos];
-    __syncthreads();
-    if (tid == 0) s_v[slot] = -1.0;
-
-    // ---- residual of the position: its row with the tokens of its existing children zeroed
-    float4 R[kMaxChunks];
-    load_row(R, draft_table + size_t(prow) * vocab, vocab);
-    if (attempt > 0) {                                           // (a first sampling has nothing to strike out)
-      s_kill[tid] = 0u;
-      __syncthreads();
-      for (int c = 1 + tid; c <= n_created; c += kVThreads)
-        if (s_ppos[c] == pos) {
-          const int yc = s_tok[c], y4 = yc >> 2;
-          atomicOr(&s_kill[y4 % kVThreads], 1u << ((y4 / kVThreads) * 4 + (yc & 3)));
-        }
-      __syncthreads();
-      const uint32_t kill = s_kill[tid];
-      if (kill) {
-#pragma unroll
-        for (int k = 0; k < kMaxChunks; ++k) {
-          if ((kill >> (4 * k)) & 1u) R[k].x = 0.f;
-          if ((kill >> (4 * k + 1)) & 1u) R[k].y = 0.f;
-          if ((kill >> (4 * k + 2)) & 1u) R[k].z = 0.f;
-          if ((kill >> (4 * k + 3)) & 1u) R[k].w = 0.f;
-        }
-      }
-    }
-    double total;
-    const float u = uniforms[draft_uniform_index(uint32_t(prow), uint32_t(attempt), uint32_t(n_uniforms))];
-    const int y = sample_inverse_cdf(R, vocab, u, total, s_vs);
-    const float py = take_element(R, y, false, s_vs);
-    const double rr = total > 0.0 ? double(py) / total : 0.0;
-
-    // ---- the new node and the two slots it opens
-    const int k = ++n_created;
-    if (tid == 0) {
-      const int krow = int(draft_row_of_child(uint32_t(prow), uint32_t(y), uint32_t(n_rows)));
-      s_row[k] = krow;
-      s_tok[k] = y;
-      s_ppos[k] = int16_t(pos);
-      write_node(out, base, k, pos, y, float(v), float(v * rr), krow);
-      int ns = n_slots;
-      if (1.0 - rr > 0.0) { s_v[ns] = v * (1.0 - rr); s_pos[ns] = int16_t(pos); s_att[ns] = int16_t(attempt + 1); ++ns; }
-      s_v[ns] = v * rr; s_pos[ns] = int16_t(k); s_att[ns] = 0;
-    }
-    n_slots += (1.0 - rr > 0.0) ? 2 : 1;
-    __syncthreads();
-  }
-  if (tid == 0) n_nodes_out[r] = n_created + 1;
-}
-
-__global__ void __launch_bounds__(kVThreads, 1)
-build_tree_threshold_kernel(const float* __restrict__ draft_table, int n_rows, int vocab, const float* __restrict__ uniforms,
-                            int n_uniforms, const int32_t* __restrict__ root_row, float threshold, int max_nodes,
-                            TreeOut out, int32_t* __restrict__ n_nodes_out) {
-  extern __shared__ __align__(16) uint8_t csm[];
-  int32_t* s_row = reinterpret_cast<int32_t*>(csm);                 // [max_nodes + 1]
-  double* s_cv = reinterpret_cast<double*>(csm + ((size_t(max_nodes + 1) * 4 + 7) & ~size_t(7)));   // [max_nodes + 1] value of the first sampling under a node
-  __shared__ VocabScratch s_vs;
-
-  const int r = blockIdx.x, tid = threadIdx.x;
-  const size_t base = size_t(r) * (max_nodes + 1);
-  if (tid == 0) {
-    s_row[0] = ((root_row[r] % n_rows) + n_rows) % n_rows;        // non-negative remainder: any int32 maps to a row
-    s_cv[0] = 1.0;
-    write_node(out, base, 0, -1, 0, 1.f, 1.f, s_row[0]);
-  }
-  __syncthreads();
-  int n_created = 0;
-  int layer_begin = 0, layer_end = 1;                               // nodes [layer_begin, layer_end) are the current leaves
-  while (layer_begin < layer_end && n_created < max_nodes) {
-    for (int node = layer_begin; node < layer_end && n_created < max_nodes; ++node) {
-      double v = s_cv[node];
-      if (!(v >= double(threshold))) continue;
-      const int prow = s_row[node];
-      float4 R[kMaxChunks];
-      load_row(R, draft_table + size_t(prow) * vocab, vocab);
-      int attempt = 0;
-      while (v >= double(threshold) && n_created < max_nodes) {
-        double total;
-        const float u = uniforms[draft_uniform_index(uint32_t(prow), uint32_t(attempt), uint32_t(n_uniforms))];
-        const int y = sample_inverse_cdf(R, vocab, u, total, s_vs);
-        const float py = take_element(R, y, true, s_vs);            // drawn tokens leave the residual
-        const double rr = total > 0.0 ? double(py) / total : 0.0;
-        const int k = ++n_created;
-        if (tid == 0) {
-          const int krow = int(draft_row_of_child(uint32_t(prow), uint32_t(y), uint32_t(n_rows)));
-          s_row[k] = krow;
-          s_cv[k] = v * rr;
-          write_node(out, base, k, node, y, float(v), float(v * rr), krow);
-        }
-        v = v * (1.0 - rr);
-        ++attempt;
-        if (!(1.0 - rr > 0.0)) break;
-      }
-    }
-    __syncthreads();
-    layer_begin = layer_end;
-    layer_end = n_created + 1;
-  }
-  if (tid == 0) n_nodes_out[r] = n_created + 1;
-}
-
-size_t build_tree_greedy_smem(int m) {
-  const size_t max_slots = 2 * size_t(m) + 2;          // value (8 bytes) + position and attempt (2 + 2) per slot
-  return 12 * max_slots + 10 * size_t(m + 1) + 64;     // row and token (4 + 4) + the 2-byte position per node
-}
 
 cudaError_t launch_build_tree_greedy(const float* draft_table, int n_rows, int vocab, const float* uniforms, int n_uniforms,
                                      const int32_t* root_row, int n_req, int m, int32_t* parents, int32_t* tokens,
                                      float* values, float* child_values, int32_t* rows, int32_t* n_nodes,
                                      cudaStream_t stream) {
   if (n_req <= 0) return cudaSuccess;
-  const size_t smem = build_tree_greedy_smem(m);
-  static DynSmemGrant grant;
-  if (cudaError_t e = grant.ensure(build_tree_greedy_kernel, smem); e != cudaSuccess) return e;
-  TreeOut out{parents, tokens, values, child_values, rows};
-  build_tree_greedy_kernel<<<n_req, kVThreads, smem, stream>>>(draft_table, n_rows, vocab, uniforms, n_uniforms, root_row, m,
-                                                               out, n_nodes);
-  return cudaGetLastError();
+  return launch_tree<true>(TreeArgs{draft_table, uniforms, root_row, n_rows, vocab, n_uniforms, m, 0u, 0.f, parents, tokens, values,
+                                    child_values, rows, n_nodes, TreeLayout{}}, n_req, stream);
 }
 
 cudaError_t launch_build_tree_threshold(const float* draft_table, int n_rows, int vocab, const float* uniforms,
@@ -234,11 +1174,8 @@ cudaError_t launch_build_tree_threshold(const float* draft_table, int n_rows, in
                                         int32_t* parents, int32_t* tokens, float* values, float* child_values, int32_t* rows,
                                         int32_t* n_nodes, cudaStream_t stream) {
   if (n_req <= 0) return cudaSuccess;
-  const size_t smem = size_t(max_nodes + 1) * 12 + 16;
-  TreeOut out{parents, tokens, values, child_values, rows};
-  build_tree_threshold_kernel<<<n_req, kVThreads, smem, stream>>>(draft_table, n_rows, vocab, uniforms, n_uniforms, root_row,
-                                                                  threshold, max_nodes, out, n_nodes);
-  return cudaGetLastError();
+  return launch_tree<false>(TreeArgs{draft_table, uniforms, root_row, n_rows, vocab, n_uniforms, max_nodes, 0u, threshold, parents,
+                                     tokens, values, child_values, rows, n_nodes, TreeLayout{}}, n_req, stream);
 }
 
 }  // namespace dyspec

@@ -1,5 +1,5 @@
-// Block-wide operations on one vocabulary-sized probability row held in registers, shared by the tree
-// verification and tree construction kernels.  A block has 1024 threads; thread t owns the float4
+// Block-wide operations of the tree verification kernel on one vocabulary-sized probability row held in
+// registers, and the draft model of the tree construction kernel.  A block has 1024 threads; thread t owns the float4
 // chunks t, t + 1024, ... of the row ("row k" of the layout = tokens [4096 k, 4096 k + 4096)), so
 // global loads are coalesced.  Vocabulary <= 8 * 1024 * 4 = 32768.
 #pragma once
@@ -17,7 +17,6 @@ struct VocabScratch {          // shared memory used by the helpers below
   double scan[32];
   float red[33];
   int pick;
-  float pub[2];
 };
 
 __device__ __forceinline__ float warp_sum(float v) {
@@ -49,29 +48,6 @@ __device__ __forceinline__ void load_row(float4 (&R)[kMaxChunks], const float* r
     const int v4 = k * kVThreads + int(threadIdx.x);
     R[k] = v4 < n_vec ? __ldg(reinterpret_cast<const float4*>(row) + v4) : make_float4(0.f, 0.f, 0.f, 0.f);
   }
-}
-
-// Element `token` of the row: its owner reads (and optionally zeroes) it and publishes it; every
-// thread gets the value.  Contains block barriers.
-__device__ __forceinline__ float take_element(float4 (&R)[kMaxChunks], int token, bool zero_it, VocabScratch& s) {
-  const int y4 = token >> 2, yk = y4 / kVThreads, yt = y4 - yk * kVThreads, ye = token & 3;
-  if (int(threadIdx.x) == yt) {
-    float val = 0.f;
-#pragma unroll
-    for (int k = 0; k < kMaxChunks; ++k) {
-      if (k == yk) {
-        val = ye == 0 ? R[k].x : ye == 1 ? R[k].y : ye == 2 ? R[k].z : R[k].w;
-        if (zero_it) {
-          if (ye == 0) R[k].x = 0.f; else if (ye == 1) R[k].y = 0.f; else if (ye == 2) R[k].z = 0.f; else R[k].w = 0.f;
-        }
-      }
-    }
-    s.pub[0] = val;
-  }
-  __syncthreads();
-  const float v = s.pub[0];
-  __syncthreads();
-  return v;
 }
 
 __device__ __forceinline__ double warp_sum_d(double v) {

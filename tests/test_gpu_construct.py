@@ -106,6 +106,50 @@ def test_zipf_rows_give_deep_trees_and_match_oracle(B):
     assert deepest >= 3            # peaked rows give chains, flat rows give stars: both shapes are exercised
 
 
+def _flat_and_peaked(seed, n_rows, vocab):
+    """Every third row flat (its node becomes the centre of a star: one stream of hundreds of draws), the others peaked."""
+    rows, uni = wl.make_draft_table(seed, n_rows, vocab, zipf=True)
+    rng = np.random.default_rng(seed + 1)
+    for i in range(0, n_rows, 3):
+        p = rng.random(vocab) + 0.05
+        rows[i] = (p / p.sum()).astype(np.float32)
+    return rows, uni
+
+
+# one and several row sums per lane (vocabularies at the edges 8192, 16384, 32768, and tiny ones), more requests than clusters
+# of 8, 4 and 2 hold at once, more rows than a worker's tables were cut for, trees of one node and of the largest size
+@pytest.mark.parametrize("vocab,n_rows,m,n_req", [(4, 3, 9, 2), (8192, 7, 70, 1), (8196, 7, 70, 1), (16384, 7, 70, 2), (16388, 7, 70, 2),
+                                                  (32768, 5, 60, 1), (2000, 40, 33, 19), (2000, 40, 33, 40), (1000, 9, 20, 80),
+                                                  (1000, 1, 40, 1), (512, 3000, 2047, 1), (4096, 900, 1, 1), (8192, 300, 1100, 1)])
+def test_greedy_tree_at_the_edges_of_the_kernel(B, vocab, n_rows, m, n_req):
+    rows, uni = _flat_and_peaked(vocab + m, n_rows, vocab)
+    roots = [(5 * r) % n_rows for r in range(n_req)]
+    got = run_gpu(B, rows, uni, roots, m=m)
+    for r in sorted({0, n_req // 2, n_req - 1}):
+        ref = orc.build_tree_greedy(rows, uni, m, root_row=roots[r])
+        if not excused(ref):
+            compare(got, r, ref)
+        else:
+            assert vocab == 4                                        # (so few tokens that equal slot values occur)
+
+
+@pytest.mark.parametrize("vocab,n_req,cap", [(2048, 1, 600), (9000, 20, 200), (20000, 1, 2047)])
+def test_threshold_stream_through_a_collapsing_residual(B, vocab, n_req, cap):
+    """Sixty tokens of probability 2^-1, 2^-2, ... and a tail of 1e-21: after some fifty draws what is left of the row is far
+    below the rounding of any sum over the whole of it, and the draws that follow must still be the oracle's.  (Halving
+    keeps 1 - r away from 0: a value v (1 - r) is only good to 1e-16 / (1 - r) in any fp64 implementation.)"""
+    rng = np.random.default_rng(vocab)
+    p = rng.random((2, vocab)) * 1e-24
+    for i in range(2):
+        p[i, rng.permutation(vocab)[:60]] = 0.5 ** np.arange(1, 61)
+    rows, uni = p.astype(np.float32), rng.random(4099, dtype=np.float32)
+    got = run_gpu(B, rows, uni, [r & 1 for r in range(n_req)], threshold=1e-25, max_nodes=cap)
+    for r in (0, n_req - 1):
+        ref = orc.build_tree_threshold(rows, uni, 1e-25, cap, root_row=r & 1)
+        assert not excused(ref) and (ref["parents"] == 0).sum() > 100 and ref["values"][100] < 2.0 ** -50
+        compare(got, r, ref)
+
+
 def test_gpu_threshold_at_last_greedy_value_builds_the_same_tree(B):
     """The paper's statement (App. B), on the GPU alone: same set of root-to-node token paths."""
     rows, uni = wl.make_draft_table(9, 32, 4096, 3.0)
