@@ -14,7 +14,10 @@
  *     "host" are ordinary host pointers that are only read during the call.
  *   - The caller owns every buffer.  Attention and mask calls enqueue kernels on `stream` and
  *     return without synchronising; the caller's buffers must stay alive until the stream reaches
- *     them.  Plan creation/destruction are the only calls that allocate or free device memory.
+ *     them.  Plan creation/destruction are the only calls that allocate or free device memory.  (A
+ *     destroyed plan may still be in use on any stream: its tables, at most 256 KB each and 32 buffers
+ *     per device, are kept for later plans and reused once the device has been waited for; destruction
+ *     itself waits for the device only now and then.  dyspec_release_cache frees them.)
  *   - Conditions only the device can see (a parent index that is not in {-1} U [0, i); a bounded
  *     wait that ran out) store a non-zero DYSPEC_ERR_* code into the optional `status` word (dev
  *     int32, the caller zeroes it) and the kernel still completes normally.

@@ -182,6 +182,7 @@ struct dyspec_plan {
   int64_t total_tiles = 0, n_groups = 0;
   // device copies (one allocation)
   void* d_blob = nullptr;
+  size_t d_blob_bytes = 0;              // (0: not from the pool, a slot's buffer)
   int device = -1;                      // the device the copies live on (the one current at creation)
   ReqInfo* d_reqs = nullptr;
   WorkItem* d_items = nullptr;
@@ -607,6 +608,74 @@ void schedule(dyspec_plan& pl) {
   }
 }
 
+// Device memory of the plans' tables.  A serving loop makes a plan for every step, and cudaMalloc, cudaFree (which waits
+// for the whole device) and a copy on the legacy stream (which waits for the step's earlier kernels) cost it about 0.9 ms
+// of host time that nothing overlapped: a step of 8 requests took 1.3 ms instead of 0.6.  So a destroyed plan's memory rests
+// here, and is used again only after a cudaFree -- one in kRestingMax destructions -- has waited for the device since:
+// whatever streams the plan ran on, nothing reads the memory any more.  Bounded to 2 kRestingMax buffers of at most
+// kPooledBytes per device (larger ones are freed at once); dyspec_release_cache gives everything back.
+constexpr size_t kPooledBytes = size_t(256) << 10;
+constexpr size_t kRestingMax = 16;
+struct TableBuffer { void* ptr; size_t bytes; };
+struct TablePool {
+  std::vector<TableBuffer> resting;     // of destroyed plans; kernels may still read them
+  std::vector<TableBuffer> idle;        // resting when the device was last waited for
+  cudaStream_t copies = nullptr;        // uploads: a stream that waits for no other
+};
+std::map<int, TablePool> g_table_pools;
+std::mutex g_table_pool_mutex;
+
+void table_pool_clear(TablePool& pool) {
+  for (auto* list : {&pool.resting, &pool.idle}) {
+    for (TableBuffer& b : *list) cudaFree(b.ptr);
+    list->clear();
+  }
+}
+
+cudaError_t table_pool_take(int device, size_t bytes, void** ptr, size_t* got, cudaStream_t* copies) {
+  std::lock_guard<std::mutex> lock(g_table_pool_mutex);
+  TablePool& pool = g_table_pools[device];
+  if (!pool.copies)
+    if (cudaError_t e = cudaStreamCreateWithFlags(&pool.copies, cudaStreamNonBlocking); e != cudaSuccess) { pool.copies = nullptr; return e; }
+  *copies = pool.copies;
+  size_t best = pool.idle.size();
+  for (size_t i = 0; i < pool.idle.size(); ++i)
+    if (pool.idle[i].bytes >= bytes && (best == pool.idle.size() || pool.idle[i].bytes < pool.idle[best].bytes)) best = i;
+  if (best < pool.idle.size()) {
+    *ptr = pool.idle[best].ptr;
+    *got = pool.idle[best].bytes;
+    pool.idle.erase(pool.idle.begin() + ptrdiff_t(best));
+    return cudaSuccess;
+  }
+  size_t size = size_t(16) << 10;       // pooled sizes are powers of two, so that a neighbouring shape's buffer fits
+  while (size < bytes) size *= 2;
+  *got = size <= kPooledBytes ? size : bytes;
+  cudaError_t e = cudaMalloc(ptr, *got);
+  if (e == cudaErrorMemoryAllocation && !(pool.resting.empty() && pool.idle.empty())) {
+    (void)cudaGetLastError();
+    table_pool_clear(pool);
+    e = cudaMalloc(ptr, *got);
+  }
+  if (e != cudaSuccess) { *ptr = nullptr; *got = 0; }
+  return e;
+}
+
+void table_pool_give(int device, void* ptr, size_t bytes) {
+  if (bytes > kPooledBytes) { cudaFree(ptr); return; }
+  std::lock_guard<std::mutex> lock(g_table_pool_mutex);
+  TablePool& pool = g_table_pools[device];
+  pool.resting.push_back({ptr, bytes});
+  if (pool.resting.size() < kRestingMax) return;
+  const TableBuffer last = pool.resting.back();
+  pool.resting.pop_back();
+  if (cudaFree(last.ptr) != cudaSuccess) return;       // (synchronises the device; on an error the rest goes on resting)
+  for (TableBuffer& b : pool.resting) {
+    if (pool.idle.size() < kRestingMax) pool.idle.push_back(b);
+    else cudaFree(b.ptr);
+  }
+  pool.resting.clear();
+}
+
 int upload(dyspec_plan& pl) {
   auto pad = [](size_t x) { return (x + 255) & ~size_t(255); };
   const size_t b_reqs = pad(std::max<size_t>(1, pl.reqs.size()) * sizeof(ReqInfo));
@@ -624,8 +693,11 @@ int upload(dyspec_plan& pl) {
   const size_t o_groups = off; off += b_groups;
   const size_t o_counters = off;
   if (cudaGetDevice(&pl.device) != cudaSuccess) return DYSPEC_ERR_CUDA;
-  if (cudaMalloc(&pl.d_blob, total) != cudaSuccess) { pl.d_blob = nullptr; return DYSPEC_ERR_CUDA; }
-  if (cudaMemcpy(pl.d_blob, host.data(), total, cudaMemcpyHostToDevice) != cudaSuccess) return DYSPEC_ERR_CUDA;
+  cudaStream_t copies = nullptr;
+  if (table_pool_take(pl.device, total, &pl.d_blob, &pl.d_blob_bytes, &copies) != cudaSuccess) return DYSPEC_ERR_CUDA;
+  if (cudaMemcpyAsync(pl.d_blob, host.data(), total, cudaMemcpyHostToDevice, copies) != cudaSuccess ||
+      cudaStreamSynchronize(copies) != cudaSuccess)
+    return DYSPEC_ERR_CUDA;
   uint8_t* base = static_cast<uint8_t*>(pl.d_blob);
   pl.d_reqs = reinterpret_cast<ReqInfo*>(base + o_reqs);
   pl.d_items = reinterpret_cast<WorkItem*>(base + o_items);
@@ -1003,7 +1075,7 @@ int dyspec_schedule_dry_run(int n_q_heads, int n_kv_heads, int head_dim, int n_r
 
 int dyspec_plan_destroy(dyspec_plan_t* plan) {
   if (!plan) return DYSPEC_OK;
-  if (plan->d_blob) cudaFree(plan->d_blob);
+  if (plan->d_blob) table_pool_give(plan->device, plan->d_blob, plan->d_blob_bytes);
   delete plan;
   return DYSPEC_OK;
 }
@@ -1229,6 +1301,15 @@ int dyspec_release_cache(void) {
     if (kv.second.workspace) cudaFree(kv.second.workspace);
   }
   g_cache.clear();
+  {
+    std::lock_guard<std::mutex> pool_lock(g_table_pool_mutex);
+    for (auto& kv : g_table_pools) {
+      if (cudaSetDevice(kv.first) != cudaSuccess) continue;
+      table_pool_clear(kv.second);
+      if (kv.second.copies) cudaStreamDestroy(kv.second.copies);
+    }
+    g_table_pools.clear();
+  }
   if (dev0 >= 0) cudaSetDevice(dev0);
   return DYSPEC_OK;
 }
