@@ -1,16 +1,17 @@
 // Parent array -> packed ancestor bitmasks and depths (Sec. 2, the mask(A) equation, plus the self bit).
 //
-// One CTA per (request, column chunk).  Rows live in shared memory and are completed by pointer
-// jumping on bitsets: every node keeps a pointer `anc` (initially its parent) and a row that covers
-// the node and all its ancestors below `anc`; one round does  row[i] |= row[anc[i]],
-// dist[i] += dist[anc[i]],  anc[i] = anc[anc[i]],  which doubles the covered path, so
-// ceil(log2(depth + 1)) rounds finish the tree.  OR-ing a row that another thread is extending in
-// the same round is harmless: every bit a row ever holds is an ancestor-or-self of its node, hence
-// an ancestor of the reader too.
-// Trees of up to 1024 nodes use one chunk (all W words of a row).  Larger trees are cut into chunks
-// of 16 words (512 columns) so that the rows still fit in shared memory: chunk c holds columns
-// [512 c, 512 c + 512) of the rows i >= 512 c (lower rows have no bit there: ancestors have smaller
-// indices) and stops following a pointer once it drops below 512 c.  Chunk 0 also writes the depths.
+// First, per 32 nodes (one word of a row) and by one warp in registers: which ancestors of a node lie in its own
+// word, and the first one that does not (pointer doubling with shuffles, at most five rounds).  Then one thread
+// per node walks from word to word to its root: parents have smaller indices, so it meets every word at
+// most once and stores it whole.  A warp's 32 rows are put together in shared memory (rows padded to an odd
+// number of words, so that the 32 threads' stores spread over the banks) and leave as one contiguous piece.
+// Rows are independent, so a request is cut into CTAs of up to 512 rows.
+// The walk takes as many steps as a node has words with ancestors: at most its depth (some 20 for a random
+// recursive tree of 2048 nodes) and at most n / 32 (a chain).  Completing all rows together by
+// pointer jumping on bitsets in one CTA per request, the earlier form of this kernel, took 1.6, 2.6, 5.1
+// and 5.4 us for random trees of 64, 512, 1024 and 2048 nodes back to back (2048: 18 us alone); now 1.2, 1.8, 2.4 and 3.6
+// (4 alone).  (Walking from parent to parent without the
+// words costs a chain of 2048 nodes 113 us.)
 // Optionally the kernel emits, per node, which 64-key tiles of the tree its row touches
 // (bit t of node_tiles[i] = row i has a visible key in columns [64 t, 64 t + 64)); the attention
 // kernel ORs these over a query tile and skips key tiles no row of it can see (App. C).
@@ -19,170 +20,138 @@
 
 namespace dyspec {
 
-// The work of one CTA: request (node0, n), column chunk blockIdx.y.
+namespace {
+constexpr int kMaskRows = 512;            // rows (threads) of a CTA at most
+
+// The work of one CTA: rows [blockDim blockIdx.y, + blockDim) of request (node0, n).
 __device__ __forceinline__ void build_tree_mask_body(const int32_t* __restrict__ parents, int node0, int n,
                                                      uint32_t* __restrict__ bits, int32_t* __restrict__ depths,
-                                                     uint32_t* __restrict__ node_tiles, int W, int CW, int32_t* status) {
+                                                     uint32_t* __restrict__ node_tiles, int W, int32_t* status) {
   extern __shared__ __align__(16) uint8_t mask_smem[];
   trigger_dependents();   // the attention kernel may start streaming K/V now; it waits for us before it reads the mask
-  if (n <= 0) return;
-  const int chunk = blockIdx.y;
-  const int W4 = W >> 2, CW4 = min(CW, W - chunk * CW) >> 2;               // 16-byte groups per row: all, this chunk's
-  const int col4 = chunk * (CW >> 2);                                      // first 16-byte group of the chunk
-  const int row0 = min(n, chunk * CW * 32);                                // rows below have no bit in these columns
-  const int nr = n - row0;
-  uint4* rows = reinterpret_cast<uint4*>(mask_smem);                       // [nr][CW4]
-  int* s_anc = reinterpret_cast<int*>(mask_smem + size_t(nr) * CW4 * 16);  // [n]
-  int* s_dist = s_anc + n;                                                 // [n]
-  uint32_t* s_occ = reinterpret_cast<uint32_t*>(s_dist + n);               // [n]
-  const int tid = threadIdx.x, nthr = blockDim.x;
+  const int nthr = int(blockDim.x), row0 = int(blockIdx.y) * nthr;
+  if (row0 >= n) return;
+  const int row_end = min(n, row0 + nthr);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int pitch = W + 1;
+  const int n_words = (row_end + 31) >> 5;
+  uint2* s_node = reinterpret_cast<uint2*>(mask_smem);          // [32 n_words] ancestors in the node's own word; the first one below it (or -1)
+  uint32_t* s_rows = reinterpret_cast<uint32_t*>(s_node + 32 * n_words) + warp * 32 * pitch;   // [32][pitch], this warp's
   bool bad = false;
-
-  for (int i = tid; i < n; i += nthr) {
-    int parent = parents[node0 + i];
-    if (parent < -1 || parent >= i) {
-      parent = -1;
-      bad = true;
+  {
+    const int step = nthr & ~31;                                 // whole warps (blockDim is a multiple of 32)
+    int i = warp * 32 + lane;
+    int parent = i < row_end ? __ldg(parents + node0 + i) : -1;
+    for (int w = warp; w < n_words; w += nthr >> 5) {
+      const int ahead = i + step < row_end ? __ldg(parents + node0 + i + step) : -1;
+      if (parent < -1 || parent >= i) {
+        bad = bad || i < row_end;
+        parent = -1;
+      }
+      uint32_t mine = 1u << lane;                                // the path from the node up to, not with, lane `up`
+      int up = parent >= w * 32 ? parent & 31 : -1, below = parent;   // `below` counts once up < 0
+      while (__any_sync(0xffffffffu, up >= 0)) {                 // every lane's path doubles: at most five rounds
+        const int src = up >= 0 ? up : lane;
+        const uint32_t m = __shfl_sync(0xffffffffu, mine, src);
+        const int u = __shfl_sync(0xffffffffu, up, src), b = __shfl_sync(0xffffffffu, below, src);
+        if (up >= 0) {
+          mine |= m;
+          up = u;
+          below = b;
+        }
+      }
+      s_node[i] = make_uint2(mine, uint32_t(below));
+      i += step;
+      parent = ahead;
     }
-    s_anc[i] = parent >= row0 ? parent : -1;        // chunk 0: row0 = 0, the plain parent
-    s_dist[i] = parent >= 0 ? 1 : 0;
-    s_occ[i] = 0u;
   }
-  for (int idx = tid; idx < nr * CW4; idx += nthr) {
-    const int r = idx / CW4, w4 = idx - r * CW4;
-    const int i = row0 + r;
-    uint4 v = make_uint4(0u, 0u, 0u, 0u);
-    if ((i >> 7) == col4 + w4) {
-      const uint32_t bit = 1u << (i & 31);
-      const int k = (i >> 5) & 3;
-      if (k == 0) v.x = bit; else if (k == 1) v.y = bit; else if (k == 2) v.z = bit; else v.w = bit;
-    }
-    rows[idx] = v;
-  }
+  for (int k = lane; k < 32 * pitch; k += 32) s_rows[k] = 0u;
   __syncthreads();
 
-  // Up to two nodes per thread (n <= 2048, 1024 threads when n > 1024).
-  for (int round = 0; round < 12; ++round) {     // 2^11 >= DYSPEC_MAX_NODES
-    int a[2] = {-1, -1}, next[2] = {-1, -1}, add[2] = {0, 0};
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      const int i = tid + k * nthr;
-      if (i < n) {
-        a[k] = s_anc[i];
-        if (a[k] >= 0) { next[k] = s_anc[a[k]]; add[k] = s_dist[a[k]]; }
-      }
+  const int i = row0 + tid;
+  uint32_t tiles = 0u;
+  int depth = -1;
+  if (i < row_end) {
+    uint32_t* row = s_rows + lane * pitch;
+    for (int a = i; a >= 0;) {                                   // every step goes to a lower word
+      const uint2 nd = s_node[a];
+      row[a >> 5] = nd.x;
+      tiles |= 1u << (a >> 6);
+      depth += __popc(nd.x);
+      a = int(nd.y);
     }
-    if (!__syncthreads_or(a[0] >= 0 || a[1] >= 0)) break;   // all pointers of this round are read before any moves
-    for (int idx = tid; idx < nr * CW4; idx += nthr) {
-      const int r = idx / CW4, w4 = idx - r * CW4;
-      const int ai = s_anc[row0 + r];            // still this round's pointer: rewritten after the next barrier
-      if (ai >= 0) {
-        const uint4 x = rows[idx], y = rows[(ai - row0) * CW4 + w4];
-        rows[idx] = make_uint4(x.x | y.x, x.y | y.y, x.z | y.z, x.w | y.w);
-      }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      const int i = tid + k * nthr;
-      if (i < n && a[k] >= 0) {
-        s_anc[i] = next[k];
-        s_dist[i] += add[k];
-      }
-    }
-    __syncthreads();
   }
+  __syncwarp();
 
   // Launched with programmatic dependent launch: everything above only read `parents` and worked in
   // shared memory, so it may overlap the tail of the kernel before it in the stream.  The outputs may
   // still be in use by that kernel (the mask of the previous call): wait for it before writing.
   grid_dependency_wait();
   if (bad && status) atomicCAS(status, 0, DYSPEC_ERR_BAD_TREE);
-  if (chunk == 0 && depths)
-    for (int i = tid; i < n; i += nthr) depths[node0 + i] = s_dist[i];
-  uint4* out = reinterpret_cast<uint4*>(bits) + size_t(node0) * W4 + col4;
-  for (int idx = tid; idx < row0 * CW4; idx += nthr) {           // rows above the chunk: all zero here
-    const int r = idx / CW4, w4 = idx - r * CW4;
-    out[size_t(r) * W4 + w4] = make_uint4(0u, 0u, 0u, 0u);
+  if (i < row_end) {
+    if (depths) depths[node0 + i] = depth;
+    if (node_tiles) node_tiles[node0 + i] = tiles;
   }
-  for (int idx = tid; idx < nr * CW4; idx += nthr) {
-    const int r = idx / CW4, w4 = idx - r * CW4;
-    const uint4 x = rows[idx];
-    out[size_t(row0 + r) * W4 + w4] = x;
-    if (node_tiles) {
-      const uint32_t t = ((x.x | x.y) ? 1u : 0u) | ((x.z | x.w) ? 2u : 0u);
-      if (t) atomicOr(&s_occ[row0 + r], t << (2 * (col4 + w4)));
-    }
-  }
-  if (node_tiles) {
-    __syncthreads();
-    if (gridDim.y == 1) {
-      for (int i = tid; i < n; i += nthr) node_tiles[node0 + i] = s_occ[i];
-    } else {
-      // a chunk of 16 words is 8 tiles: byte `chunk` of the node's word; the last chunk clears the bytes above it
-      uint8_t* o8 = reinterpret_cast<uint8_t*>(node_tiles + node0);
-      for (int i = tid; i < n; i += nthr) {
-        o8[4 * i + chunk] = uint8_t(s_occ[i] >> (8 * chunk));
-        if (chunk == int(gridDim.y) - 1)
-          for (int b = chunk + 1; b < 4; ++b) o8[4 * i + b] = 0;
-      }
-    }
+  const int first = row0 + warp * 32, rows = min(32, row_end - first), W4 = W >> 2;
+  uint4* out = reinterpret_cast<uint4*>(bits) + size_t(node0 + first) * W4;
+  for (int k = lane; k < rows * W4; k += 32) {
+    const int r = k / W4, w = (k - r * W4) * 4;
+    const uint32_t* x = s_rows + r * pitch + w;
+    out[k] = make_uint4(x[0], x[1], x[2], x[3]);
   }
 }
+}  // namespace
 
 // Request list in a plan's device table (or one request given by its size).
-__global__ void __launch_bounds__(1024, 1)
+__global__ void __launch_bounds__(kMaskRows)
 build_tree_mask_kernel(const int32_t* __restrict__ parents, const ReqInfo* __restrict__ reqs, int single_n,
                        uint32_t* __restrict__ bits, int32_t* __restrict__ depths, uint32_t* __restrict__ node_tiles,
-                       int W, int CW, int32_t* status) {
+                       int W, int32_t* status) {
   int node0 = 0, n = single_n;
   if (reqs != nullptr) {
     node0 = reqs[blockIdx.x].node0;
     n = reqs[blockIdx.x].n_nodes;
   }
-  build_tree_mask_body(parents, node0, n, bits, depths, node_tiles, W, CW, status);
+  build_tree_mask_body(parents, node0, n, bits, depths, node_tiles, W, status);
 }
 
 // Request list passed by value (kernel parameter space): a ragged batch without a plan, one launch for
 // up to kMaskBatchMax requests, one status word per request.
-__global__ void __launch_bounds__(1024, 1)
+__global__ void __launch_bounds__(kMaskRows)
 build_tree_mask_batch_kernel(const int32_t* __restrict__ parents, const __grid_constant__ MaskBatch batch,
-                             uint32_t* __restrict__ bits, int32_t* __restrict__ depths, int W, int CW, int32_t* status) {
+                             uint32_t* __restrict__ bits, int32_t* __restrict__ depths, int W, int32_t* status) {
   const int node0 = batch.node0[blockIdx.x], n = batch.node0[blockIdx.x + 1] - node0;
-  build_tree_mask_body(parents, node0, n, bits, depths, nullptr, W, CW, status ? status + batch.first_req + blockIdx.x : nullptr);
+  build_tree_mask_body(parents, node0, n, bits, depths, nullptr, W, status ? status + batch.first_req + blockIdx.x : nullptr);
 }
 
 namespace {
-struct MaskLaunch { int CW, n_chunks, threads; size_t smem; };
-MaskLaunch mask_launch_shape(int max_n, int W) {
-  MaskLaunch m;
-  m.CW = W <= 32 ? W : 16;                 // words per column chunk
-  m.n_chunks = (W + m.CW - 1) / m.CW;
-  m.smem = size_t(max_n) * m.CW * 4 + size_t(max_n) * 12;
-  m.threads = ((max_n + 31) / 32) * 32;
-  if (m.threads < 256) m.threads = 256;
-  if (m.threads > 1024) m.threads = 1024;
-  return m;
-}
+// Launch shape and programmatic dependent launch, the same for both kernels.  A CTA takes up to 512 rows: the attention kernel that follows starts early and wants whole SMs, and every SM that holds
+// a mask CTA waiting for its predecessor is one it cannot have yet (with 128 rows a CTA a call of 512 nodes came out
+// 0.5 % slower although its mask was there sooner).
+struct MaskLaunch {
+  cudaLaunchAttribute attr[1];
+  cudaLaunchConfig_t cfg = {};
+  MaskLaunch(int n_req, int max_n, int W, cudaStream_t stream) {
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    const int all = (max_n + 31) & ~31, rows = all < kMaskRows ? all : kMaskRows;
+    cfg.gridDim = dim3(unsigned(n_req), unsigned((max_n + rows - 1) / rows));
+    cfg.blockDim = dim3(unsigned(rows));
+    cfg.dynamicSmemBytes = size_t(all) * 8 + size_t(rows) * size_t(W + 1) * 4;   // at most 146 KB
+    cfg.stream = stream;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+  }
+};
 }  // namespace
 
 cudaError_t launch_build_tree_mask_batch(const int32_t* parents, const MaskBatch& batch, int n_req, int max_n, uint32_t* bits,
                                          int32_t* depths, int W, int32_t* status, cudaStream_t stream) {
   if (n_req <= 0 || max_n <= 0) return cudaSuccess;
-  const MaskLaunch m = mask_launch_shape(max_n, W);
+  const MaskLaunch m(n_req, max_n, W, stream);
   static DynSmemGrant grant;
-  if (cudaError_t e = grant.ensure(build_tree_mask_batch_kernel, m.smem); e != cudaSuccess) return e;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(unsigned(n_req), unsigned(m.n_chunks));
-  cfg.blockDim = dim3(unsigned(m.threads));
-  cfg.dynamicSmemBytes = m.smem;
-  cfg.stream = stream;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, build_tree_mask_batch_kernel, parents, batch, bits, depths, W, m.CW, status);
+  if (cudaError_t e = grant.ensure(build_tree_mask_batch_kernel, m.cfg.dynamicSmemBytes); e != cudaSuccess) return e;
+  const cudaError_t e = cudaLaunchKernelEx(&m.cfg, build_tree_mask_batch_kernel, parents, batch, bits, depths, W, status);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
@@ -190,23 +159,11 @@ cudaError_t launch_build_tree_mask(const int32_t* parents, const ReqInfo* reqs, 
                                    uint32_t* bits, int32_t* depths, uint32_t* node_tiles, int W, int32_t* status,
                                    cudaStream_t stream) {
   if (n_req <= 0 || max_n <= 0) return cudaSuccess;
-  const MaskLaunch ml = mask_launch_shape(max_n, W);
-  const int CW = ml.CW, n_chunks = ml.n_chunks, threads = ml.threads;
-  const size_t smem = ml.smem;
+  const MaskLaunch m(n_req, max_n, W, stream);
   static DynSmemGrant grant;
-  if (cudaError_t e = grant.ensure(build_tree_mask_kernel, smem); e != cudaSuccess) return e;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(unsigned(n_req), unsigned(n_chunks));
-  cfg.blockDim = dim3(unsigned(threads));
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = stream;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, build_tree_mask_kernel, parents, reqs, single_n, bits, depths, node_tiles, W,
-                                     CW, status);
+  if (cudaError_t e = grant.ensure(build_tree_mask_kernel, m.cfg.dynamicSmemBytes); e != cudaSuccess) return e;
+  const cudaError_t e = cudaLaunchKernelEx(&m.cfg, build_tree_mask_kernel, parents, reqs, single_n, bits, depths, node_tiles, W,
+                                           status);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
