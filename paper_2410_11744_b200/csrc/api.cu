@@ -1347,6 +1347,14 @@ int dyspec_tree_attention(const void* q, const void* k_cache, const void* v_cach
       if (cudaMemsetAsync(sc.workspace, 0, worst, st) != cudaSuccess) { delete pl; return DYSPEC_ERR_CUDA; }
       sc.workspace_bytes = worst;
     }
+    if (!pl->split_groups.empty()) {
+      // The counter pairs must be zero when a call starts and are left zero by it.  Plans of other sizes write their
+      // partials into the same workspace, so the counters may not follow this plan's partials as they do
+      // elsewhere: they lie behind the largest partials that any plan of the shape can have.
+      const size_t partials = pl->counters_offset, counters = pl->workspace_bytes - pl->counters_offset;
+      pl->counters_offset = (sc.workspace_bytes - (16 * size_t(pl->n_sms) + 1024)) & ~size_t(255);
+      pl->workspace_bytes = std::max(partials > pl->counters_offset ? sc.workspace_bytes + 1 : 0, pl->counters_offset + counters);
+    }
     if (pl->workspace_bytes > sc.workspace_bytes) { delete pl; return DYSPEC_ERR_WORKSPACE; }   // cannot happen (see above)
     size_t needed = 0;
     rc = send_tables(*pl, lru->blob, lru->blob_bytes, st, &needed);
