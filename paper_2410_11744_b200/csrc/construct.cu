@@ -16,10 +16,9 @@
 // draws; but streams of different rows are independent of each other and of the order in which the
 // tree takes them.  One thread-block cluster per request therefore splits the work by role:
 //
-//   planner  (warp 0 of CTA 0)  the serial part only.  Keys of the open positions lie in shared memory in
-//            groups of 32, the groups' champions in registers, the best of all in a scalar; the two values
-//            a step makes are compared with that scalar, so only a step that turns to another position needs
-//            reductions (two), and those overlap the load of that position's draw.
+//   planner  (warp 0 of CTA 0)  the serial part only.  Open positions lie in shared memory, 32 lists of them with
+//            a lane's best in its registers and the best of all in a scalar; the two values a step makes are
+//            compared with that scalar, so only a step that turns to another position needs reductions (two).
 //   helpers  (warps 1 and 2 of CTA 0)  one node behind it.  One finds the child's row in a hash table of the rows
 //            met so far and orders the row's load and first draws where it is new; the other orders further
 //            draws ahead of their use (more of them the longer a stream has become).
@@ -34,15 +33,18 @@
 //            tokens (per chunk of 1024) and over the chunks, as unevaluated pairs of doubles (error 2^-100 of
 //            the row's sum), which a draw updates by subtraction; when the residual has fallen below 2^-40
 //            of the sum the tables were built from, they are built again.  No scan is left in a draw: two
-//            compares with a ballot and eight tokens.
+//            compares with a ballot and eight tokens.  It runs ahead of the orders, which only say where its
+//            draws go.
 //
 // Messages are single words that validate themselves (a draw's record in CTA 0, a load order or a ring
 // entry in a worker CTA; written through distributed shared memory), so no hand-over needs a fence or
 // a block barrier.  Every wait is bounded; when one runs out the request reports 0 nodes.
 //
-// Measured on a B200 (vocabulary 32000, 256 language-model rows): one greedy tree of 768 nodes 5504 us with
-// the whole row re-read and re-summed by one block per node, 429 us now; eight threshold trees of 512
-// nodes 2517 -> 320 us.
+// Measured on a B200 (vocabulary 32000, 256 language-model rows): one greedy tree of 768 nodes 5466 us with
+// the whole row re-read and re-summed by one block per node, 351 us now; eight threshold trees of 512
+// nodes 2518 -> 289 us.  What bounds it: single warps' chains of dependent instructions, about four cycles
+// each -- the hot stream's 900 cycles a draw (chunk 240, sub-block 165, token 260, tables 210), the planner's
+// 500 a step, about 150 us for the first 127 nodes, whose draws are still cold (2600 cycles a draw in a stream).
 #include "vocab_ops.cuh"
 
 namespace dyspec {
@@ -55,10 +57,14 @@ constexpr int kLoadWarps = 8, kBatch = 2 * kLoadWarps;         // leaves that co
 constexpr int kMaxStages = 4;
 constexpr int kRoles = 3;              // planner and two helpers; then the drawers, the fetcher, the loaders
 constexpr int kTreeThreads = 32 * (kRoles + kDrawWarps + 1 + kLoadWarps);
-constexpr int kHotAfter = 12;          // draws used of a row before a hot CTA takes it over
-constexpr int kHotRing = 32;           // orders to a hot CTA in flight (at most kMaxAhead)
+// Draws used of a row before a hot CTA takes it over.  The root's row (with three hot CTAs) goes to the first at once: every
+// path starts there.  The second is given away early, the last one late, to a row that is sure to run on.
+constexpr int kHotSoon = 6, kHotAfter = 14;
+constexpr int kHotRing = 32;           // orders to a hot CTA in flight (at most kMaxAhead - 1 + 16)
+constexpr int kHotAhead = 256;         // draws a hot CTA may have ready before they are ordered
 constexpr int kMaxHot = 3;
 constexpr int kSub = 8, kChunk = 1024, kChunks = 32;          // hot tables: tokens per sub-block, per chunk; chunks
+constexpr int kSubs = kChunk / kSub / 32;                     // sub-blocks of a chunk per lane
 constexpr int kMaxAhead = 8;           // draws of a row that may be ordered before they are used
 constexpr uint32_t kEmpty = 0xFFFFFFFFu;
 constexpr uint32_t kFollow = 0x80000000u;   // slot: the record after this one, not linked yet when the slot was written
@@ -85,11 +91,15 @@ struct TreeLayout {
   int n_workers, first_worker, n_hot;  // hot CTAs follow CTA 0, the workers follow them
   int n_records, open_records, hash_size, ring_size, ring_shift, n_stages;
   // byte offsets
-  int rec, key, val, seq, slot, ev, first, row, rec_owner, hash_row, hash_val, entry;
+  int rec, open, note, first, rec_owner, hash_row, hash_val, entry;
   int stage, sums, load_row, attempts, number, ring, log;
-  int hot_row, hot_sub, hot_ring, hot_pub;
+  int hot_row, hot_sub, hot_ring, hot_pub, hot_number;
   int bytes;
 };
+
+__host__ __device__ inline bool root_is_hot(const TreeLayout& l) { return l.n_hot >= 3; }
+
+__host__ __device__ inline int first_loaded(const TreeLayout& l) { return root_is_hot(l) ? 1 : 0; }   // first entry that the workers see
 
 struct TreeArgs {
   const float* table;
@@ -153,21 +163,32 @@ __device__ __forceinline__ bool wait_until(F ready, const uint32_t* exit_flag) {
   }
 }
 
+// The same for a wait that may be long in ordinary operation (nothing to do yet): it ends with the tree.
+template <typename F>
+__device__ __forceinline__ bool poll(F ready, const uint32_t* exit_flag) {
+  uint64_t t0 = 0;
+  for (uint32_t spins = 1;; ++spins) {
+    if (ready()) return true;
+    if (ld_relaxed(exit_flag)) return false;
+    if ((spins & 1023u) == 0) {
+      const uint64_t now = global_timer_ns();
+      if (t0 == 0) t0 = now;
+      if (now - t0 > 4 * kWaitLimitNs) return false;
+    }
+  }
+}
+
 __device__ __forceinline__ uint32_t ld_remote(uint32_t cluster_addr) {
   uint32_t v;
   asm volatile("ld.relaxed.cluster.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(cluster_addr) : "memory");
   return v;
 }
 
-__device__ __forceinline__ unsigned long long key_of(double v) {       // order of v >= 0; 0 = no slot (taken, or NaN)
-  return v >= 0.0 ? (unsigned long long)__double_as_longlong(v + 0.0) + 1ull : 0ull;
-}
-__device__ __forceinline__ double value_of(unsigned long long key) { return __longlong_as_double((long long)(key - 1ull)); }
-
-// Lane with the largest key (ties: the smallest sequence number); `best` = that key.
-__device__ __forceinline__ int warp_best(unsigned long long key, uint32_t seq, unsigned long long& best) {
-  const uint32_t hi = uint32_t(key >> 32), lo = uint32_t(key);
-  const uint32_t mh = __reduce_max_sync(0xffffffffu, hi);
+// Lane with the largest value v (v >= 0, or -1 for none; ties: the smallest sequence number); `best` = that value.
+__device__ __forceinline__ int warp_best(double v, uint32_t seq, double& best) {
+  const int hi = __double2hiint(v);                            // grows with v; negative for -1
+  const uint32_t lo = uint32_t(__double2loint(v));
+  const int mh = __reduce_max_sync(0xffffffffu, hi);
   bool c = hi == mh;
   uint32_t b = __ballot_sync(0xffffffffu, c);
   if (b & (b - 1)) {
@@ -180,11 +201,11 @@ __device__ __forceinline__ int warp_best(unsigned long long key, uint32_t seq, u
     }
   }
   const int src = __ffs(b) - 1;
-  best = ((unsigned long long)mh << 32) | __shfl_sync(0xffffffffu, lo, src);
+  best = __hiloint2double(mh, int(__shfl_sync(0xffffffffu, lo, src)));
   return src;
 }
 
-struct Draw { double r; uint32_t token, next; };
+struct Draw { double r; uint32_t next; };
 
 // The record that `slot` stands for and its content, when it has been drawn.
 __device__ __forceinline__ bool wait_draw(const DrawRecord* recs, uint32_t& slot, Draw& d, const uint32_t* exit_flag) {
@@ -194,22 +215,34 @@ __device__ __forceinline__ bool wait_draw(const DrawRecord* recs, uint32_t& slot
     if (!wait_until([&] { nx = ld_relaxed(&recs[prev].next); return nx != kEmpty; }, exit_flag)) return false;
     slot = nx;
   }
-  const DrawRecord* rc = recs + slot;
-  unsigned long long rb = 0;
-  uint32_t t = 0;
-  if (!wait_until([&] { rb = ld_relaxed64(&rc->r_bits); t = ld_relaxed(&rc->token); return rb != ~0ull && t != kEmpty; }, exit_flag))
+  const uint32_t at = smem_u32(recs + slot);
+  unsigned long long rb = 0, tn = 0;                           // two words that are each read at once: r; token and next record
+  if (!wait_until([&] {
+        asm volatile("ld.volatile.shared.v2.u64 {%0, %1}, [%2];" : "=l"(rb), "=l"(tn) : "r"(at) : "memory");
+        return rb != ~0ull && uint32_t(tn) != kEmpty;
+      }, exit_flag))
     return false;
   d.r = __longlong_as_double((long long)rb);
-  d.token = t;
-  d.next = ld_relaxed(&rc->next);
+  d.next = uint32_t(tn >> 32);
   return true;
 }
 
+struct __align__(16) OpenSlot {        // greedy: an open position; threshold: value of the first sampling under a node
+  double v;                            // value of the position's next sampling; -1: none
+  uint32_t seq;                        // order of opening
+  uint32_t slot;                       // record of that sampling (or the one before it and kFollow)
+};
+struct __align__(16) NodeNote {
+  double v;                            // value the node was created with
+  uint32_t event;                      // parent position << 13 | record of the draw (all ones = not created)
+  uint32_t row;                        // written by the helper that reads the event
+};
+
 struct Shared {                        // pointers into one CTA's shared memory
   DrawRecord* rec;
-  unsigned long long* key;             // greedy: slot keys; threshold: value of the first sampling under a node
-  unsigned long long* val;             // value a node was created with
-  uint32_t *seq, *slot, *ev, *first, *row, *rec_owner, *hash_row;
+  OpenSlot* open;                      // greedy: position p at [p % 32][p / 32]; threshold: node k at [k]
+  NodeNote* note;
+  uint32_t *first, *rec_owner, *hash_row;
   uint32_t* hash_val;                  // entry << 16 | first record
   EntryState* entry;
 };
@@ -217,13 +250,9 @@ struct Shared {                        // pointers into one CTA's shared memory
 __device__ __forceinline__ Shared planner_view(uint8_t* sm, const TreeLayout& l) {
   Shared s;
   s.rec = reinterpret_cast<DrawRecord*>(sm + l.rec);
-  s.key = reinterpret_cast<unsigned long long*>(sm + l.key);
-  s.val = reinterpret_cast<unsigned long long*>(sm + l.val);
-  s.seq = reinterpret_cast<uint32_t*>(sm + l.seq);
-  s.slot = reinterpret_cast<uint32_t*>(sm + l.slot);
-  s.ev = reinterpret_cast<uint32_t*>(sm + l.ev);
+  s.open = reinterpret_cast<OpenSlot*>(sm + l.open);
+  s.note = reinterpret_cast<NodeNote*>(sm + l.note);
   s.first = reinterpret_cast<uint32_t*>(sm + l.first);
-  s.row = reinterpret_cast<uint32_t*>(sm + l.row);
   s.rec_owner = reinterpret_cast<uint32_t*>(sm + l.rec_owner);
   s.hash_row = reinterpret_cast<uint32_t*>(sm + l.hash_row);
   s.hash_val = reinterpret_cast<uint32_t*>(sm + l.hash_val);
@@ -231,80 +260,80 @@ __device__ __forceinline__ Shared planner_view(uint8_t* sm, const TreeLayout& l)
   return s;
 }
 
-// A node for the helpers: parent position and the record of its draw (13 bits).  Its value is for the end.
+// A node for the helpers (one lane).
 __device__ __forceinline__ void announce(const Shared& s, int k, int pos, uint32_t rec, double v) {
-  s.val[k] = (unsigned long long)__double_as_longlong(v);
-  st_relaxed(&s.ev[k], (uint32_t(pos) << 13) | rec);
-}
-
-// An open position: key, sequence number (order of opening), position.
-struct Open {
-  unsigned long long key;
-  uint32_t seq;
-  int pos;
-};
-__device__ __forceinline__ bool better(const Open& a, const Open& b) {
-  return a.key > b.key || (a.key == b.key && a.seq < b.seq);
+  s.note[k].v = v;                               // (read at the end only)
+  st_relaxed(&s.note[k].event, (uint32_t(pos) << 13) | rec);
 }
 
 // Algorithm 1's order.  Returns the number of nodes created, -1 when a wait ran out.
+// One warp, so every instruction of a step counts about four cycles.
 __device__ int plan_greedy(const TreeArgs& a, const Shared& s, const uint32_t* exit_flag) {
-  const int lane = threadIdx.x & 31;
-  const Open none{0ull, kEmpty, 0};
-  Open c0 = none, c1 = none;                     // champions of groups `lane` and `lane + 32`, without the current position
-  Open rest = none;                              // the best of them all (the same in every lane)
-  Open cur{key_of(1.0), 0u, 0};
-  uint32_t slot = kEmpty;                        // record of the current position's next draw; kEmpty: the helper names it
-  auto insert = [&](const Open& o, uint32_t rec) {
-    if (lane == 0) { s.key[o.pos] = o.key; s.seq[o.pos] = o.seq; s.slot[o.pos] = rec; }
-    const int g = o.pos >> 5;
-    if (lane == (g & 31)) {
-      if (g < 32) { if (better(o, c0)) c0 = o; }
-      else if (better(o, c1)) c1 = o;
+  const int lane = threadIdx.x & 31, per_lane = a.lay.nodes_pad >> 5;
+  double c_v = -1.0, rest_v = -1.0;              // the best open position p with p % 32 == lane; the best of all: both without the current one
+  uint32_t c_seq = kEmpty;
+  int c_pos = 0, rest_pos = 0;
+  double v = 1.0;                                // the current position, its next sampling's value and record (kEmpty: a helper names it)
+  int pos = 0;
+  uint32_t slot = kEmpty;
+  auto insert = [&](int p, double val, uint32_t seq, uint32_t rec) {
+    if (lane == (p & 31)) {
+      s.open[(p & 31) * per_lane + (p >> 5)] = OpenSlot{val, seq, rec};
+      if (val > c_v) { c_v = val; c_seq = seq; c_pos = p; }    // (opened last: it loses a tie)
     }
   };
   int n = 0;
-  while (n < a.m && cur.key != 0ull) {
-    if (slot == kEmpty && !wait_until([&] { slot = ld_relaxed(&s.first[cur.pos]); return slot != kEmpty; }, exit_flag)) return -1;
+  while (n < a.m) {
+    if (slot == kEmpty && !wait_until([&] { slot = ld_relaxed(&s.first[pos]); return slot != kEmpty; }, exit_flag)) return -1;
     Draw d;
     if (!wait_draw(s.rec, slot, d, exit_flag)) return -1;
-    const double v = value_of(cur.key), left = 1.0 - d.r;
     const int k = ++n;
-    Open stay{left > 0.0 ? key_of(v * left) : 0ull, 2u * k, cur.pos}, child{key_of(v * d.r), 2u * k + 1u, k};
+    if (lane == 0) announce(s, k, pos, slot, v);
+    const double left = 1.0 - d.r;
+    double stay = v * left, child = v * d.r;
+    if (!(left > 0.0)) stay = -1.0;
+    if (!(child >= 0.0)) child = -1.0;           // (NaN: never taken)
     const uint32_t next = d.next != kEmpty ? d.next : (slot | kFollow);
-    if (lane == 0) announce(s, k, cur.pos, slot, v);
-    const bool s_c = better(stay, child), s_r = better(stay, rest), c_r = better(child, rest);
-    if (s_c && s_r) {                            // the same position again
-      insert(child, kEmpty);
-      if (c_r) rest = child;
-      cur = stay;
+    // (equal values: the one opened first; the rest was opened before either)
+    if (stay >= child && stay > rest_v) {        // the same position again
+      insert(k, child, 2u * k + 1u, kEmpty);
+      if (child > rest_v) { rest_v = child; rest_pos = k; }
+      v = stay;
       slot = next;
-    } else if (!s_c && c_r) {                    // straight on to the new node
-      insert(stay, next);
-      if (s_r) rest = stay;
-      cur = child;
+    } else if (child > stay && child > rest_v) { // straight on to the new node
+      insert(pos, stay, 2u * k, next);
+      if (stay > rest_v) { rest_v = stay; rest_pos = pos; }
+      v = child;
+      pos = k;
       slot = kEmpty;
-    } else {                                     // another position: take it out of its group, find the best of the others
-      insert(stay, next);
-      insert(child, kEmpty);
-      cur = rest;
-      if (cur.key == 0ull) break;
+    } else {                                     // another position: take it out of its lane's list, find the best of the others
+      insert(pos, stay, 2u * k, next);
+      insert(k, child, 2u * k + 1u, kEmpty);
+      if (rest_v < 0.0) break;                   // no open position
+      v = rest_v;
+      pos = rest_pos;
       __syncwarp();
-      const int g = cur.pos >> 5;
-      slot = s.slot[cur.pos];
-      Open o{s.key[(g << 5) + lane], s.seq[(g << 5) + lane], (g << 5) + lane};
-      if (lane == (cur.pos & 31)) { o.key = 0ull; o.seq = kEmpty; s.key[cur.pos] = 0ull; s.seq[cur.pos] = kEmpty; }
-      Open top;
-      top.pos = (g << 5) + warp_best(o.key, o.seq, top.key);
-      top.seq = __shfl_sync(0xffffffffu, o.seq, top.pos & 31);
-      if (lane == (g & 31)) { if (g < 32) c0 = top; else c1 = top; }
-      const bool h = better(c1, c0);
-      const Open mine{h ? c1.key : c0.key, h ? c1.seq : c0.seq, h ? c1.pos : c0.pos};
-      const int src = warp_best(mine.key, mine.seq, rest.key);
-      rest.seq = __shfl_sync(0xffffffffu, mine.seq, src);
-      rest.pos = __shfl_sync(0xffffffffu, mine.pos, src);
+      const int src = pos & 31, at = pos >> 5;
+      OpenSlot* list = s.open + src * per_lane;
+      slot = list[at].slot;
+      double o_v = -1.0;
+      uint32_t o_seq = kEmpty;
+      int o_at = lane;
+      for (int j = lane; j < per_lane; j += 32) {              // one round up to 1024 nodes, two beyond
+        const double x = list[j].v;
+        const uint32_t q = list[j].seq;
+        if (j != at && (x > o_v || (x == o_v && q < o_seq))) { o_v = x; o_seq = q; o_at = j; }
+      }
+      if (lane == 0) list[at].v = -1.0;
+      double top;
+      const int from = warp_best(o_v, o_seq, top);
+      const uint32_t top_seq = __shfl_sync(0xffffffffu, o_seq, from);
+      const int top_at = __shfl_sync(0xffffffffu, o_at, from);
+      if (lane == src) { c_v = top; c_seq = top_seq; c_pos = top_at * 32 + src; }
+      const int who = warp_best(c_v, c_seq, rest_v);
+      rest_pos = __shfl_sync(0xffffffffu, c_pos, who);
+      __syncwarp();
     }
-    __syncwarp();
   }
   return n;
 }
@@ -313,11 +342,11 @@ __device__ int plan_greedy(const TreeArgs& a, const Shared& s, const uint32_t* e
 __device__ int plan_threshold(const TreeArgs& a, const Shared& s, const uint32_t* exit_flag) {
   const int lane = threadIdx.x & 31;
   const double t = double(a.threshold);
-  if (lane == 0) s.key[0] = (unsigned long long)__double_as_longlong(1.0);
+  if (lane == 0) s.open[0].v = 1.0;
   __syncwarp();
   int n = 0;
   for (int pos = 0; pos <= n && n < a.m; ++pos) {
-    double v = __longlong_as_double((long long)s.key[pos]);
+    double v = s.open[pos].v;
     if (!(v >= t)) continue;
     uint32_t slot = kEmpty;
     if (!wait_until([&] { slot = ld_relaxed(&s.first[pos]); return slot != kEmpty; }, exit_flag)) return -1;
@@ -326,7 +355,7 @@ __device__ int plan_threshold(const TreeArgs& a, const Shared& s, const uint32_t
       if (!wait_draw(s.rec, slot, d, exit_flag)) return -1;
       const int k = ++n;
       if (lane == 0) {
-        st_relaxed64(&s.key[k], (unsigned long long)__double_as_longlong(v * d.r));
+        st_relaxed64(&s.open[k].v, (unsigned long long)__double_as_longlong(v * d.r));
         announce(s, k, pos, slot, v);
       }
       v = v * (1.0 - d.r);
@@ -338,12 +367,17 @@ __device__ int plan_threshold(const TreeArgs& a, const Shared& s, const uint32_t
   return n;
 }
 
-// Sends the order for draw `ordinal` of a row, to be put into record `rec` (one lane).  Two warps send to the workers' rings.
-__device__ __forceinline__ void send_order(const TreeLayout& l, uint32_t* s_tail, uint32_t ring, uint32_t el_unit, uint32_t rec) {
-  const uint32_t unit = el_unit & 0xFFu, i = atomicAdd(&s_tail[unit], 1u);
+// Sends the orders for the next `n` draws of a row, to be put into records rec, rec + 1, ... (whole warp, n <= 32).  Two warps
+// send to the workers' rings.
+__device__ __forceinline__ void send_orders(const TreeLayout& l, uint32_t* s_tail, uint32_t ring, uint32_t el_unit, uint32_t rec, int n) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t unit = el_unit & 0xFFu;
+  uint32_t i = 0;
+  if (lane == 0) i = atomicAdd(&s_tail[unit], uint32_t(n));
+  i = __shfl_sync(0xffffffffu, i, 0) + uint32_t(lane);
   const bool hot = unit >= 8 * kDrawWarps;
-  const uint32_t size = hot ? uint32_t(kHotRing) : uint32_t(l.ring_size), shift = hot ? 5u : uint32_t(l.ring_shift);
-  st_remote(ring + (i & (size - 1)) * 4, (((i >> shift) & 1u) << 31) | ((el_unit >> 8) << 13) | rec);
+  const uint32_t mask = hot ? uint32_t(kHotRing - 1) : uint32_t(l.ring_size - 1), shift = hot ? 5u : uint32_t(l.ring_shift);
+  if (lane < n) st_remote(ring + (i & mask) * 4, (((i >> shift) & 1u) << 31) | ((el_unit >> 8) << 13) | (rec + uint32_t(lane)));
 }
 
 // The next node for a helper warp; false when the tree is complete (or a wait ran out).
@@ -351,7 +385,7 @@ __device__ __forceinline__ bool next_event(const Shared& s, int m, int k, uint32
   bool over = false;
   const bool got = wait_until([&] {
     if (k <= m) {
-      ev = ld_relaxed(&s.ev[k]);
+      ev = ld_relaxed(&s.note[k].event);
       if (ev != kEmpty) return true;
     }
     const uint32_t fin = ld_relaxed(s_final);
@@ -361,9 +395,9 @@ __device__ __forceinline__ bool next_event(const Shared& s, int m, int k, uint32
   return got && !over;
 }
 
-// Helper 1: rows of new nodes.
+// Helper 1: rows of new nodes.  `hot_addr` (both helpers): the hot CTAs' hand-over words, at the same offset in each.
 template <bool kGreedy>
-__device__ __forceinline__ void run_opener(const TreeArgs& a, const Shared& s, uint8_t* sm, uint32_t* s_tail, const uint32_t* s_final,
+__device__ __forceinline__ void run_opener(const TreeArgs& a, const Shared& s, uint8_t* sm, uint32_t* s_tail, uint32_t hot_addr, const uint32_t* s_final,
                                            const uint32_t* exit_flag, int req) {
   const TreeLayout& l = a.lay;
   const int lane = threadIdx.x & 31;
@@ -392,9 +426,13 @@ __device__ __forceinline__ void run_opener(const TreeArgs& a, const Shared& s, u
         const int w = next_worker, el = next_el;
         if (++next_worker == l.n_workers) { next_worker = 0; ++next_el; }
         const uint32_t cta = uint32_t(w + l.first_worker);
-        if (lane < l.n_workers) st_remote(map_to_cta(sm_addr + l.load_row + e * 4, uint32_t(l.first_worker + lane)), row);
-        const EntryState st{0, uint16_t(want), uint32_t(rec0 + want - 1), map_to_cta(sm_addr + l.ring + (el % kDrawWarps) * l.ring_size * 4, cta),
-                            (uint32_t(el) << 8) | uint32_t(w * kDrawWarps + el % kDrawWarps)};
+        const bool hot = k == 0 && root_is_hot(l);             // no draw of it is ordered elsewhere, and no worker needs the row
+        if (hot) {
+          if (lane == 0) { st_remote(map_to_cta(hot_addr + 4, 1u), 0u); st_remote(map_to_cta(hot_addr, 1u), row); }
+        } else if (lane < l.n_workers) st_remote(map_to_cta(sm_addr + l.load_row + e * 4, uint32_t(l.first_worker + lane)), row);
+        const EntryState st{0, uint16_t(want), uint32_t(rec0 + want - 1),
+                            hot ? map_to_cta(sm_addr + l.hot_ring, 1u) : map_to_cta(sm_addr + l.ring + (el % kDrawWarps) * l.ring_size * 4, cta),
+                            hot ? uint32_t(8 * kDrawWarps) : (uint32_t(el) << 8) | uint32_t(w * kDrawWarps + el % kDrawWarps)};
         if (lane < want) {
           s.rec_owner[rec0 + lane] = (uint32_t(e) << 16) | uint32_t(lane);
           if (lane + 1 < want) st_relaxed(&s.rec[rec0 + lane].next, uint32_t(rec0 + lane + 1));
@@ -404,10 +442,11 @@ __device__ __forceinline__ void run_opener(const TreeArgs& a, const Shared& s, u
           s.entry[e] = st;
           s.hash_row[at] = row;
           s.hash_val[at] = (uint32_t(e) << 16) | uint32_t(rec0);
-          __threadfence_block();                 // helper 2 reads the entry once one of these draws has been used
-          for (int i = 0; i < want; ++i) send_order(l, s_tail, st.ring, st.el_unit, uint32_t(rec0 + i));
           st_relaxed(&s.first[k], uint32_t(rec0));
         }
+        __threadfence_block();                   // helper 2 reads the entry once one of these draws has been used
+        __syncwarp();
+        send_orders(l, s_tail, st.ring, st.el_unit, uint32_t(rec0), want);
         break;
       }
     }
@@ -416,32 +455,32 @@ __device__ __forceinline__ void run_opener(const TreeArgs& a, const Shared& s, u
 
   const int32_t rr0 = a.root_row[req];
   const uint32_t row0 = uint32_t(((rr0 % a.n_rows) + a.n_rows) % a.n_rows);      // non-negative remainder: any int32 maps to a row
-  if (lane == 0) s.row[0] = row0;
+  if (lane == 0) s.note[0].row = row0;
   if (a.m > 0) open_row(0, row0);
   __syncwarp();
   uint32_t ev = kEmpty;
   for (int k = 1; next_event(s, a.m, k, ev, s_final, exit_flag); ++k) {
-    const uint32_t rec = ev & 0x1FFFu, prow = s.row[ev >> 13];
+    const uint32_t rec = ev & 0x1FFFu, prow = s.note[ev >> 13].row;
     const uint32_t y = ld_relaxed(&s.rec[rec].token);          // drawn: the planner has used it
     // row of the child (draft_row_of_child), the remainder by the prepared inverse
     const uint32_t h = prow * 2654435761u + (y + 1u) * 40503u;
     uint32_t row = h - __umulhi(h, a.rows_inverse) * uint32_t(a.n_rows);
     while (row >= uint32_t(a.n_rows)) row -= uint32_t(a.n_rows);                 // (the quotient is at most two short)
-    if (lane == 0) s.row[k] = row;
+    if (lane == 0) s.note[k].row = row;
     bool expand = k < a.m;
-    if (!kGreedy) expand = __longlong_as_double((long long)ld_relaxed64(&s.key[k])) >= t;   // (written before the event)
+    if (!kGreedy) expand = __longlong_as_double((long long)ld_relaxed64(&s.open[k].v)) >= t;   // (written before the event)
     if (expand) open_row(k, row);
     else __syncwarp();
   }
 }
 
-// Helper 2: a used draw lets its row's stream run on.  `hot_addr`: the hot CTAs' hand-over words (same offset in each).
+// Helper 2: a used draw lets its row's stream run on.
 template <bool kGreedy>
 __device__ __forceinline__ void run_orderer(const TreeArgs& a, const Shared& s, uint8_t* sm, uint32_t* s_tail, uint32_t hot_addr,
                                             const uint32_t* s_final, const uint32_t* exit_flag) {
   const TreeLayout& l = a.lay;
   const int lane = threadIdx.x & 31;
-  int next_rec = l.open_records, n_hot = 0;
+  int next_rec = l.open_records, n_hot = root_is_hot(l) ? 1 : 0;
   const uint32_t sm_addr = smem_u32(sm);
   uint32_t ev = kEmpty;
   for (int k = 1; next_event(s, a.m, k, ev, s_final, exit_flag); ++k) {
@@ -450,7 +489,7 @@ __device__ __forceinline__ void run_orderer(const TreeArgs& a, const Shared& s, 
     EntryState st = s.entry[e];
     if ((owner & 0xFFFFu) == st.consumed) {
       const int c = ++st.consumed;
-      if (c >= kHotAfter && n_hot < l.n_hot && (st.el_unit & 0xFFu) < 8 * kDrawWarps) {
+      if (n_hot < l.n_hot && c >= (n_hot + 1 < l.n_hot ? kHotSoon : kHotAfter) && (st.el_unit & 0xFFu) < 8 * kDrawWarps) {
         // to a hot CTA: the row and the records of the draws ordered so far
         const uint32_t cta = uint32_t(1 + n_hot), at = map_to_cta(hot_addr, cta), pos = ev >> 13;
         uint32_t r = ld_relaxed(&s.first[pos]), mine = r;
@@ -459,29 +498,31 @@ __device__ __forceinline__ void run_orderer(const TreeArgs& a, const Shared& s, 
           if (lane == i) mine = r;
         }
         if (lane < int(st.ordered)) st_remote(at + 8 + lane * 4, mine);
-        if (lane == 0) { st_remote(at + 4, st.ordered); st_remote(at, s.row[pos]); }
+        if (lane == 0) { st_remote(at + 4, st.ordered); st_remote(at, s.note[pos].row); }
         st.ring = map_to_cta(sm_addr + l.hot_ring, cta);
         st.el_unit = uint32_t(8 * kDrawWarps + n_hot);
         ++n_hot;
       }
-      // one record is due to every node still to come; the rest of the pool lets streams run further ahead the longer they are
-      const int spare = max(0, l.n_records - next_rec - (a.m - k) - 1);
+      // One record is due to every node still to come; the rest of the pool lets streams run further ahead the longer they
+      // are.  A hot stream, whose draws are there before they are ordered, gets its orders 16 at a time.
+      const bool hot = (st.el_unit & 0xFFu) >= 8 * kDrawWarps;
       const int lead = int(st.ordered) - c;
-      const int add = max(0, max(1, min(min(2 + c, kMaxAhead), lead + spare)) - lead);
-      if (lane < add) {
-        const uint32_t rec = uint32_t(next_rec + lane);
-        s.rec_owner[rec] = (uint32_t(e) << 16) | uint32_t(st.ordered + lane);
-        st_relaxed(&s.rec[lane ? rec - 1 : st.last].next, rec);
+      int add = hot ? (lead < kMaxAhead ? 16 : 0) : max(0, min(2 + c, kMaxAhead) - lead);
+      if (add > 0) {
+        add = min(add, max(lead < 1 ? 1 : 0, l.n_records - next_rec - (a.m - k) - 1));
+        if (add > 0) {
+          if (lane < add) {
+            const uint32_t rec = uint32_t(next_rec + lane);
+            s.rec_owner[rec] = (uint32_t(e) << 16) | uint32_t(st.ordered + lane);
+            st_relaxed(&s.rec[lane ? rec - 1 : st.last].next, rec);
+          }
+          send_orders(l, s_tail, st.ring, st.el_unit, uint32_t(next_rec), add);
+          st.ordered = uint16_t(st.ordered + add);
+          next_rec += add;
+          st.last = uint32_t(next_rec - 1);
+        }
       }
-      if (add) {
-        st.last = uint32_t(next_rec + add - 1);
-        st.ordered = uint16_t(st.ordered + add);
-      }
-      if (lane == 0) {
-        for (int i = 0; i < add; ++i) send_order(l, s_tail, st.ring, st.el_unit, uint32_t(next_rec + i));
-        s.entry[e] = st;
-      }
-      next_rec += add;
+      if (lane == 0) s.entry[e] = st;
     }
     __syncwarp();
   }
@@ -495,20 +536,6 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_
                ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
 }
 
-// Polls a barrier's phase; false once the tree is finished (or the limit has passed).
-__device__ __forceinline__ bool wait_phase(uint32_t bar, uint32_t parity, const uint32_t* exit_flag) {
-  uint64_t t0 = 0;
-  for (uint32_t spins = 0;; ++spins) {
-    if (mbar_test_wait(bar, parity)) return true;
-    if (ld_relaxed(exit_flag)) return false;
-    if ((spins & 1023u) == 0) {
-      const uint64_t now = global_timer_ns();
-      if (t0 == 0) t0 = now;
-      if (now - t0 > 4 * kWaitLimitNs) return false;
-    }
-  }
-}
-
 template <int K>
 __device__ __forceinline__ void run_fetcher(const TreeArgs& a, uint8_t* sm, int worker, unsigned long long* s_full, unsigned long long* s_empty,
                                             const uint32_t* s_never, const uint32_t* exit_flag) {
@@ -520,22 +547,12 @@ __device__ __forceinline__ void run_fetcher(const TreeArgs& a, uint8_t* sm, int 
   const int leaf0 = kLeaves * worker / l.n_workers, leaf1 = kLeaves * (worker + 1) / l.n_workers;
   uint32_t stage = 0, round = 0, issued = 0;
   bool go = true;
-  for (int e = 0; go && e < l.max_entries; ++e) {
-    uint32_t row = kEmpty;
-    uint64_t t0 = 0;
-    for (uint32_t spins = 0; go; ++spins) {                    // idle until a row is ordered or the tree is finished
-      row = ld_relaxed(s_row + e);
-      if (row != kEmpty) break;
-      if (ld_relaxed(exit_flag)) go = false;
-      if ((spins & 1023u) == 0) {
-        const uint64_t now = global_timer_ns();
-        if (t0 == 0) t0 = now;
-        if (now - t0 > 4 * kWaitLimitNs) go = false;
-      }
-    }
+  for (int e = first_loaded(l); go && e < l.max_entries; ++e) {
+    uint32_t row = kEmpty;                                     // idle until a row is ordered or the tree is finished
+    go = poll([&] { row = ld_relaxed(s_row + e); return row != kEmpty; }, exit_flag);
     for (int first = leaf0; go && first < leaf1; first += kBatch) {
       const uint32_t full = smem_u32(s_full + stage);
-      if (round > 0 && !wait_phase(smem_u32(s_empty + stage), (round - 1) & 1u, exit_flag)) { go = false; break; }
+      if (round > 0 && !poll([&] { return mbar_test_wait(smem_u32(s_empty + stage), (round - 1) & 1u); }, exit_flag)) { go = false; break; }
       const int begin = first * kLeafTokens, end = min(min(first + kBatch, leaf1) * kLeafTokens, a.vocab);
       if (end > begin) {
         const uint32_t bytes = uint32_t(end - begin) * 4u;
@@ -555,7 +572,7 @@ __device__ __forceinline__ void run_fetcher(const TreeArgs& a, uint8_t* sm, int 
   for (uint32_t k = 0; k < uint32_t(l.n_stages) && k < issued; ++k) {
     if (stage == 0) { stage = uint32_t(l.n_stages); --round; }
     --stage;
-    wait_phase(smem_u32(s_full + stage), round & 1u, s_never);
+    poll([&] { return mbar_test_wait(smem_u32(s_full + stage), round & 1u); }, s_never);
   }
 }
 
@@ -567,12 +584,12 @@ __device__ __forceinline__ void run_loader(const TreeArgs& a, uint8_t* sm, int l
   const uint32_t sums = smem_u32(sm) + uint32_t(l.sums);
   const int leaf0 = kLeaves * worker / l.n_workers, leaf1 = kLeaves * (worker + 1) / l.n_workers;
   uint32_t stage = 0, round = 0;
-  int el = 0, owner = 0;
-  for (int e = 0; e < l.max_entries; ++e) {
+  int el = first_loaded(l) / l.n_workers, owner = first_loaded(l) % l.n_workers;
+  for (int e = first_loaded(l); e < l.max_entries; ++e) {
     const uint32_t dst = map_to_cta(sums + uint32_t(el) * (kLeaves * 8), uint32_t(l.first_worker + owner));
     if (++owner == l.n_workers) { owner = 0; ++el; }
     for (int first = leaf0; first < leaf1; first += kBatch) {
-      if (!wait_phase(smem_u32(s_full + stage), round & 1u, exit_flag)) return;
+      if (!poll([&] { return mbar_test_wait(smem_u32(s_full + stage), round & 1u); }, exit_flag)) return;
       const float4* src = reinterpret_cast<const float4*>(sm + l.stage) + stage * (kBatch * K * 32);
       double q[2];
 #pragma unroll
@@ -617,17 +634,7 @@ __device__ __forceinline__ void run_drawer(const TreeArgs& a, uint8_t* sm, int d
   for (uint32_t i = 0;; ++i) {
     const uint32_t at = i & uint32_t(l.ring_size - 1), phase = (i >> l.ring_shift) & 1u;
     uint32_t msg = kEmpty;
-    uint64_t t0 = 0;
-    for (uint32_t spins = 0;; ++spins) {
-      msg = ld_relaxed(ring + at);
-      if (msg != kEmpty && (msg >> 31) == phase) break;
-      if (ld_relaxed(exit_flag)) return;
-      if ((spins & 1023u) == 0) {
-        const uint64_t now = global_timer_ns();
-        if (t0 == 0) t0 = now;
-        if (now - t0 > 4 * kWaitLimitNs) return;
-      }
-    }
+    if (!poll([&] { msg = ld_relaxed(ring + at); return msg != kEmpty && (msg >> 31) == phase; }, exit_flag)) return;
     const uint32_t el = (msg >> 13) & 0xFFFu, rec = msg & 0x1FFFu;
     uint32_t row = kEmpty, ub = kEmpty;
     if (!wait_until([&] { row = ld_relaxed(s_row + el * l.n_workers + worker); return row != kEmpty; }, exit_flag)) return;
@@ -764,7 +771,7 @@ __device__ __forceinline__ void run_drawer(const TreeArgs& a, uint8_t* sm, int d
 
 // ---- hot CTA: one row's stream from a copy of the row and prefix sums in shared memory ----
 struct __align__(16) Pair { double hi, lo; };   // hi + lo, unevaluated
-struct __align__(16) Published { double sum; unsigned long long word; };   // residual sum; phase, record, token, probability
+struct __align__(16) Published { double sum; unsigned long long word; };   // residual sum; phase, token, probability
 __device__ __forceinline__ Pair add(Pair a, Pair b) {
   const double s = a.hi + b.hi, t = s - a.hi;
   const double e = (a.hi - (s - t)) + (b.hi - t);            // Knuth's two-sum
@@ -786,20 +793,20 @@ __device__ __forceinline__ Pair scan(Pair v, int lane) {
   return v;
 }
 
-// Prefix sums over the sub-blocks of chunk c (one warp; lane = 4 sub-blocks).  Sub-block 4 l + j of a chunk lies at [j][l].
+// Prefix sums over the sub-blocks of chunk c (one warp; lane = kSubs sub-blocks).  Sub-block kSubs l + j of a chunk lies at [j][l].
 __device__ __forceinline__ void build_chunk(const float* s_row, Pair* s_sub, int c, int lane) {
-  Pair v[4];
+  Pair v[kSubs];
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
+  for (int j = 0; j < kSubs; ++j) {
     v[j] = Pair{0.0, 0.0};
-    const float* x = s_row + c * kChunk + (4 * lane + j) * kSub;
+    const float* x = s_row + c * kChunk + (kSubs * lane + j) * kSub;
 #pragma unroll
     for (int i = 0; i < kSub; ++i) v[j] = add(v[j], Pair{double(x[(i + lane) & (kSub - 1)]), 0.0});   // (any order; rotated: fewer bank conflicts)
     if (j) v[j] = add(v[j - 1], v[j]);
   }
-  const Pair upto = shfl_up_pair(scan(v[3], lane), 1);
+  const Pair upto = shfl_up_pair(scan(v[kSubs - 1], lane), 1);
 #pragma unroll
-  for (int j = 0; j < 4; ++j) s_sub[(c * 4 + j) * 32 + lane] = lane ? add(upto, v[j]) : v[j];
+  for (int j = 0; j < kSubs; ++j) s_sub[(c * kSubs + j) * 32 + lane] = lane ? add(upto, v[j]) : v[j];
 }
 
 __device__ __forceinline__ void run_hot(const TreeArgs& a, uint8_t* sm, const uint32_t* s_hot, uint32_t* s_go, const uint32_t* exit_flag) {
@@ -813,20 +820,11 @@ __device__ __forceinline__ void run_hot(const TreeArgs& a, uint8_t* sm, const ui
   // ---- one thread waits for a row: its number and how many draws have been ordered elsewhere (each word validates itself)
   if (tid == 0) {
     uint32_t row = kEmpty, n_prev = kEmpty;
-    uint64_t t0 = 0;
-    for (uint32_t spins = 0;; ++spins) {
-      row = ld_relaxed(s_hot);
-      n_prev = ld_relaxed(s_hot + 1);
-      if (row != kEmpty && n_prev != kEmpty) break;
-      if (ld_relaxed(exit_flag)) { row = kEmpty; break; }
-      if ((spins & 1023u) == 0) {
-        const uint64_t now = global_timer_ns();
-        if (t0 == 0) t0 = now;
-        if (now - t0 > 4 * kWaitLimitNs) { row = kEmpty; break; }
-      }
-    }
+    if (!poll([&] { row = ld_relaxed(s_hot); n_prev = ld_relaxed(s_hot + 1); return row != kEmpty && n_prev != kEmpty; }, exit_flag))
+      row = kEmpty;
     s_go[0] = row;
     s_go[1] = n_prev;
+    s_go[2] = 0u;                                              // draws sent
   }
   __syncthreads();
   const uint32_t row = s_go[0], n_prev = s_go[1];
@@ -834,6 +832,9 @@ __device__ __forceinline__ void run_hot(const TreeArgs& a, uint8_t* sm, const ui
   const float4* src = reinterpret_cast<const float4*>(a.table + size_t(row) * a.vocab);
   for (int i = tid; i < kChunks * kChunk / 4; i += kTreeThreads)
     reinterpret_cast<float4*>(s_row)[i] = i < (a.vocab >> 2) ? __ldg(src + i) : make_float4(0.f, 0.f, 0.f, 0.f);
+  float* s_num = reinterpret_cast<float*>(sm + l.hot_number);
+  for (int i = tid; i < a.m; i += kTreeThreads)
+    s_num[i] = __ldg(a.uniforms + draft_uniform_index(row, n_prev + uint32_t(i), uint32_t(a.n_uniforms)));
   bool good = true;
   uint32_t prev = kEmpty, gone = kEmpty;                       // (a draw ordered elsewhere may still be under way)
   if (warp == 0 && lane < int(n_prev)) {
@@ -845,93 +846,85 @@ __device__ __forceinline__ void run_hot(const TreeArgs& a, uint8_t* sm, const ui
   __syncthreads();
   for (int c = warp; c < kChunks; c += kTreeThreads / 32) build_chunk(s_row, s_sub, c, lane);
   __syncthreads();
-  if (warp == 1) {                                             // divides and sends, one draw behind the stream
+  if (warp == 1) {                                             // divides, waits for the order and sends
     if (lane != 0) return;
-    for (uint32_t i = 0;; ++i) {
-      const uint32_t at = i & uint32_t(kHotRing - 1), phase = (i / kHotRing) & 1u;
+    for (uint32_t i = 0; i < uint32_t(a.m); ++i) {
+      const Published* from = s_pub + (i & (kHotAhead - 1));
+      const uint32_t* order = ring + (i & (kHotRing - 1));
+      const uint32_t made = (i / kHotAhead) & 1u, asked = (i / kHotRing) & 1u;
       unsigned long long w = 0;
-      uint64_t t0 = 0;
-      for (uint32_t spins = 0;; ++spins) {
-        w = ld_acquire64(&s_pub[at].word);
-        if (uint32_t(w >> 63) == phase) break;
-        if (ld_relaxed(exit_flag)) return;
-        if ((spins & 1023u) == 0) {
-          const uint64_t now = global_timer_ns();
-          if (t0 == 0) t0 = now;
-          if (now - t0 > 4 * kWaitLimitNs) return;
-        }
-      }
-      const double sum = s_pub[at].sum, p = double(__uint_as_float(uint32_t(w)));
+      if (!poll([&] { w = ld_acquire64(&from->word); return uint32_t(w >> 63) == made; }, exit_flag)) return;
+      const double sum = from->sum, p = double(__uint_as_float(uint32_t(w)));
       const double r = sum > 0.0 ? p / sum : 0.0;
-      const uint32_t rec = uint32_t(w >> 47) & 0x1FFFu;
+      uint32_t msg = kEmpty;
+      if (!poll([&] { msg = ld_relaxed(order); return msg != kEmpty && (msg >> 31) == asked; }, exit_flag)) return;
+      const uint32_t rec = msg & 0x1FFFu;
       st_remote64(rec_base + rec * 16, (unsigned long long)__double_as_longlong(r));
       st_remote(rec_base + rec * 16 + 8, uint32_t(w >> 32) & 0x7FFFu);
+      st_relaxed(s_go + 2, i + 1);
     }
+    return;
   }
   if (warp != 0 || !__all_sync(0xffffffffu, good)) return;
 
   // ---- the stream.  Lane c holds the prefix sum over chunks 0 .. c.
-  Pair upto = scan(s_sub[(lane * 4 + 3) * 32 + 31], lane);
+  Pair upto = scan(s_sub[(lane * kSubs + kSubs - 1) * 32 + 31], lane);
   Pair total{__shfl_sync(0xffffffffu, upto.hi, 31), __shfl_sync(0xffffffffu, upto.lo, 31)};
   double built = total.hi;
-  float u_next = __ldg(a.uniforms + draft_uniform_index(row, n_prev, uint32_t(a.n_uniforms)));
-  for (uint32_t i = 0;; ++i) {
-    const uint32_t at = i & uint32_t(kHotRing - 1), phase = (i / kHotRing) & 1u;
+  uint32_t sent = 0;
+  float u_next = s_num[0];
+  for (uint32_t i = 0; i < uint32_t(a.m); ++i) {               // ahead of the orders, as far as the buffer goes
+    const uint32_t at = i & (kHotAhead - 1), phase = (i / kHotAhead) & 1u;
+    if (i - sent >= uint32_t(kHotAhead) &&
+        !poll([&] { sent = ld_relaxed(s_go + 2); return i - sent < uint32_t(kHotAhead); }, exit_flag))
+      return;
+    const uint32_t stop = ld_relaxed(exit_flag);
     const float u = u_next;
-    u_next = __ldg(a.uniforms + draft_uniform_index(row, n_prev + i + 1, uint32_t(a.n_uniforms)));
+    u_next = s_num[min(i + 1, uint32_t(a.m - 1))];
     const double sum = total.hi + total.lo, target = double(u) * sum;
     const double mine = upto.hi + upto.lo;
-    uint32_t msg = kEmpty;
-    uint64_t t0 = 0;
-    for (uint32_t spins = 0;; ++spins) {
-      msg = ld_relaxed(ring + at);
-      if (msg != kEmpty && (msg >> 31) == phase) break;
-      if (ld_relaxed(exit_flag)) return;
-      if ((spins & 1023u) == 0) {
-        const uint64_t now = global_timer_ns();
-        if (t0 == 0) t0 = now;
-        if (now - t0 > 4 * kWaitLimitNs) return;
-      }
-    }
-    const uint32_t rec = msg & 0x1FFFu;
     // chunk, then sub-block, then token: the first whose prefix sum exceeds the target
     const uint32_t in_chunk = __ballot_sync(0xffffffffu, mine > target);
     const bool none = in_chunk == 0u;                          // rounding (or an empty residual) left no crossing: the last token
     const int c = none ? (a.vocab - 1) / kChunk : __ffs(in_chunk) - 1;
     const double up = __shfl_sync(0xffffffffu, mine, (c - 1) & 31), before = c ? up : 0.0;
-    Pair q[4];
-    double w[4];
+    Pair q[kSubs];
+    double w[kSubs];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) q[j] = s_sub[(c * 4 + j) * 32 + lane];
+    for (int j = 0; j < kSubs; ++j) q[j] = s_sub[(c * kSubs + j) * 32 + lane];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) w[j] = before + (q[j].hi + q[j].lo);
-    const uint32_t in_sub = __ballot_sync(0xffffffffu, w[3] > target);
-    const double left = __shfl_up_sync(0xffffffffu, w[3], 1);
+    for (int j = 0; j < kSubs; ++j) w[j] = before + (q[j].hi + q[j].lo);
+    const uint32_t in_sub = __ballot_sync(0xffffffffu, w[kSubs - 1] > target);
+    const double left = __shfl_up_sync(0xffffffffu, w[kSubs - 1], 1);
     double from = lane ? left : before;                        // prefix sum in front of this lane's crossing sub-block
-    int sub = 4 * lane;
+    int sub = kSubs * lane;
 #pragma unroll
-    for (int j = 0; j < 3; ++j)
-      if (!(w[j] > target)) { from = w[j]; sub = 4 * lane + j + 1; }
+    for (int j = 0; j < kSubs - 1; ++j)
+      if (!(w[j] > target)) { from = w[j]; sub = kSubs * lane + j + 1; }
     const int who = in_sub ? __ffs(in_sub) - 1 : 31;
     sub = __shfl_sync(0xffffffffu, sub, who);
     from = __shfl_sync(0xffffffffu, from, who);
     if (none) sub = ((a.vocab - 1) % kChunk) / kSub;
     float* xs = s_row + c * kChunk + sub * kSub;
     // two tokens per lane, lanes 0 .. 3 (the others repeat them): prefix sums in front of each pair
-    const int t = lane & 3;
+    constexpr int kPairs = kSub / 2;
+    static_assert(kPairs == 4, "three lanes in front at most");
+    constexpr uint32_t kPairLanes = (1u << kPairs) - 1u;
+    const int t = lane & (kPairs - 1);
     const float2 x = reinterpret_cast<const float2*>(xs)[t];
     const double d0 = x.x, d1 = x.y, both = d0 + d1;
-    double pa = __shfl_up_sync(0xffffffffu, both, 1, 4);
-    if (t < 1) pa = 0.0;
-    double pb = __shfl_up_sync(0xffffffffu, both + pa, 2, 4);
-    if (t < 2) pb = 0.0;
-    const double at_pair = from + (pb + pa);
+    double z1 = __shfl_up_sync(0xffffffffu, both, 1, kPairs), z2 = __shfl_up_sync(0xffffffffu, both, 2, kPairs),
+           z3 = __shfl_up_sync(0xffffffffu, both, 3, kPairs);    // (three at once: a step of a scan waits for the one before)
+    if (t < 1) z1 = 0.0;
+    if (t < 2) z2 = 0.0;
+    if (t < 3) z3 = 0.0;
+    const double at_pair = from + (z3 + (z2 + z1));
     const bool h0 = at_pair + d0 > target, h1 = at_pair + both > target;
-    const uint32_t b0 = __ballot_sync(0xffffffffu, h0), b1 = __ballot_sync(0xffffffffu, h1) & 0xFu;
+    const uint32_t b0 = __ballot_sync(0xffffffffu, h0), b1 = __ballot_sync(0xffffffffu, h1) & kPairLanes;
     int lt = __ffs(b1) - 1, pick = 2 * lt + (((b0 >> (lt & 31)) & 1u) ? 0 : 1);
     double p = __shfl_sync(0xffffffffu, h0 ? d0 : d1, lt & 31);
     if (none || b1 == 0u) {                                    // rounding left no crossing: the last token with mass
-      const uint32_t m = __ballot_sync(0xffffffffu, x.x > 0.f || x.y > 0.f) & 0xFu, m1 = __ballot_sync(0xffffffffu, x.y > 0.f);
+      const uint32_t m = __ballot_sync(0xffffffffu, x.x > 0.f || x.y > 0.f) & kPairLanes, m1 = __ballot_sync(0xffffffffu, x.y > 0.f);
       lt = m ? 31 - __clz(m) : 0;
       pick = 2 * lt + int((m1 >> lt) & 1u);
       if (none) pick = (a.vocab - 1) & (kSub - 1);
@@ -943,22 +936,23 @@ __device__ __forceinline__ void run_hot(const TreeArgs& a, uint8_t* sm, const ui
     if (lane == 0) {
       xs[pick] = 0.f;
       s_pub[at].sum = sum;
-      st_release64(&s_pub[at].word, ((unsigned long long)phase << 63) | ((unsigned long long)rec << 47) | ((unsigned long long)y << 32) |
+      st_release64(&s_pub[at].word, ((unsigned long long)phase << 63) | ((unsigned long long)y << 32) |
                                         (unsigned long long)__float_as_uint(float(p)));
     }
     total = take_off(total, p);
     const Pair cut = take_off(upto, p);
     if (lane >= c) upto = cut;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
+    for (int j = 0; j < kSubs; ++j) {
       q[j] = take_off(q[j], p);
-      if (4 * lane + j >= sub) s_sub[(c * 4 + j) * 32 + lane] = q[j];
+      if (kSubs * lane + j >= sub) s_sub[(c * kSubs + j) * 32 + lane] = q[j];
     }
     __syncwarp();
+    if (stop) return;
     if (total.hi + total.lo < built * 0x1p-40) {               // (rare: what is left is small against the tables' rounding)
       for (int k = 0; k < kChunks; ++k) build_chunk(s_row, s_sub, k, lane);
       __syncwarp();
-      upto = scan(s_sub[(lane * 4 + 3) * 32 + 31], lane);
+      upto = scan(s_sub[(lane * kSubs + kSubs - 1) * 32 + 31], lane);
       total = Pair{__shfl_sync(0xffffffffu, upto.hi, 31), __shfl_sync(0xffffffffu, upto.lo, 31)};
       built = total.hi;
     }
@@ -971,7 +965,7 @@ build_tree_kernel(const __grid_constant__ TreeArgs a) {
   extern __shared__ __align__(16) uint8_t csm[];
   __shared__ uint32_t s_exit, s_never, s_final, s_log_n;       // (planner and helper do not listen to s_exit)
   __shared__ uint32_t s_tail[8 * kDrawWarps + kMaxHot];
-  __shared__ uint32_t s_hot[2 + 32], s_go[2];
+  __shared__ uint32_t s_hot[2 + 32], s_go[3];
   __shared__ uint32_t s_mask[kDrawWarps][32];
   __shared__ __align__(8) unsigned long long s_full[kMaxStages], s_empty[kMaxStages];
   const TreeLayout& l = a.lay;
@@ -997,9 +991,8 @@ build_tree_kernel(const __grid_constant__ TreeArgs a) {
   };
   if (planner_cta) {
     fill(l.rec, l.n_records * 4, kEmpty);
-    fill(l.key, l.nodes_pad * 2, 0u);
-    fill(l.seq, l.nodes_pad, kEmpty);
-    fill(l.ev, l.nodes_pad, kEmpty);
+    fill(l.note, l.nodes_pad * 4, kEmpty);
+    for (int i = tid; i < l.nodes_pad; i += kTreeThreads) reinterpret_cast<OpenSlot*>(csm + l.open)[i] = OpenSlot{-1.0, kEmpty, kEmpty};
     fill(l.first, l.nodes_pad, kEmpty);
     fill(l.hash_row, l.hash_size, kEmpty);
   }
@@ -1013,7 +1006,7 @@ build_tree_kernel(const __grid_constant__ TreeArgs a) {
   }
   if (hot_cta) {
     fill(l.hot_ring, kHotRing, kEmpty);
-    fill(l.hot_pub, kHotRing * int(sizeof(Published)) / 4, kEmpty);
+    fill(l.hot_pub, kHotAhead * int(sizeof(Published)) / 4, kEmpty);
   }
   __syncthreads();
   cluster_sync_all();
@@ -1032,7 +1025,7 @@ build_tree_kernel(const __grid_constant__ TreeArgs a) {
       for (uint32_t c = uint32_t(lane); c < n_cta; c += 32) st_remote(map_to_cta(smem_u32(&s_exit), c), 1u);
     }
   } else if (warp == 1) {
-    if (planner_cta) run_opener<kGreedy>(a, s, csm, s_tail, &s_final, &s_never, req);
+    if (planner_cta) run_opener<kGreedy>(a, s, csm, s_tail, smem_u32(s_hot), &s_final, &s_never, req);
   } else if (warp == 2) {
     if (planner_cta) run_orderer<kGreedy>(a, s, csm, s_tail, smem_u32(s_hot), &s_final, &s_never);
   } else if (worker_cta) {
@@ -1047,13 +1040,13 @@ build_tree_kernel(const __grid_constant__ TreeArgs a) {
     const int n = int(s_final);
     const size_t base = size_t(req) * (a.m + 1);
     for (int k = tid; k <= n; k += kTreeThreads) {
-      const DrawRecord rc = s.rec[k ? s.ev[k] & 0x1FFFu : 0u];
-      const double v = k ? __longlong_as_double((long long)s.val[k]) : 1.0;
-      a.parents[base + k] = k ? int32_t(s.ev[k] >> 13) : -1;
+      const NodeNote note = s.note[k];
+      const DrawRecord rc = s.rec[k ? note.event & 0x1FFFu : 0u];
+      a.parents[base + k] = k ? int32_t(note.event >> 13) : -1;
       a.tokens[base + k] = k ? int32_t(rc.token) : 0;
-      a.values[base + k] = float(v);
-      a.child_values[base + k] = k ? float(v * __longlong_as_double((long long)rc.r_bits)) : 1.f;
-      a.rows[base + k] = int32_t(s.row[k]);
+      a.values[base + k] = k ? float(note.v) : 1.f;
+      a.child_values[base + k] = k ? float(note.v * __longlong_as_double((long long)rc.r_bits)) : 1.f;
+      a.rows[base + k] = int32_t(note.row);
     }
   }
 }
@@ -1081,13 +1074,9 @@ bool tree_layout(int nodes, int n_rows, int leaf_bytes, int C, int n_hot, TreeLa
     int at = 0;
     auto take = [&](int bytes) { const int o = at; at = (at + bytes + 15) & ~15; return o; };
     l.rec = take(l.n_records * 16);
-    l.key = take(l.nodes_pad * 8);
-    l.val = take(l.nodes_pad * 8);
-    l.seq = take(l.nodes_pad * 4);
-    l.slot = take(l.nodes_pad * 4);
-    l.ev = take(l.nodes_pad * 4);
+    l.open = take(l.nodes_pad * int(sizeof(OpenSlot)));
+    l.note = take(l.nodes_pad * int(sizeof(NodeNote)));
     l.first = take(l.nodes_pad * 4);
-    l.row = take(l.nodes_pad * 4);
     l.rec_owner = take(l.n_records * 4);
     l.hash_row = take(l.hash_size * 4);
     l.hash_val = take(l.hash_size * 4);
@@ -1106,7 +1095,8 @@ bool tree_layout(int nodes, int n_rows, int leaf_bytes, int C, int n_hot, TreeLa
     l.hot_row = take(n_hot ? kChunks * kChunk * 4 : 0);
     l.hot_sub = take(n_hot ? kChunks * kChunk / kSub * int(sizeof(Pair)) : 0);
     l.hot_ring = take(n_hot ? kHotRing * 4 : 0);
-    l.hot_pub = take(n_hot ? kHotRing * int(sizeof(Published)) : 0);
+    l.hot_pub = take(n_hot ? kHotAhead * int(sizeof(Published)) : 0);
+    l.hot_number = take(n_hot ? nodes * 4 : 0);
     if (at > l.bytes) l.bytes = at;
     if (l.bytes <= 224 * 1024 && l.n_records <= kMaxRecords) return true;
     if (l.n_stages > 2) l.n_stages = 2;
