@@ -85,8 +85,10 @@ def _ptr(t) -> Optional[int]:
 
 def _stream(stream=None) -> int:
     if stream is None:
+        # The handle of torch.cuda.current_stream() without the Stream object around it: 0.4 us where that took 3.3 of the
+        # 8 - 11 us that a call cost the host, which is what a small call is bound by.
         import torch
-        return torch.cuda.current_stream().cuda_stream
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
