@@ -37,8 +37,8 @@
 //            draws go.
 //
 // Messages are single words that validate themselves (a draw's record in CTA 0, a load order or a ring
-// entry in a worker CTA; written through distributed shared memory), so no hand-over needs a fence or
-// a block barrier.  Every wait is bounded; when one runs out the request reports 0 nodes.
+// entry in a worker CTA; written through distributed shared memory), so hardly a hand-over needs
+// a fence and none a block barrier.  Every wait is bounded; when one runs out the request reports 0 nodes.
 //
 // Measured on a B200 (vocabulary 32000, 256 language-model rows): one greedy tree of 768 nodes 5466 us with
 // the whole row re-read and re-summed by one block per node, 351 us now; eight threshold trees of 512
