@@ -59,7 +59,11 @@ constexpr int kRoles = 3;              // planner and two helpers; then the draw
 constexpr int kTreeThreads = 32 * (kRoles + kDrawWarps + 1 + kLoadWarps);
 // Draws used of a row before a hot CTA takes it over.  The root's row (with three hot CTAs) goes to the first at once: every
 // path starts there.  The second is given away early, the last one late, to a row that is sure to run on.
-constexpr int kHotSoon = 6, kHotAfter = 14;
+// (6 and 14, or 4 and 8, are as good on average, but now and then give a place away to a row that stops, and the long one
+// stays with the drawers: 486 and 1457 us where 10 and 20 take 395 and 351.  A fourth hot CTA leaves three
+// workers: 127 nodes 123 us instead of 96.)
+constexpr int kHotSoon = 10, kHotAfter = 20;
+constexpr int kHotLeast = 10;          // trees up to this size have no hot CTA: its tables would not be ready in time
 constexpr int kHotRing = 32;           // orders to a hot CTA in flight (at most kMaxAhead - 1 + 16)
 constexpr int kHotAhead = 256;         // draws a hot CTA may have ready before they are ordered
 constexpr int kMaxHot = 3;
@@ -149,7 +153,8 @@ __device__ __forceinline__ void st_remote64(uint32_t cluster_addr, unsigned long
   asm volatile("st.relaxed.cluster.shared::cluster.u64 [%0], %1;" ::"r"(cluster_addr), "l"(v) : "memory");
 }
 
-// Polls `ready` (warp-uniform) until it holds; false once the exit flag is up or the limit has passed.
+// Polls `ready` (warp-uniform) until it holds; false once the limit has passed.  For the planner and the helpers, whose flag
+// never rises; the others use poll(), which ends with the tree.
 template <typename F>
 __device__ __forceinline__ bool wait_until(F ready, const uint32_t* exit_flag) {
 #pragma unroll 1
@@ -163,7 +168,7 @@ __device__ __forceinline__ bool wait_until(F ready, const uint32_t* exit_flag) {
   }
 }
 
-// The same for a wait that may be long in ordinary operation (nothing to do yet): it ends with the tree.
+// The same for a wait that may be long or in vain in ordinary operation.
 template <typename F>
 __device__ __forceinline__ bool poll(F ready, const uint32_t* exit_flag) {
   uint64_t t0 = 0;
@@ -637,12 +642,12 @@ __device__ __forceinline__ void run_drawer(const TreeArgs& a, uint8_t* sm, int d
     if (!poll([&] { msg = ld_relaxed(ring + at); return msg != kEmpty && (msg >> 31) == phase; }, exit_flag)) return;
     const uint32_t el = (msg >> 13) & 0xFFFu, rec = msg & 0x1FFFu;
     uint32_t row = kEmpty, ub = kEmpty;
-    if (!wait_until([&] { row = ld_relaxed(s_row + el * l.n_workers + worker); return row != kEmpty; }, exit_flag)) return;
+    if (!poll([&] { row = ld_relaxed(s_row + el * l.n_workers + worker); return row != kEmpty; }, exit_flag)) return;
     const uint32_t att = s_att[el];
     const float u_next = __ldg(a.uniforms + draft_uniform_index(row, att + 1, uint32_t(a.n_uniforms)));   // arrives behind this draw
     unsigned long long* sums = s_sums + size_t(el) * kLeaves;
     unsigned long long b0 = 0, b1 = 0;
-    if (!wait_until([&] {
+    if (!poll([&] {                                            // (may be cut short: the tree can be finished before the row is there)
           b0 = ld_relaxed64(sums + 2 * lane);
           b1 = ld_relaxed64(sums + 2 * lane + 1);
           ub = ld_relaxed(s_num + el);
@@ -838,8 +843,8 @@ __device__ __forceinline__ void run_hot(const TreeArgs& a, uint8_t* sm, const ui
   bool good = true;
   uint32_t prev = kEmpty, gone = kEmpty;                       // (a draw ordered elsewhere may still be under way)
   if (warp == 0 && lane < int(n_prev)) {
-    good = wait_until([&] { prev = ld_relaxed(s_hot + 2 + lane); return prev != kEmpty; }, exit_flag);
-    if (good) good = wait_until([&] { gone = ld_remote(rec_base + (prev & (kMaxRecords - 1)) * 16 + 8); return gone != kEmpty; }, exit_flag);
+    good = poll([&] { prev = ld_relaxed(s_hot + 2 + lane); return prev != kEmpty; }, exit_flag);
+    if (good) good = poll([&] { gone = ld_remote(rec_base + (prev & (kMaxRecords - 1)) * 16 + 8); return gone != kEmpty; }, exit_flag);
   }
   __syncthreads();
   if (gone != kEmpty) s_row[gone] = 0.f;
@@ -1138,7 +1143,7 @@ cudaError_t launch_tree(TreeArgs a, int n_req, cudaStream_t stream) {
   for (;; C *= 2) {
     bool fits = false;
     for (int hot = C == 8 ? kMaxHot : C == 4 ? 1 : 0; hot >= 0 && !fits; --hot)
-      fits = (hot == 0 || a.m > 2 * kHotAfter) && tree_layout(a.m, a.n_rows, leaf_bytes, C, hot, a.lay);
+      fits = (hot == 0 || a.m > kHotLeast) && tree_layout(a.m, a.n_rows, leaf_bytes, C, hot, a.lay);
     if (fits) break;
     if (C == 8) return cudaErrorInvalidConfiguration;          // not reached: 2047 nodes and rows fit
   }
