@@ -1136,7 +1136,9 @@ cudaError_t launch_tree(const TreeArgs& a, int n_req, int C, cudaStream_t stream
 
 template <bool kGreedy>
 cudaError_t launch_tree(TreeArgs a, int n_req, cudaStream_t stream) {
-  // The largest cluster with which all requests run at once; where none does, the smallest that holds the tree.
+  // The largest cluster for which the SMs suffice, n_req C <= 148; where none does, the smallest that holds the tree.  (15 clusters of
+  // 8 run at once, an SM's neighbours being what they are, but 16 - 18 requests in two waves of them take 181 us for
+  // 127 nodes where clusters of 4 take 204; 35 requests take 243 us with clusters of 4 and 409 with 2.)
   const int leaf_bytes = 512 * (a.vocab <= kLeaves * 128 ? 1 : a.vocab <= kLeaves * 256 ? 2 : 4);
   int C = 8;
   while (C > 1 && int64_t(n_req) * C > kDefaultSMs) C /= 2;
