@@ -41,8 +41,8 @@
 // a fence and none a block barrier.  Every wait is bounded; when one runs out the request reports 0 nodes.
 //
 // Measured on a B200 (vocabulary 32000, 256 language-model rows): one greedy tree of 768 nodes 5466 us with
-// the whole row re-read and re-summed by one block per node, 351 us now; eight threshold trees of 512
-// nodes 2518 -> 289 us.  What bounds it: single warps' chains of dependent instructions, about four cycles
+// the whole row re-read and re-summed by one block per node, 343 - 410 us now; eight threshold trees of 512
+// nodes 2518 -> 300 us.  What bounds it: single warps' chains of dependent instructions, about four cycles
 // each -- the hot stream's 900 cycles a draw (chunk 240, sub-block 165, token 260, tables 210), the planner's
 // 500 a step, about 150 us for the first 127 nodes, whose draws are still cold (2600 cycles a draw in a stream).
 #include "vocab_ops.cuh"
@@ -1142,17 +1142,25 @@ cudaError_t launch_tree(TreeArgs a, int n_req, cudaStream_t stream) {
   const int leaf_bytes = 512 * (a.vocab <= kLeaves * 128 ? 1 : a.vocab <= kLeaves * 256 ? 2 : 4);
   int C = 8;
   while (C > 1 && int64_t(n_req) * C > kDefaultSMs) C /= 2;
-  for (;; C *= 2) {
-    bool fits = false;
-    for (int hot = C == 8 ? kMaxHot : C == 4 ? 1 : 0; hot >= 0 && !fits; --hot)
-      fits = (hot == 0 || a.m > kHotLeast) && tree_layout(a.m, a.n_rows, leaf_bytes, C, hot, a.lay);
-    if (fits) break;
+  auto fits = [&](int c) {
+    for (int hot = c == 8 ? kMaxHot : c == 4 ? 1 : 0; hot >= 0; --hot)
+      if ((hot == 0 || a.m > kHotLeast) && tree_layout(a.m, a.n_rows, leaf_bytes, c, hot, a.lay)) return true;
+    return false;
+  };
+  while (!fits(C)) {
     if (C == 8) return cudaErrorInvalidConfiguration;          // not reached: 2047 nodes and rows fit
+    C *= 2;
   }
   a.rows_inverse = uint32_t((1ull << 32) / uint64_t(a.n_rows) - (a.n_rows == 1 ? 1 : 0));
-  if (a.vocab <= kLeaves * 128) return launch_tree<kGreedy, 1>(a, n_req, C, stream);
-  if (a.vocab <= kLeaves * 256) return launch_tree<kGreedy, 2>(a, n_req, C, stream);
-  return launch_tree<kGreedy, 4>(a, n_req, C, stream);
+  for (;;) {
+    const cudaError_t e = a.vocab <= kLeaves * 128   ? launch_tree<kGreedy, 1>(a, n_req, C, stream)
+                          : a.vocab <= kLeaves * 256 ? launch_tree<kGreedy, 2>(a, n_req, C, stream)
+                                                     : launch_tree<kGreedy, 4>(a, n_req, C, stream);
+    // a share of a device whose SMs hold no cluster of this size: a smaller one, if the tree fits there
+    if (e != cudaErrorInvalidClusterSize || C == 1 || !fits(C / 2)) return e;
+    (void)cudaGetLastError();
+    C /= 2;
+  }
 }
 
 }  // namespace

@@ -418,16 +418,15 @@ cudaError_t launch_verify_tree(const int32_t* parents, const int32_t* tokens, co
   const int n_chunks = (vocab + 4 * kVThreads - 1) / (4 * kVThreads);
   int C = 8, K = 1;
   while (C > 1 && (C >= 2 * n_chunks || int64_t(n_req) * C > kDefaultSMs)) C /= 2;
-  while (K * C < n_chunks) K *= 2;
   auto go = [&](auto launch) {
     return launch(C, parents, tokens, draft_probs, target_probs, accept_u, sample_u, node_offsets, n_req, max_nodes, vocab,
                   bonus_at_leaf, out_tokens, out_nodes, out_count, max_out, status, stream);
   };
-  switch (K) {
-    case 1: return go(launch_parts<1>);
-    case 2: return go(launch_parts<2>);
-    case 4: return go(launch_parts<4>);
-    default: return go(launch_parts<8>);
+  for (;; C /= 2) {
+    while (K * C < n_chunks) K *= 2;
+    const cudaError_t e = K == 1 ? go(launch_parts<1>) : K == 2 ? go(launch_parts<2>) : K == 4 ? go(launch_parts<4>) : go(launch_parts<8>);
+    if (e != cudaErrorInvalidClusterSize || C == 1) return e;
+    (void)cudaGetLastError();            // a share of a device whose SMs hold no cluster of this size: a smaller one
   }
 }
 
