@@ -467,8 +467,8 @@ __device__ __forceinline__ void run_opener(const TreeArgs& a, const Shared& s, u
   for (int k = 1; next_event(s, a.m, k, ev, s_final, exit_flag); ++k) {
     const uint32_t rec = ev & 0x1FFFu, prow = s.note[ev >> 13].row;
     const uint32_t y = ld_relaxed(&s.rec[rec].token);          // drawn: the planner has used it
-    // row of the child (draft_row_of_child), the remainder by the prepared inverse
-    const uint32_t h = prow * 2654435761u + (y + 1u) * 40503u;
+    // row of the child: the remainder by the prepared inverse
+    const uint32_t h = draft_child_hash(prow, y);
     uint32_t row = h - __umulhi(h, a.rows_inverse) * uint32_t(a.n_rows);
     while (row >= uint32_t(a.n_rows)) row -= uint32_t(a.n_rows);                 // (the quotient is at most two short)
     if (lane == 0) s.note[k].row = row;
