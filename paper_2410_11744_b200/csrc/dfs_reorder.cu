@@ -25,53 +25,12 @@
 // A parent outside {-1} U [0, i) makes that node a root and reports DYSPEC_ERR_BAD_TREE, as in the
 // mask builder.
 #include "common.cuh"
+#include "dfs_layout.h"
 
 namespace dyspec {
 
 namespace {
 constexpr uint32_t kNone = 0xFFFFu;
-
-// Splitters among E tour elements.
-constexpr uint32_t kSpread = 2654435769u;          // odd
-constexpr uint32_t spread_inverse() {              // modulo 2^32, hence modulo every smaller power of two (Newton)
-  uint32_t x = kSpread;
-  for (int k = 0; k < 5; ++k) x *= 2u - kSpread * x;
-  return x;
-}
-constexpr uint32_t kSpreadInverse = spread_inverse();
-static_assert(kSpread * kSpreadInverse == 1u, "inverse");
-struct Splitters {
-  uint32_t mask;                                   // a power of two - 1, at least E - 1
-  int count;                                       // numbers 0 .. count - 1 (some stand for no element)
-  __host__ __device__ explicit Splitters(int E) : mask(31u) {
-#ifdef __CUDA_ARCH__
-    mask |= 0xFFFFFFFFu >> __clz(E - 1 | 1);
-#else
-    while (mask < uint32_t(E - 1)) mask = 2u * mask + 1u;
-#endif
-    count = mask < 128u ? int(mask) + 1 : 7 * int((mask + 1u) >> 5);   // (short lists: all of them, no walk)
-  }
-  __device__ __forceinline__ int number(uint32_t e) const { return int((e * kSpread) & mask); }        // a splitter if < count
-  __device__ __forceinline__ uint32_t element(int k) const { return (uint32_t(k) * kSpreadInverse) & mask; }
-};
-
-// Shared memory of a tree of n nodes (byte offsets).
-struct DfsLayout {
-  int par, fc, ns, chunks, table, next, at, jump, bytes;
-  __host__ __device__ explicit DfsLayout(int n) {
-    const int n16 = (n + 1 + 31) & ~31;
-    par = 0;
-    fc = par + 2 * n16;
-    ns = fc + 2 * n16;
-    chunks = ns + 2 * n16;
-    table = chunks + 8 * n16;
-    next = table;                                  // the table of step 1 is dead when the tour is written
-    at = next + 4 * n16;
-    jump = at + 8 * n16;
-    const int lists = jump + 8 * Splitters(2 * n).count, tabled = table + (n + 1) * ((n + 31) >> 5);
-    bytes = lists > tabled ? lists : tabled;
-  }
-};
 constexpr int kJumpThreads = 256;
 }
 

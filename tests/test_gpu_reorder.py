@@ -243,3 +243,31 @@ def test_reorder_reports_bad_parent(rt):
     torch.cuda.synchronize()
     assert int(status.item()) == -5
     assert order.cpu().numpy().tolist() == orc.dfs_order(fixed)
+
+
+@pytest.mark.parametrize("sizes", [[64, 65], [65, 64], [64, 95], [33, 64, 80], [64, 96], [1, 32, 64, 65, 128, 129], [63, 64, 256, 257], [64, 2048, 65]])
+def test_dfs_reorder_ragged_sizes_share_one_launch(rt, sizes):
+    """Requests whose shared-memory layouts differ, in one launch sized by the largest."""
+    import torch
+    B, _ = rt
+    rng = np.random.default_rng(sum(sizes))
+    trees = [wl.random_tree(rng, n) for n in sizes]
+    total, rows = sum(sizes), [10 + n for n in sizes]
+    plan = B.Plan(4, 4, 64, [10] * len(sizes), sizes, np.concatenate([[0], np.cumsum(rows)[:-1]]).tolist(), sum(rows),
+                  B.dyspec_words_per_row(max(sizes)), 0.0)
+    dev = "cuda:0"
+    parents = torch.from_numpy(np.concatenate(trees).astype(np.int32)).to(dev)
+    order, new_of_old, new_parents = (torch.full((total,), -7, dtype=torch.int32, device=dev) for _ in range(3))
+    status = torch.zeros(1, dtype=torch.int32, device=dev)
+    B.dyspec_plan_dfs_reorder(plan, parents, order, new_of_old, new_parents, status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    at = 0
+    for tree in trees:
+        n = len(tree)
+        ref_order = orc.dfs_order(tree)
+        ref_parents, ref_new_of_old = orc.relabel_tree(tree, ref_order)
+        assert np.array_equal(order.cpu().numpy()[at:at + n], np.asarray(ref_order, np.int32))
+        assert np.array_equal(new_of_old.cpu().numpy()[at:at + n], ref_new_of_old)
+        assert np.array_equal(new_parents.cpu().numpy()[at:at + n], ref_parents)
+        at += n
