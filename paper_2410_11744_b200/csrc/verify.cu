@@ -96,8 +96,9 @@ verify_tree_kernel(const int32_t* __restrict__ parents, const int32_t* __restric
       out_count[r] = 0;
       if (n > max_nodes && status) atomicCAS(status, 0, DYSPEC_ERR_INVALID_ARG);
     }
-    return;
+    return;                                 // (all CTAs of the request)
   }
+  cluster_arrive();                         // "this CTA has started": only then may the others write its shared memory
   bool bad = false;
   for (int i = tid; i < n; i += kVThreads) {
     int p_ = parents[node0 + i];
@@ -128,6 +129,7 @@ verify_tree_kernel(const int32_t* __restrict__ parents, const int32_t* __restric
     s_go[p] = go;
   }
   __syncthreads();
+  cluster_wait();                           // (here, where every path passes; the loads above hide it)
 
   auto emit = [&](int token, int node) {
     if (writer && n_out < max_out) { out_tokens[size_t(r) * max_out + n_out] = token; out_nodes[size_t(r) * max_out + n_out] = node; }

@@ -19,3 +19,14 @@ def test_every_split_of_the_vocabulary(B, vocab, n_req):  # noqa: F811
              else wl.greedy_tree(rng, 6, 3, 0.5) for r in range(n_req)]
     case = wl.make_verify_case(vocab + n_req, vocab, trees, sharpness=2.0, disagreement=(0.2, 1.5)[n_req & 1])
     check(B, case, bonus=bool(vocab & 4), max_excused=1 + n_req // 25)
+
+
+@pytest.mark.parametrize("n_req", [1, 18, 37, 74])
+@pytest.mark.parametrize("bonus", [True, False])
+def test_requests_that_reach_an_exchange_at_once(B, n_req, bonus):  # noqa: F811
+    """Single nodes (with the bonus token: a draw straight away; without: no exchange at all), pairs and empty requests beside
+    each other: the shortest way from a CTA's start to its first store into another's memory, and the ways around it."""
+    trees = [wl.chain_tree(1 + r % 2) if r % 5 else np.zeros(0, np.int32) for r in range(1, n_req + 1)]
+    case = wl.make_verify_case(n_req, 32000, trees, sharpness=2.0, disagreement=1.5)
+    for _ in range(3):
+        check(B, case, bonus=bonus, max_excused=1 + n_req // 25)
