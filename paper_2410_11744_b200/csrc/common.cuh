@@ -116,23 +116,28 @@ struct AttnParams {
   int32_t n_items_total;
 };
 
-// Dynamic shared memory above 48 KB has to be granted per (kernel, device).  One of these per kernel
-// remembers what each device of the process has been granted so far; safe to call from several
-// host threads (the worst case is a repeated, idempotent grant).
+// Without a grant a launch is held to 48 KB of shared memory, static and dynamic together.  One of these per kernel
+// grants it all that is left beside its static part, once per device of the process: what a later launch
+// may ask for does not depend on what earlier ones did.  Safe to call from several host threads (the worst case
+// is a repeated, identical grant).
 struct DynSmemGrant {
   static constexpr int kDevices = 64;
   std::atomic<size_t> granted[kDevices];
   template <typename Kernel>
   cudaError_t ensure(Kernel kernel, size_t bytes) {
-    if (bytes <= 48 * 1024) return cudaSuccess;
     int dev = -1;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     const bool cached = dev >= 0 && dev < kDevices;
     if (cached && granted[dev].load(std::memory_order_acquire) >= bytes) return cudaSuccess;
-    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes));
-    if (e != cudaSuccess) return e;
-    if (cached) granted[dev].store(bytes, std::memory_order_release);
+    cudaFuncAttributes attr;
+    int most = 0;
+    if (e = cudaFuncGetAttributes(&attr, kernel); e != cudaSuccess) return e;
+    if (e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev); e != cudaSuccess) return e;
+    most -= int(attr.sharedSizeBytes);
+    if (size_t(most) < bytes) return cudaErrorInvalidConfiguration;      // no grant would do: no launch either
+    if (e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most); e != cudaSuccess) return e;
+    if (cached) granted[dev].store(size_t(most), std::memory_order_release);
     return cudaSuccess;
   }
 };
