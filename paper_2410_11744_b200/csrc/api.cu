@@ -47,13 +47,13 @@ cudaError_t launch_compact_kv(void* k_cache, void* v_cache, const int64_t* kv_ro
                               const int32_t* accepted_nodes, const int32_t* n_accepted, int n_req, int max_out,
                               int row_bytes, int keep_root, int32_t* new_prefix_len, cudaStream_t stream);
 cudaError_t launch_attn_small(int head_dim, int n_ctas, const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv,
-                            const AttnParams& p, const WorkItem* host_items, cudaStream_t stream);
+                            const AttnParams& p, const WorkItem* host_items, bool early_start, cudaStream_t stream);
 cudaError_t launch_combine(int head_dim, int bm, int n_split_groups, const AttnParams& p, cudaStream_t stream);
 int attn_tc_max_clusters(int head_dim, int cluster_size);
 int attn_small_max_clusters(int head_dim, int cluster_size);
 size_t attn_tc_cluster_workspace_per_cta(int head_dim, int cluster_size);
 cudaError_t launch_attn_tc(int head_dim, int n_ctas, const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv,
-                           const AttnParams& p, const WorkItem* host_items, cudaStream_t stream);
+                           const AttnParams& p, const WorkItem* host_items, bool early_start, cudaStream_t stream);
 }  // namespace dyspec
 
 using namespace dyspec;
@@ -1156,10 +1156,15 @@ int dyspec_tree_attention_ragged(const dyspec_plan_t* plan, const void* q, const
                                              workspace_bytes, status, stream);
 }
 
+// Whether an attention launch reads the work list before it waits for the kernels in front of it: every item but the first
+// of the first kFirstItems CTAs, which travel with the launch.  Such a launch may not start early right behind
+// write_table.  (Holding back every launch behind a table took a decoding loop of ten new sizes from 272 to 289 us.)
+static bool list_read_early(const dyspec_plan& pl) { return pl.items_stride > 1 || pl.n_ctas > kFirstItems; }
+
 static int run_attention(const dyspec_plan_t* plan, const void* q, const void* k_cache, const void* v_cache,
                          const int32_t* page_table, int pages_per_req, const uint32_t* ancestor_bits,
                          const uint32_t* node_tiles, void* out, void* workspace, size_t workspace_bytes, int32_t* status,
-                         dyspec_stream_t stream);
+                         dyspec_stream_t stream, bool tables_in_stream = false);
 
 int dyspec_tree_attention_ragged_sparse(const dyspec_plan_t* plan, const void* q, const void* k_cache,
                                         const void* v_cache, const uint32_t* ancestor_bits, const uint32_t* node_tiles,
@@ -1187,7 +1192,7 @@ int dyspec_tree_attention_paged(const dyspec_plan_t* plan, const void* q, const 
 static int run_attention(const dyspec_plan_t* plan, const void* q, const void* k_cache, const void* v_cache,
                          const int32_t* page_table, int pages_per_req, const uint32_t* ancestor_bits,
                          const uint32_t* node_tiles, void* out, void* workspace, size_t workspace_bytes, int32_t* status,
-                         dyspec_stream_t stream) {
+                         dyspec_stream_t stream, bool tables_in_stream) {
   if (!plan) return DYSPEC_ERR_INVALID_ARG;
   if (!aligned(node_tiles, 4)) return DYSPEC_ERR_INVALID_ARG;
   if (plan->n_ctas == 0) return DYSPEC_OK;
@@ -1234,8 +1239,9 @@ static int run_attention(const dyspec_plan_t* plan, const void* q, const void* k
   for (p.page_shift = 0; page_table && (1 << p.page_shift) < plan->page_size; ++p.page_shift) {}
 
   cudaError_t e;
-  if (plan->regime == 0) e = launch_attn_small(plan->d, plan->n_ctas, mq, mk, mv, p, plan->items_strided.data(), st);
-  else e = launch_attn_tc(plan->d, plan->n_ctas, mq, mk, mv, p, plan->items_strided.data(), st);
+  const bool early = !tables_in_stream || !list_read_early(*plan);
+  if (plan->regime == 0) e = launch_attn_small(plan->d, plan->n_ctas, mq, mk, mv, p, plan->items_strided.data(), early, st);
+  else e = launch_attn_tc(plan->d, plan->n_ctas, mq, mk, mv, p, plan->items_strided.data(), early, st);
   if (e != cudaSuccess) return cuda_failed(e, "attention launch");
   if (plan->merge_in_kernel) return DYSPEC_OK;
   e = launch_combine(plan->d, bm, int(plan->split_groups.size()), p, st);
@@ -1329,6 +1335,7 @@ int dyspec_tree_attention(const void* q, const void* k_cache, const void* v_cach
   memcpy(&scale_bits, &g_shape.scale, 4);
   ShapeCache& sc = g_cache[std::make_tuple(dev, g_shape.hq, g_shape.hkv, g_shape.d, g_shape.W, scale_bits)];
   SingleSlot* hit = nullptr;
+  bool tables_in_stream = false;        // the tables are written by a launch right in front of the attention call
   SingleSlot* lru = &sc.slot[0];
   for (SingleSlot& sl : sc.slot) {
     if (sl.plan && sl.prefix_len == prefix_len && sl.n_nodes == n_nodes) hit = &sl;
@@ -1372,10 +1379,11 @@ int dyspec_tree_attention(const void* q, const void* k_cache, const void* v_cach
     delete lru->plan;
     lru->plan = pl; lru->prefix_len = prefix_len; lru->n_nodes = n_nodes;
     hit = lru;
+    tables_in_stream = true;
   }
   hit->used = ++sc.clock;
-  return dyspec_tree_attention_ragged(hit->plan, q, k_cache, v_cache, ancestor_bits, out, sc.workspace,
-                                      sc.workspace_bytes, nullptr, stream);
+  return run_attention(hit->plan, q, k_cache, v_cache, nullptr, 0, ancestor_bits, nullptr, out, sc.workspace, sc.workspace_bytes,
+                       nullptr, stream, tables_in_stream);
 }
 
 }  // extern "C"
@@ -1469,8 +1477,9 @@ extern "C" int dyspec_tree_attention_static(const void* q, const void* k_cache, 
   p.cluster_size = pl->cluster;
 
   cudaError_t e;
-  if (pl->regime == 0) e = launch_attn_small(pl->d, pl->n_ctas, mq, mk, mv, p, pl->items_strided.data(), st);
-  else e = launch_attn_tc(pl->d, pl->n_ctas, mq, mk, mv, p, pl->items_strided.data(), st);
+  const bool early = !list_read_early(*pl);   // (the launch in front writes the list)
+  if (pl->regime == 0) e = launch_attn_small(pl->d, pl->n_ctas, mq, mk, mv, p, pl->items_strided.data(), early, st);
+  else e = launch_attn_tc(pl->d, pl->n_ctas, mq, mk, mv, p, pl->items_strided.data(), early, st);
   if (e != cudaSuccess) return DYSPEC_ERR_CUDA;
   if (pl->merge_in_kernel) return DYSPEC_OK;
   e = launch_combine(pl->d, bm, int(pl->split_groups.size()), p, st);

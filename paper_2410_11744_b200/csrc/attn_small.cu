@@ -830,7 +830,8 @@ int attn_small_max_clusters(int head_dim, int cluster_size) {
 }
 
 cudaError_t launch_attn_small(int head_dim, int n_ctas, const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv,
-                            const AttnParams& p, const WorkItem* host_items, cudaStream_t stream) {
+                            const AttnParams& p, const WorkItem* host_items, bool early_start, cudaStream_t stream) {
+  // early_start: programmatic dependent launch, which reads the work list before it waits for the kernels in front of it.
   // host_items: the host copy of p.items (same stride); each CTA's first item travels as a kernel parameter
   FirstItems first;
   for (int c = 0; c < kFirstItems; ++c)
@@ -838,18 +839,23 @@ cudaError_t launch_attn_small(int head_dim, int n_ctas, const CUtensorMap& mq, c
   const size_t smem = attn_small_smem_bytes(head_dim);
   static DynSmemGrant grant[2];
   cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  attr[1].id = cudaLaunchAttributeClusterDimension;
-  attr[1].val.clusterDim.x = unsigned(p.cluster_size > 1 ? p.cluster_size : 1);
-  attr[1].val.clusterDim.y = 1;
-  attr[1].val.clusterDim.z = 1;
+  unsigned n_attr = 0;
+  if (early_start) {
+    attr[n_attr].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[n_attr++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (p.cluster_size > 1) {
+    attr[n_attr].id = cudaLaunchAttributeClusterDimension;      // cluster plans: one cluster per split group
+    attr[n_attr].val.clusterDim.x = unsigned(p.cluster_size);
+    attr[n_attr].val.clusterDim.y = 1;
+    attr[n_attr++].val.clusterDim.z = 1;
+  }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(unsigned(n_ctas));
   cfg.blockDim = dim3(unsigned(kThreads));
   cfg.stream = stream;
   cfg.attrs = attr;
-  cfg.numAttrs = p.cluster_size > 1 ? 2 : 1;
+  cfg.numAttrs = n_attr;
   cudaError_t e = cudaSuccess;
   if (head_dim == 128) {
     if (cudaError_t ge = grant[0].ensure(tree_attn_small_kernel<128>, smem); ge != cudaSuccess) return ge;

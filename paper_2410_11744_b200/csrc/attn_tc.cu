@@ -1369,24 +1369,30 @@ int attn_tc_max_clusters(int head_dim, int cluster_size) {
 }
 
 cudaError_t launch_attn_tc(int head_dim, int n_ctas, const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv,
-                           const AttnParams& p, const WorkItem* host_items, cudaStream_t stream) {
+                           const AttnParams& p, const WorkItem* host_items, bool early_start, cudaStream_t stream) {
+  // early_start: programmatic dependent launch, which reads the work list before it waits for the kernels in front of it.
   // host_items: the host copy of p.items (same layout); each CTA's first item travels as a kernel parameter
   FirstItems first;
   const size_t stride = p.queue != nullptr ? 1 : size_t(p.items_stride);
   for (int c = 0; c < kFirstItems; ++c) first.item[c] = c < n_ctas ? host_items[size_t(c) * stride] : WorkItem{};
   cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  attr[1].id = cudaLaunchAttributeClusterDimension;      // cluster plans: one cluster per split group
-  attr[1].val.clusterDim.x = unsigned(p.cluster_size > 1 ? p.cluster_size : 1);
-  attr[1].val.clusterDim.y = 1;
-  attr[1].val.clusterDim.z = 1;
+  unsigned n_attr = 0;
+  if (early_start) {
+    attr[n_attr].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[n_attr++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (p.cluster_size > 1) {
+    attr[n_attr].id = cudaLaunchAttributeClusterDimension;      // cluster plans: one cluster per split group
+    attr[n_attr].val.clusterDim.x = unsigned(p.cluster_size);
+    attr[n_attr].val.clusterDim.y = 1;
+    attr[n_attr++].val.clusterDim.z = 1;
+  }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(unsigned(n_ctas));
   cfg.blockDim = dim3(unsigned(kThreads));
   cfg.stream = stream;
   cfg.attrs = attr;
-  cfg.numAttrs = p.cluster_size > 1 ? 2 : 1;
+  cfg.numAttrs = n_attr;
   const bool dyn = p.queue != nullptr;
   cudaError_t le = cudaSuccess;
   if (head_dim == 128) {
