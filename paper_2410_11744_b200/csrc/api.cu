@@ -630,6 +630,7 @@ struct TablePool {
   std::vector<TableBuffer> resting;     // of destroyed plans; kernels may still read them
   std::vector<TableBuffer> idle;        // resting when the device was last waited for
   cudaStream_t copies = nullptr;        // uploads: a stream that waits for no other
+  int uploads = 0;                      // of plans being created: the stream stays as long as there are any
 };
 std::map<int, TablePool> g_table_pools;
 std::mutex g_table_pool_mutex;
@@ -641,6 +642,7 @@ void table_pool_clear(TablePool& pool) {
   }
 }
 
+// On success an upload is counted, until table_pool_uploaded.
 cudaError_t table_pool_take(int device, size_t bytes, void** ptr, size_t* got, cudaStream_t* copies) {
   std::lock_guard<std::mutex> lock(g_table_pool_mutex);
   TablePool& pool = g_table_pools[device];
@@ -654,6 +656,7 @@ cudaError_t table_pool_take(int device, size_t bytes, void** ptr, size_t* got, c
     *ptr = pool.idle[best].ptr;
     *got = pool.idle[best].bytes;
     pool.idle.erase(pool.idle.begin() + ptrdiff_t(best));
+    ++pool.uploads;
     return cudaSuccess;
   }
   size_t size = size_t(16) << 10;       // pooled sizes are powers of two, so that a neighbouring shape's buffer fits
@@ -666,7 +669,13 @@ cudaError_t table_pool_take(int device, size_t bytes, void** ptr, size_t* got, c
     e = cudaMalloc(ptr, *got);
   }
   if (e != cudaSuccess) { *ptr = nullptr; *got = 0; }
+  else ++pool.uploads;
   return e;
+}
+
+void table_pool_uploaded(int device) {
+  std::lock_guard<std::mutex> lock(g_table_pool_mutex);
+  --g_table_pools[device].uploads;
 }
 
 void table_pool_give(int device, void* ptr, size_t bytes) {
@@ -715,9 +724,10 @@ int upload(dyspec_plan& pl) {
   if (cudaGetDevice(&pl.device) != cudaSuccess) return DYSPEC_ERR_CUDA;
   cudaStream_t copies = nullptr;
   if (table_pool_take(pl.device, image.bytes, &pl.d_blob, &pl.d_blob_bytes, &copies) != cudaSuccess) return DYSPEC_ERR_CUDA;
-  if (cudaMemcpyAsync(pl.d_blob, host.data(), image.bytes, cudaMemcpyHostToDevice, copies) != cudaSuccess ||
-      cudaStreamSynchronize(copies) != cudaSuccess)
-    return DYSPEC_ERR_CUDA;
+  const bool sent = cudaMemcpyAsync(pl.d_blob, host.data(), image.bytes, cudaMemcpyHostToDevice, copies) == cudaSuccess &&
+                    cudaStreamSynchronize(copies) == cudaSuccess;
+  table_pool_uploaded(pl.device);
+  if (!sent) return DYSPEC_ERR_CUDA;
   image.point(pl, pl.d_blob);
   return DYSPEC_OK;
 }
@@ -1313,11 +1323,14 @@ int dyspec_release_cache(void) {
   {
     std::lock_guard<std::mutex> pool_lock(g_table_pool_mutex);
     for (auto& kv : g_table_pools) {
+      TablePool& pool = kv.second;
       if (cudaSetDevice(kv.first) != cudaSuccess) continue;
-      table_pool_clear(kv.second);
-      if (kv.second.copies) cudaStreamDestroy(kv.second.copies);
+      table_pool_clear(pool);
+      if (pool.copies && pool.uploads == 0) {          // (else another thread is creating a plan: the next release frees it)
+        cudaStreamDestroy(pool.copies);
+        pool.copies = nullptr;
+      }
     }
-    g_table_pools.clear();
   }
   if (dev0 >= 0) cudaSetDevice(dev0);
   return DYSPEC_OK;

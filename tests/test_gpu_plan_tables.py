@@ -48,3 +48,38 @@ def test_plans_destroyed_with_their_kernels_still_queued():
     again.step()
     torch.cuda.synchronize()
     assert torch.equal(again.out, kept[0].out)
+
+
+def test_plans_created_while_the_cache_is_released():
+    """A thread that gives everything back must not take the upload stream from another one's plan creation."""
+    import threading
+    import torch
+    from paper_2410_11744_b200 import build
+    build.build()
+    from paper_2410_11744_b200 import binding as B, runner as R
+
+    b = R.DeviceBatch(wl.make_custom(3, 8, 2, 128, [700, 33], [wl.greedy_tree(np.random.default_rng(3), n, 6, 0.3) for n in (40, 8)]))
+    b.step()
+    torch.cuda.synchronize()
+    w, failed = b.w, []
+
+    def create():
+        try:
+            stream = torch.cuda.Stream()
+            with torch.cuda.stream(stream):
+                for _ in range(60):
+                    plan = B.Plan(w.n_q_heads, w.n_kv_heads, w.head_dim, w.prefix_len, w.n_nodes, w.kv_row_offset, b.kv_total_rows, b.W, 0.0)
+                    bits = torch.zeros_like(b.bits)
+                    B.dyspec_plan_build_tree_mask(plan, b.parents, bits)
+                    plan.destroy()
+                    stream.synchronize()
+                    assert torch.equal(bits, b.bits)
+        except Exception as e:                               # noqa: BLE001  (reported by the main thread)
+            failed.append(e)
+
+    threads = [threading.Thread(target=create) for _ in range(3)]
+    for t in threads:
+        t.start()
+    while any(t.is_alive() for t in threads):
+        B.dyspec_release_cache()
+    assert not failed, failed
