@@ -620,8 +620,10 @@ void schedule(dyspec_plan& pl) {
 // Device memory of the plans' tables.  A serving loop makes a plan for every step, and cudaMalloc, cudaFree (which waits
 // for the whole device) and a copy on the legacy stream (which waits for the step's earlier kernels) cost it about 0.9 ms
 // of host time that nothing overlapped: a step of 8 requests took 1.3 ms instead of 0.6.  So a destroyed plan's memory rests
-// here, and is used again only after a cudaFree -- one in kRestingMax destructions -- has waited for the device since:
-// whatever streams the plan ran on, nothing reads the memory any more.  Bounded to 2 kRestingMax buffers of at most
+// here, and is used again only after a cudaFree -- one in kRestingMax destructions -- has waited for its device since:
+// whatever streams the plan ran on, nothing reads the memory any more.  (Not cudaDeviceSynchronize, which waits for the same
+// but ends every stream capture under way in the process, in whatever mode; cudaFree ends none when the calling thread's
+// mode is relaxed.)  Bounded to 2 kRestingMax buffers of at most
 // kPooledBytes per device (larger ones are freed at once); dyspec_release_cache gives everything back.
 constexpr size_t kPooledBytes = size_t(256) << 10;
 constexpr size_t kRestingMax = 16;
@@ -634,6 +636,20 @@ struct TablePool {
 };
 std::map<int, TablePool> g_table_pools;
 std::mutex g_table_pool_mutex;
+
+// Frees memory of `device` after waiting for all work on it.
+cudaError_t free_after_wait(int device, void* ptr) {
+  int current = -1;
+  cudaError_t e = cudaGetDevice(&current);
+  if (e == cudaSuccess && current != device) e = cudaSetDevice(device);
+  if (e != cudaSuccess) return e;
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  e = cudaFree(ptr);
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  if (current != device) cudaSetDevice(current);
+  return e;
+}
 
 void table_pool_clear(TablePool& pool) {
   for (auto* list : {&pool.resting, &pool.idle}) {
@@ -679,17 +695,16 @@ void table_pool_uploaded(int device) {
 }
 
 void table_pool_give(int device, void* ptr, size_t bytes) {
-  if (bytes > kPooledBytes) { cudaFree(ptr); return; }
+  if (bytes > kPooledBytes) { free_after_wait(device, ptr); return; }
   std::lock_guard<std::mutex> lock(g_table_pool_mutex);
   TablePool& pool = g_table_pools[device];
   pool.resting.push_back({ptr, bytes});
   if (pool.resting.size() < kRestingMax) return;
-  const TableBuffer last = pool.resting.back();
+  if (free_after_wait(device, pool.resting.back().ptr) != cudaSuccess) return;      // all of it goes on resting
   pool.resting.pop_back();
-  if (cudaFree(last.ptr) != cudaSuccess) return;       // (synchronises the device; on an error the rest goes on resting)
   for (TableBuffer& b : pool.resting) {
     if (pool.idle.size() < kRestingMax) pool.idle.push_back(b);
-    else cudaFree(b.ptr);
+    else free_after_wait(device, b.ptr);
   }
   pool.resting.clear();
 }

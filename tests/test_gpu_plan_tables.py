@@ -83,3 +83,55 @@ def test_plans_created_while_the_cache_is_released():
     while any(t.is_alive() for t in threads):
         B.dyspec_release_cache()
     assert not failed, failed
+
+
+def _tiny_plans(B, count):
+    return [B.Plan(4, 4, 64, [10], [4], [0], 14, 4, 0.0) for _ in range(count)]
+
+
+def test_memory_is_reused_only_after_a_wait_for_the_device():
+    """Sixteen destructions behind a queued kernel, on a stream that waits for no other: by then the device has been waited for."""
+    import torch
+    from paper_2410_11744_b200 import build
+    build.build()
+    from paper_2410_11744_b200 import binding as B
+    B.dyspec_release_cache()
+    plans = _tiny_plans(B, 16)
+    stream, done = torch.cuda.Stream(), torch.cuda.Event()
+    x = torch.zeros(1 << 28, device="cuda:0")
+    torch.cuda.synchronize()
+    with torch.cuda.stream(stream):
+        for _ in range(100):                                 # some 30 ms
+            x.add_(1.0)
+        done.record()
+    assert not done.query()
+    for p in plans:
+        p.destroy()
+    assert done.query()
+    B.dyspec_release_cache()
+
+
+@pytest.mark.parametrize("mode", ["Global", "ThreadLocal", "Relaxed"])
+def test_destruction_leaves_a_capture_alone(mode):
+    """Plans are destroyed when Python collects them, in the middle of a stream capture too: the capture goes on, and what was
+    to be waited for is used again afterwards."""
+    import torch
+    rt = pytest.importorskip("cuda.bindings.runtime")
+    from paper_2410_11744_b200 import build
+    build.build()
+    from paper_2410_11744_b200 import binding as B
+    B.dyspec_release_cache()
+    plans, x = _tiny_plans(B, 40), torch.ones(1024, device="cuda:0")
+    stream = torch.cuda.Stream()
+    h = stream.cuda_stream
+    torch.cuda.synchronize()
+    assert rt.cudaStreamBeginCapture(h, getattr(rt.cudaStreamCaptureMode, "cudaStreamCaptureMode" + mode))[0] == 0
+    for p in plans:
+        p.destroy()
+    assert rt.cudaMemsetAsync(x.data_ptr(), 0, 4096, h)[0] == 0
+    err, graph = rt.cudaStreamEndCapture(h)
+    assert err == 0
+    rt.cudaGraphDestroy(graph)
+    for p in _tiny_plans(B, 20):
+        p.destroy()
+    B.dyspec_release_cache()
