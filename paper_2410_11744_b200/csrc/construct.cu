@@ -37,8 +37,11 @@
 //            draws go.
 //
 // Messages are single words that validate themselves (a draw's record in CTA 0, a load order or a ring
-// entry in a worker CTA; written through distributed shared memory), so hardly a hand-over needs
-// a fence and none a block barrier.  Every wait is bounded; when one runs out the request reports 0 nodes.
+// entry in a worker CTA; written through distributed shared memory), and no hand-over needs a block barrier.
+// What a message does not carry itself is ordered by a release and an acquire inside CTA 0: a node's event, behind which
+// lie its value and the token of its draw, from the planner to the helpers; the number of nodes opened, behind which
+// lie the rows, their entries and first records, from the opener to the orderer; and a hot CTA's buffer of
+// draws, in both directions.  Every wait is bounded; when one runs out the request reports 0 nodes.
 //
 // Measured on a B200 (vocabulary 32000, 256 language-model rows): one greedy tree of 768 nodes 5466 us with
 // the whole row re-read and re-summed by one block per node, 343 - 410 us now; eight threshold trees of 512
@@ -137,6 +140,14 @@ __device__ __forceinline__ void st_relaxed(const void* p, uint32_t v) {
 }
 __device__ __forceinline__ void st_relaxed64(const void* p, unsigned long long v) {
   asm volatile("st.relaxed.cluster.shared::cta.u64 [%0], %1;" ::"r"(smem_u32(p)), "l"(v) : "memory");
+}
+__device__ __forceinline__ uint32_t ld_acquire(const void* p) {
+  uint32_t v;
+  asm volatile("ld.acquire.cta.shared::cta.u32 %0, [%1];" : "=r"(v) : "r"(smem_u32(p)) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_release(const void* p, uint32_t v) {
+  asm volatile("st.release.cta.shared::cta.u32 [%0], %1;" ::"r"(smem_u32(p)), "r"(v) : "memory");
 }
 __device__ __forceinline__ unsigned long long ld_acquire64(const void* p) {
   unsigned long long v;
@@ -265,10 +276,10 @@ __device__ __forceinline__ Shared planner_view(uint8_t* sm, const TreeLayout& l)
   return s;
 }
 
-// A node for the helpers (one lane).
+// A node for the helpers (one lane, which has seen the draw).
 __device__ __forceinline__ void announce(const Shared& s, int k, int pos, uint32_t rec, double v) {
   s.note[k].v = v;                               // (read at the end only)
-  st_relaxed(&s.note[k].event, (uint32_t(pos) << 13) | rec);
+  st_release(&s.note[k].event, (uint32_t(pos) << 13) | rec);
 }
 
 // Algorithm 1's order.  Returns the number of nodes created, -1 when a wait ran out.
@@ -390,7 +401,7 @@ __device__ __forceinline__ bool next_event(const Shared& s, int m, int k, uint32
   bool over = false;
   const bool got = wait_until([&] {
     if (k <= m) {
-      ev = ld_relaxed(&s.note[k].event);
+      ev = ld_acquire(&s.note[k].event);
       if (ev != kEmpty) return true;
     }
     const uint32_t fin = ld_relaxed(s_final);
@@ -402,8 +413,8 @@ __device__ __forceinline__ bool next_event(const Shared& s, int m, int k, uint32
 
 // Helper 1: rows of new nodes.  `hot_addr` (both helpers): the hot CTAs' hand-over words, at the same offset in each.
 template <bool kGreedy>
-__device__ __forceinline__ void run_opener(const TreeArgs& a, const Shared& s, uint8_t* sm, uint32_t* s_tail, uint32_t hot_addr, const uint32_t* s_final,
-                                           const uint32_t* exit_flag, int req) {
+__device__ __forceinline__ void run_opener(const TreeArgs& a, const Shared& s, uint8_t* sm, uint32_t* s_tail, uint32_t hot_addr, uint32_t* s_opened,
+                                           const uint32_t* s_final, const uint32_t* exit_flag, int req) {
   const TreeLayout& l = a.lay;
   const int lane = threadIdx.x & 31;
   const double t = double(a.threshold);
@@ -449,7 +460,6 @@ __device__ __forceinline__ void run_opener(const TreeArgs& a, const Shared& s, u
           s.hash_val[at] = (uint32_t(e) << 16) | uint32_t(rec0);
           st_relaxed(&s.first[k], uint32_t(rec0));
         }
-        __threadfence_block();                   // helper 2 reads the entry once one of these draws has been used
         __syncwarp();
         send_orders(l, s_tail, st.ring, st.el_unit, uint32_t(rec0), want);
         break;
@@ -463,6 +473,7 @@ __device__ __forceinline__ void run_opener(const TreeArgs& a, const Shared& s, u
   if (lane == 0) s.note[0].row = row0;
   if (a.m > 0) open_row(0, row0);
   __syncwarp();
+  if (lane == 0) st_release(s_opened, 1u);       // nodes opened: what the whole warp wrote for them is in front of this
   uint32_t ev = kEmpty;
   for (int k = 1; next_event(s, a.m, k, ev, s_final, exit_flag); ++k) {
     const uint32_t rec = ev & 0x1FFFu, prow = s.note[ev >> 13].row;
@@ -475,20 +486,23 @@ __device__ __forceinline__ void run_opener(const TreeArgs& a, const Shared& s, u
     bool expand = k < a.m;
     if (!kGreedy) expand = __longlong_as_double((long long)ld_relaxed64(&s.open[k].v)) >= t;   // (written before the event)
     if (expand) open_row(k, row);
-    else __syncwarp();
+    __syncwarp();
+    if (lane == 0) st_release(s_opened, uint32_t(k) + 1u);
   }
 }
 
 // Helper 2: a used draw lets its row's stream run on.
 template <bool kGreedy>
 __device__ __forceinline__ void run_orderer(const TreeArgs& a, const Shared& s, uint8_t* sm, uint32_t* s_tail, uint32_t hot_addr,
-                                            const uint32_t* s_final, const uint32_t* exit_flag) {
+                                            const uint32_t* s_opened, const uint32_t* s_final, const uint32_t* exit_flag) {
   const TreeLayout& l = a.lay;
   const int lane = threadIdx.x & 31;
   int next_rec = l.open_records, n_hot = root_is_hot(l) ? 1 : 0;
   const uint32_t sm_addr = smem_u32(sm);
-  uint32_t ev = kEmpty;
+  uint32_t ev = kEmpty, opened = 0;
   for (int k = 1; next_event(s, a.m, k, ev, s_final, exit_flag); ++k) {
+    // the draw's row was opened with the position or before it; the opener may only just have named the record
+    if (opened <= (ev >> 13) && !wait_until([&] { opened = ld_acquire(s_opened); return opened > (ev >> 13); }, exit_flag)) return;
     const uint32_t owner = s.rec_owner[ev & 0x1FFFu];
     const int e = int(owner >> 16);
     EntryState st = s.entry[e];
@@ -829,7 +843,7 @@ __device__ __forceinline__ void run_hot(const TreeArgs& a, uint8_t* sm, const ui
       row = kEmpty;
     s_go[0] = row;
     s_go[1] = n_prev;
-    s_go[2] = 0u;                                              // draws sent
+    s_go[2] = 0u;                                              // draws taken out of the buffer
   }
   __syncthreads();
   const uint32_t row = s_go[0], n_prev = s_go[1];
@@ -860,13 +874,13 @@ __device__ __forceinline__ void run_hot(const TreeArgs& a, uint8_t* sm, const ui
       unsigned long long w = 0;
       if (!poll([&] { w = ld_acquire64(&from->word); return uint32_t(w >> 63) == made; }, exit_flag)) return;
       const double sum = from->sum, p = double(__uint_as_float(uint32_t(w)));
+      st_release(s_go + 2, i + 1);                             // read: the place may be written again
       const double r = sum > 0.0 ? p / sum : 0.0;
       uint32_t msg = kEmpty;
       if (!poll([&] { msg = ld_relaxed(order); return msg != kEmpty && (msg >> 31) == asked; }, exit_flag)) return;
       const uint32_t rec = msg & 0x1FFFu;
       st_remote64(rec_base + rec * 16, (unsigned long long)__double_as_longlong(r));
       st_remote(rec_base + rec * 16 + 8, uint32_t(w >> 32) & 0x7FFFu);
-      st_relaxed(s_go + 2, i + 1);
     }
     return;
   }
@@ -876,12 +890,12 @@ __device__ __forceinline__ void run_hot(const TreeArgs& a, uint8_t* sm, const ui
   Pair upto = scan(s_sub[(lane * kSubs + kSubs - 1) * 32 + 31], lane);
   Pair total{__shfl_sync(0xffffffffu, upto.hi, 31), __shfl_sync(0xffffffffu, upto.lo, 31)};
   double built = total.hi;
-  uint32_t sent = 0;
+  uint32_t taken = 0;
   float u_next = s_num[0];
   for (uint32_t i = 0; i < uint32_t(a.m); ++i) {               // ahead of the orders, as far as the buffer goes
     const uint32_t at = i & (kHotAhead - 1), phase = (i / kHotAhead) & 1u;
-    if (i - sent >= uint32_t(kHotAhead) &&
-        !poll([&] { sent = ld_relaxed(s_go + 2); return i - sent < uint32_t(kHotAhead); }, exit_flag))
+    if (i - taken >= uint32_t(kHotAhead) &&
+        !poll([&] { taken = ld_acquire(s_go + 2); return i - taken < uint32_t(kHotAhead); }, exit_flag))
       return;
     const uint32_t stop = ld_relaxed(exit_flag);
     const float u = u_next;
@@ -968,7 +982,7 @@ template <bool kGreedy, int K>
 __global__ void __launch_bounds__(kTreeThreads, 1)
 build_tree_kernel(const __grid_constant__ TreeArgs a) {
   extern __shared__ __align__(16) uint8_t csm[];
-  __shared__ uint32_t s_exit, s_never, s_final, s_log_n;       // (planner and helper do not listen to s_exit)
+  __shared__ uint32_t s_exit, s_never, s_final, s_opened, s_log_n;       // (planner and helper do not listen to s_exit)
   __shared__ uint32_t s_tail[8 * kDrawWarps + kMaxHot];
   __shared__ uint32_t s_hot[2 + 32], s_go[3];
   __shared__ uint32_t s_mask[kDrawWarps][32];
@@ -982,7 +996,7 @@ build_tree_kernel(const __grid_constant__ TreeArgs a) {
   const bool planner_cta = rank == 0, worker_cta = int(rank) >= l.first_worker, hot_cta = !planner_cta && !worker_cta;
 
   // ---- every word that another warp or CTA will write starts as "not there yet"
-  if (tid == 0) { s_exit = 0u; s_never = 0u; s_final = kEmpty; s_log_n = 0u; }
+  if (tid == 0) { s_exit = 0u; s_never = 0u; s_final = kEmpty; s_opened = 0u; s_log_n = 0u; }
   if (tid < kMaxStages) {
     mbar_init(smem_u32(s_full + tid), 1);
     mbar_init(smem_u32(s_empty + tid), kLoadWarps);
@@ -1030,9 +1044,9 @@ build_tree_kernel(const __grid_constant__ TreeArgs a) {
       for (uint32_t c = uint32_t(lane); c < n_cta; c += 32) st_remote(map_to_cta(smem_u32(&s_exit), c), 1u);
     }
   } else if (warp == 1) {
-    if (planner_cta) run_opener<kGreedy>(a, s, csm, s_tail, smem_u32(s_hot), &s_final, &s_never, req);
+    if (planner_cta) run_opener<kGreedy>(a, s, csm, s_tail, smem_u32(s_hot), &s_opened, &s_final, &s_never, req);
   } else if (warp == 2) {
-    if (planner_cta) run_orderer<kGreedy>(a, s, csm, s_tail, smem_u32(s_hot), &s_final, &s_never);
+    if (planner_cta) run_orderer<kGreedy>(a, s, csm, s_tail, smem_u32(s_hot), &s_opened, &s_final, &s_never);
   } else if (worker_cta) {
     if (warp < kRoles + kDrawWarps) run_drawer<K>(a, csm, warp - kRoles, int(rank) - l.first_worker, s_mask, &s_log_n, &s_exit);
     else if (warp == kRoles + kDrawWarps) run_fetcher<K>(a, csm, int(rank) - l.first_worker, s_full, s_empty, &s_never, &s_exit);
