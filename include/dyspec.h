@@ -370,7 +370,8 @@ int dyspec_verify_tree(const int32_t* parents, const int32_t* tokens, const floa
  *   parents, tokens, rows  dev int32 [n_req][S];  values, child_values  dev float [n_req][S]
  *                 values[k] = the estimated acceptance rate node k was created with, child_values[k] =
  *                 that of the first sampling under it;  n_nodes dev int32 [n_req] = nodes incl. the root
- *                 (0 if a bounded wait inside the kernel ran out, which ordinary operation never sees)
+ *                 (0 if a bounded wait inside the kernel ran out, which ordinary operation never sees: node 0 alone is
+ *                 written then)
  * m, max_nodes <= DYSPEC_MAX_NODES - 1.  Values are fp32; as for dyspec_verify_tree, a choice between
  * numbers closer than rounding may fall differently from another implementation's.
  */
@@ -381,6 +382,18 @@ int dyspec_build_tree_threshold(const float* draft_table, int n_rows, int vocab,
                                 const int32_t* root_row, int n_req, float threshold, int max_nodes, int32_t* parents,
                                 int32_t* tokens, float* values, float* child_values, int32_t* rows, int32_t* n_nodes,
                                 dyspec_stream_t stream);
+
+/* The same two with a report of such a wait and its bound in the caller's hand.
+ *   wait_limit_ns  how long one wait may take, 1 .. 1000000000 ns; 0 = 1000000000 (what the calls above use)
+ *   status         dev int32 [1] or NULL: DYSPEC_ERR_TIMEOUT when a wait of any request ran out */
+int dyspec_build_tree_greedy_bounded(const float* draft_table, int n_rows, int vocab, const float* uniforms, int n_uniforms,
+                                     const int32_t* root_row, int n_req, int m, int32_t* parents, int32_t* tokens,
+                                     float* values, float* child_values, int32_t* rows, int32_t* n_nodes, int wait_limit_ns,
+                                     int32_t* status, dyspec_stream_t stream);
+int dyspec_build_tree_threshold_bounded(const float* draft_table, int n_rows, int vocab, const float* uniforms, int n_uniforms,
+                                        const int32_t* root_row, int n_req, float threshold, int max_nodes, int32_t* parents,
+                                        int32_t* tokens, float* values, float* child_values, int32_t* rows, int32_t* n_nodes,
+                                        int wait_limit_ns, int32_t* status, dyspec_stream_t stream);
 
 /*
  * (7) Keeping the accepted path in the KV cache (after dyspec_verify_tree; the paper only says that the

@@ -51,6 +51,8 @@ SIGNATURES = {
     "dyspec_verify_tree": (_i32, [_vp, _vp, _vp, _vp, _vp, _vp, _vp, _i32, _i32, _i32, _i32, _vp, _vp, _vp, _i32, _vp, _vp]),
     "dyspec_build_tree_greedy": (_i32, [_vp, _i32, _i32, _vp, _i32, _vp, _i32, _i32, _vp, _vp, _vp, _vp, _vp, _vp, _vp]),
     "dyspec_build_tree_threshold": (_i32, [_vp, _i32, _i32, _vp, _i32, _vp, _i32, _f32, _i32, _vp, _vp, _vp, _vp, _vp, _vp, _vp]),
+    "dyspec_build_tree_greedy_bounded": (_i32, [_vp, _i32, _i32, _vp, _i32, _vp, _i32, _i32, _vp, _vp, _vp, _vp, _vp, _vp, _i32, _vp, _vp]),
+    "dyspec_build_tree_threshold_bounded": (_i32, [_vp, _i32, _i32, _vp, _i32, _vp, _i32, _f32, _i32, _vp, _vp, _vp, _vp, _vp, _vp, _i32, _vp, _vp]),
     "dyspec_compact_kv": (_i32, [_vp, _vp, _vp, _vp, _vp, _vp, _i32, _i32, _i32, _i32, _i32, _vp, _vp]),
     "dyspec_plan_create_paged": (_i32, [_c.POINTER(_vp), _i32, _i32, _i32, _i32, _vp, _vp, _vp, _i64, _i32, _i32, _f32]),
     "dyspec_tree_attention_paged": (_i32, [_vp, _vp, _vp, _vp, _vp, _i32, _vp, _vp, _vp, _vp, _sz, _vp, _vp]),
@@ -323,6 +325,27 @@ def dyspec_build_tree_threshold(draft_table, n_rows: int, vocab: int, uniforms, 
                                            n_req, float(threshold), max_nodes, _ptr(parents), _ptr(tokens), _ptr(values),
                                            _ptr(child_values), _ptr(rows), _ptr(n_nodes), _stream(stream)),
            "dyspec_build_tree_threshold")
+
+
+def dyspec_build_tree_greedy_bounded(draft_table, n_rows: int, vocab: int, uniforms, n_uniforms: int, root_row, n_req: int,
+                                     m: int, parents, tokens, values, child_values, rows, n_nodes, wait_limit_ns: int = 0,
+                                     status=None, stream=None) -> None:
+    """dyspec_build_tree_greedy with a bound on its waits (0: one second) and a status word for one that ran out."""
+    _check(lib.dyspec_build_tree_greedy_bounded(_ptr(draft_table), n_rows, vocab, _ptr(uniforms), n_uniforms, _ptr(root_row),
+                                                n_req, m, _ptr(parents), _ptr(tokens), _ptr(values), _ptr(child_values),
+                                                _ptr(rows), _ptr(n_nodes), wait_limit_ns, _ptr(status), _stream(stream)),
+           "dyspec_build_tree_greedy_bounded")
+
+
+def dyspec_build_tree_threshold_bounded(draft_table, n_rows: int, vocab: int, uniforms, n_uniforms: int, root_row, n_req: int,
+                                        threshold: float, max_nodes: int, parents, tokens, values, child_values, rows,
+                                        n_nodes, wait_limit_ns: int = 0, status=None, stream=None) -> None:
+    """dyspec_build_tree_threshold with a bound on its waits (0: one second) and a status word for one that ran out."""
+    _check(lib.dyspec_build_tree_threshold_bounded(_ptr(draft_table), n_rows, vocab, _ptr(uniforms), n_uniforms,
+                                                   _ptr(root_row), n_req, float(threshold), max_nodes, _ptr(parents),
+                                                   _ptr(tokens), _ptr(values), _ptr(child_values), _ptr(rows), _ptr(n_nodes),
+                                                   wait_limit_ns, _ptr(status), _stream(stream)),
+           "dyspec_build_tree_threshold_bounded")
 
 
 def dyspec_compact_kv(k_cache, v_cache, kv_row_offset, prefix_len, accepted_nodes, n_accepted, n_req: int, max_out: int,

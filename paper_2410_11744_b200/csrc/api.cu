@@ -33,11 +33,11 @@ cudaError_t launch_verify_tree(const int32_t* parents, const int32_t* tokens, co
 cudaError_t launch_build_tree_greedy(const float* draft_table, int n_rows, int vocab, const float* uniforms, int n_uniforms,
                                      const int32_t* root_row, int n_req, int m, int32_t* parents, int32_t* tokens,
                                      float* values, float* child_values, int32_t* rows, int32_t* n_nodes,
-                                     cudaStream_t stream);
+                                     uint32_t wait_limit_ns, int32_t* status, cudaStream_t stream);
 cudaError_t launch_build_tree_threshold(const float* draft_table, int n_rows, int vocab, const float* uniforms,
                                         int n_uniforms, const int32_t* root_row, int n_req, float threshold, int max_nodes,
                                         int32_t* parents, int32_t* tokens, float* values, float* child_values, int32_t* rows,
-                                        int32_t* n_nodes, cudaStream_t stream);
+                                        int32_t* n_nodes, uint32_t wait_limit_ns, int32_t* status, cudaStream_t stream);
 cudaError_t launch_compact_kv_paged(void* k_cache, void* v_cache, const int64_t* tree_row_offset, const int32_t* page_table,
                                     int pages_per_req, int page_shift, const int32_t* prefix_len,
                                     const int32_t* accepted_nodes, const int32_t* n_accepted, int n_req, int max_out,
@@ -905,14 +905,24 @@ static int check_tree_build_args(const float* draft_table, int n_rows, int vocab
   return DYSPEC_OK;
 }
 
+static uint32_t tree_wait_limit(int wait_limit_ns) { return wait_limit_ns > 0 ? uint32_t(wait_limit_ns) : uint32_t(kWaitLimitNs); }
 int dyspec_build_tree_greedy(const float* draft_table, int n_rows, int vocab, const float* uniforms, int n_uniforms,
                              const int32_t* root_row, int n_req, int m, int32_t* parents, int32_t* tokens, float* values,
                              float* child_values, int32_t* rows, int32_t* n_nodes, dyspec_stream_t stream) {
+  return dyspec_build_tree_greedy_bounded(draft_table, n_rows, vocab, uniforms, n_uniforms, root_row, n_req, m, parents, tokens,
+                                          values, child_values, rows, n_nodes, 0, nullptr, stream);
+}
+int dyspec_build_tree_greedy_bounded(const float* draft_table, int n_rows, int vocab, const float* uniforms, int n_uniforms,
+                                     const int32_t* root_row, int n_req, int m, int32_t* parents, int32_t* tokens,
+                                     float* values, float* child_values, int32_t* rows, int32_t* n_nodes, int wait_limit_ns,
+                                     int32_t* status, dyspec_stream_t stream) {
   const int rc = check_tree_build_args(draft_table, n_rows, vocab, uniforms, n_uniforms, root_row, n_req, m, parents, tokens,
                                        values, child_values, rows, n_nodes);
   if (rc != DYSPEC_OK || n_req == 0) return rc;
+  if (wait_limit_ns < 0 || wait_limit_ns > int(kWaitLimitNs) || !aligned(status, 4)) return DYSPEC_ERR_INVALID_ARG;
   cudaError_t e = launch_build_tree_greedy(draft_table, n_rows, vocab, uniforms, n_uniforms, root_row, n_req, m, parents,
-                                           tokens, values, child_values, rows, n_nodes, reinterpret_cast<cudaStream_t>(stream));
+                                           tokens, values, child_values, rows, n_nodes, tree_wait_limit(wait_limit_ns), status,
+                                           reinterpret_cast<cudaStream_t>(stream));
   return e == cudaSuccess ? DYSPEC_OK : cuda_failed(e, "greedy tree launch");
 }
 
@@ -920,13 +930,21 @@ int dyspec_build_tree_threshold(const float* draft_table, int n_rows, int vocab,
                                 const int32_t* root_row, int n_req, float threshold, int max_nodes, int32_t* parents,
                                 int32_t* tokens, float* values, float* child_values, int32_t* rows, int32_t* n_nodes,
                                 dyspec_stream_t stream) {
+  return dyspec_build_tree_threshold_bounded(draft_table, n_rows, vocab, uniforms, n_uniforms, root_row, n_req, threshold,
+                                             max_nodes, parents, tokens, values, child_values, rows, n_nodes, 0, nullptr, stream);
+}
+int dyspec_build_tree_threshold_bounded(const float* draft_table, int n_rows, int vocab, const float* uniforms, int n_uniforms,
+                                        const int32_t* root_row, int n_req, float threshold, int max_nodes, int32_t* parents,
+                                        int32_t* tokens, float* values, float* child_values, int32_t* rows, int32_t* n_nodes,
+                                        int wait_limit_ns, int32_t* status, dyspec_stream_t stream) {
   const int rc = check_tree_build_args(draft_table, n_rows, vocab, uniforms, n_uniforms, root_row, n_req, max_nodes, parents,
                                        tokens, values, child_values, rows, n_nodes);
   if (rc != DYSPEC_OK || n_req == 0) return rc;
+  if (wait_limit_ns < 0 || wait_limit_ns > int(kWaitLimitNs) || !aligned(status, 4)) return DYSPEC_ERR_INVALID_ARG;
   if (!(threshold > 0.f)) return DYSPEC_ERR_INVALID_ARG;
   cudaError_t e = launch_build_tree_threshold(draft_table, n_rows, vocab, uniforms, n_uniforms, root_row, n_req, threshold,
                                               max_nodes, parents, tokens, values, child_values, rows, n_nodes,
-                                              reinterpret_cast<cudaStream_t>(stream));
+                                              tree_wait_limit(wait_limit_ns), status, reinterpret_cast<cudaStream_t>(stream));
   return e == cudaSuccess ? DYSPEC_OK : cuda_failed(e, "threshold tree launch");
 }
 

@@ -41,7 +41,7 @@
 // What a message does not carry itself is ordered by a release and an acquire inside CTA 0: a node's event, behind which
 // lie its value and the token of its draw, from the planner to the helpers; the number of nodes opened, behind which
 // lie the rows, their entries and first records, from the opener to the orderer; and a hot CTA's buffer of
-// draws, in both directions.  Every wait is bounded; when one runs out the request reports 0 nodes.
+// draws, in both directions.  Every wait is bounded; when one runs out the request reports 0 nodes and DYSPEC_ERR_TIMEOUT.
 //
 // Measured on a B200 (vocabulary 32000, 256 language-model rows): one greedy tree of 768 nodes 5466 us with
 // the whole row re-read and re-summed by one block per node, 343 - 410 us now; eight threshold trees of 512
@@ -74,6 +74,7 @@ constexpr int kSub = 8, kChunk = 1024, kChunks = 32;          // hot tables: tok
 constexpr int kSubs = kChunk / kSub / 32;                     // sub-blocks of a chunk per lane
 constexpr int kMaxAhead = 8;           // draws of a row that may be ordered before they are used
 constexpr uint32_t kEmpty = 0xFFFFFFFFu;
+constexpr uint32_t kPatientNs = 1000000;     // waits with a limit below this look at the clock at every probe
 constexpr uint32_t kFollow = 0x80000000u;   // slot: the record after this one, not linked yet when the slot was written
 constexpr int kMaxRecords = 8192;      // 13 bits of a ring entry
 
@@ -115,6 +116,8 @@ struct TreeArgs {
   int n_rows, vocab, n_uniforms, m;
   uint32_t rows_inverse;               // floor(2^32 / n_rows), at most 2^32 - 1
   float threshold;                     // threshold algorithm only
+  uint32_t wait_limit_ns;              // of the planner's waits, at most kWaitLimitNs
+  int32_t* status;                     // may be null
   int32_t* parents;
   int32_t* tokens;
   float* values;
@@ -166,16 +169,17 @@ __device__ __forceinline__ void st_remote64(uint32_t cluster_addr, unsigned long
 
 // Polls `ready` (warp-uniform) until it holds; false once the limit has passed.  For the planner and the helpers, whose flag
 // never rises; the others use poll(), which ends with the tree.
-template <typename F>
-__device__ __forceinline__ bool wait_until(F ready, const uint32_t* exit_flag) {
+// kPatient: hundreds of probes before the clock is looked at, and seldom then; else (a limit below a millisecond) at every probe.
+template <bool kPatient = true, typename F>
+__device__ __forceinline__ bool wait_until(F ready, const uint32_t* exit_flag, uint32_t limit_ns = uint32_t(kWaitLimitNs)) {
 #pragma unroll 1
-  for (int i = 0; i < 512; ++i)
+  for (int i = 0; i < (kPatient ? 512 : 1); ++i)
     if (ready()) return true;
   const uint64_t t0 = global_timer_ns();
   for (uint32_t spins = 1;; ++spins) {
     if (ready()) return true;
     if (ld_relaxed(exit_flag)) return false;
-    if ((spins & 255u) == 0 && global_timer_ns() - t0 > kWaitLimitNs) return false;
+    if ((!kPatient || (spins & 255u) == 0) && global_timer_ns() - t0 >= limit_ns) return false;
   }
 }
 
@@ -224,19 +228,20 @@ __device__ __forceinline__ int warp_best(double v, uint32_t seq, double& best) {
 struct Draw { double r; uint32_t next; };
 
 // The record that `slot` stands for and its content, when it has been drawn.
-__device__ __forceinline__ bool wait_draw(const DrawRecord* recs, uint32_t& slot, Draw& d, const uint32_t* exit_flag) {
+template <bool kPatient>
+__device__ __forceinline__ bool wait_draw(const DrawRecord* recs, uint32_t& slot, Draw& d, const uint32_t* exit_flag, uint32_t limit_ns) {
   if (slot & kFollow) {
     const uint32_t prev = slot & ~kFollow;
     uint32_t nx = kEmpty;
-    if (!wait_until([&] { nx = ld_relaxed(&recs[prev].next); return nx != kEmpty; }, exit_flag)) return false;
+    if (!wait_until<kPatient>([&] { nx = ld_relaxed(&recs[prev].next); return nx != kEmpty; }, exit_flag, limit_ns)) return false;
     slot = nx;
   }
   const uint32_t at = smem_u32(recs + slot);
   unsigned long long rb = 0, tn = 0;                           // two words that are each read at once: r; token and next record
-  if (!wait_until([&] {
+  if (!wait_until<kPatient>([&] {
         asm volatile("ld.volatile.shared.v2.u64 {%0, %1}, [%2];" : "=l"(rb), "=l"(tn) : "r"(at) : "memory");
         return rb != ~0ull && uint32_t(tn) != kEmpty;
-      }, exit_flag))
+      }, exit_flag, limit_ns))
     return false;
   d.r = __longlong_as_double((long long)rb);
   d.next = uint32_t(tn >> 32);
@@ -284,6 +289,7 @@ __device__ __forceinline__ void announce(const Shared& s, int k, int pos, uint32
 
 // Algorithm 1's order.  Returns the number of nodes created, -1 when a wait ran out.
 // One warp, so every instruction of a step counts about four cycles.
+template <bool kPatient>
 __device__ int plan_greedy(const TreeArgs& a, const Shared& s, const uint32_t* exit_flag) {
   const int lane = threadIdx.x & 31, per_lane = a.lay.nodes_pad >> 5;
   double c_v = -1.0, rest_v = -1.0;              // the best open position p with p % 32 == lane; the best of all: both without the current one
@@ -300,9 +306,9 @@ __device__ int plan_greedy(const TreeArgs& a, const Shared& s, const uint32_t* e
   };
   int n = 0;
   while (n < a.m) {
-    if (slot == kEmpty && !wait_until([&] { slot = ld_relaxed(&s.first[pos]); return slot != kEmpty; }, exit_flag)) return -1;
+    if (slot == kEmpty && !wait_until<kPatient>([&] { slot = ld_relaxed(&s.first[pos]); return slot != kEmpty; }, exit_flag, a.wait_limit_ns)) return -1;
     Draw d;
-    if (!wait_draw(s.rec, slot, d, exit_flag)) return -1;
+    if (!wait_draw<kPatient>(s.rec, slot, d, exit_flag, a.wait_limit_ns)) return -1;
     const int k = ++n;
     if (lane == 0) announce(s, k, pos, slot, v);
     const double left = 1.0 - d.r;
@@ -355,6 +361,7 @@ __device__ int plan_greedy(const TreeArgs& a, const Shared& s, const uint32_t* e
 }
 
 // Algorithm 2's order: positions in index order (which is layer order) draw while v >= t.
+template <bool kPatient>
 __device__ int plan_threshold(const TreeArgs& a, const Shared& s, const uint32_t* exit_flag) {
   const int lane = threadIdx.x & 31;
   const double t = double(a.threshold);
@@ -365,10 +372,10 @@ __device__ int plan_threshold(const TreeArgs& a, const Shared& s, const uint32_t
     double v = s.open[pos].v;
     if (!(v >= t)) continue;
     uint32_t slot = kEmpty;
-    if (!wait_until([&] { slot = ld_relaxed(&s.first[pos]); return slot != kEmpty; }, exit_flag)) return -1;
+    if (!wait_until<kPatient>([&] { slot = ld_relaxed(&s.first[pos]); return slot != kEmpty; }, exit_flag, a.wait_limit_ns)) return -1;
     while (v >= t && n < a.m) {
       Draw d;
-      if (!wait_draw(s.rec, slot, d, exit_flag)) return -1;
+      if (!wait_draw<kPatient>(s.rec, slot, d, exit_flag, a.wait_limit_ns)) return -1;
       const int k = ++n;
       if (lane == 0) {
         st_relaxed64(&s.open[k].v, (unsigned long long)__double_as_longlong(v * d.r));
@@ -1035,10 +1042,13 @@ build_tree_kernel(const __grid_constant__ TreeArgs a) {
     run_hot(a, csm, s_hot, s_go, &s_exit);
   } else if (warp == 0) {
     if (planner_cta) {
-      const int n = kGreedy ? plan_greedy(a, s, &s_never) : plan_threshold(a, s, &s_never);
+      const bool patient = a.wait_limit_ns >= kPatientNs;
+      const int n = kGreedy ? (patient ? plan_greedy<true>(a, s, &s_never) : plan_greedy<false>(a, s, &s_never))
+                            : (patient ? plan_threshold<true>(a, s, &s_never) : plan_threshold<false>(a, s, &s_never));
       __syncwarp();
       if (lane == 0) {
         a.n_nodes[req] = n + 1;                                // 0: a wait ran out
+        if (n < 0 && a.status) atomicCAS(a.status, 0, DYSPEC_ERR_TIMEOUT);
         st_relaxed(&s_final, n < 0 ? 0u : uint32_t(n));
       }
       for (uint32_t c = uint32_t(lane); c < n_cta; c += 32) st_remote(map_to_cta(smem_u32(&s_exit), c), 1u);
@@ -1182,18 +1192,18 @@ cudaError_t launch_tree(TreeArgs a, int n_req, cudaStream_t stream) {
 cudaError_t launch_build_tree_greedy(const float* draft_table, int n_rows, int vocab, const float* uniforms, int n_uniforms,
                                      const int32_t* root_row, int n_req, int m, int32_t* parents, int32_t* tokens,
                                      float* values, float* child_values, int32_t* rows, int32_t* n_nodes,
-                                     cudaStream_t stream) {
+                                     uint32_t wait_limit_ns, int32_t* status, cudaStream_t stream) {
   if (n_req <= 0) return cudaSuccess;
-  return launch_tree<true>(TreeArgs{draft_table, uniforms, root_row, n_rows, vocab, n_uniforms, m, 0u, 0.f, parents, tokens, values,
+  return launch_tree<true>(TreeArgs{draft_table, uniforms, root_row, n_rows, vocab, n_uniforms, m, 0u, 0.f, wait_limit_ns, status, parents, tokens, values,
                                     child_values, rows, n_nodes, TreeLayout{}}, n_req, stream);
 }
 
 cudaError_t launch_build_tree_threshold(const float* draft_table, int n_rows, int vocab, const float* uniforms,
                                         int n_uniforms, const int32_t* root_row, int n_req, float threshold, int max_nodes,
                                         int32_t* parents, int32_t* tokens, float* values, float* child_values, int32_t* rows,
-                                        int32_t* n_nodes, cudaStream_t stream) {
+                                        int32_t* n_nodes, uint32_t wait_limit_ns, int32_t* status, cudaStream_t stream) {
   if (n_req <= 0) return cudaSuccess;
-  return launch_tree<false>(TreeArgs{draft_table, uniforms, root_row, n_rows, vocab, n_uniforms, max_nodes, 0u, threshold, parents,
+  return launch_tree<false>(TreeArgs{draft_table, uniforms, root_row, n_rows, vocab, n_uniforms, max_nodes, 0u, threshold, wait_limit_ns, status, parents,
                                      tokens, values, child_values, rows, n_nodes, TreeLayout{}}, n_req, stream);
 }
 

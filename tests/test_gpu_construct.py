@@ -188,3 +188,36 @@ def test_constructed_tree_feeds_the_mask_builder(B):
     ref_bits, ref_depths = orc.build_tree_mask(parents, W)
     assert np.array_equal(bits.cpu().numpy().view(np.uint32), ref_bits)
     assert np.array_equal(depths.cpu().numpy(), ref_depths)
+
+
+@pytest.mark.parametrize("greedy", [True, False])
+@pytest.mark.parametrize("n_req", [1, 40, 150])
+def test_a_wait_that_runs_out_is_reported(B, greedy, n_req):
+    """With a bound of a nanosecond the wait for the first draw, whose row has yet to come from memory, cannot succeed: every request
+    reports 0 nodes and the status word says why; the next call, with the usual bound, is right."""
+    import torch
+    vocab, n_rows, m = 32000, 16, 24
+    rows, uni = wl.make_draft_table(11, n_rows, vocab, 3.0)
+    roots = [r % n_rows for r in range(n_req)]
+    dev = "cuda:0"
+    t = lambda a: torch.from_numpy(np.ascontiguousarray(a)).to(dev)
+    ints = [torch.full((n_req, m + 1), -9, dtype=torch.int32, device=dev) for _ in range(3)]
+    vals = [torch.zeros((n_req, m + 1), device=dev) for _ in range(2)]
+    n_nodes, status = torch.full((n_req,), -9, dtype=torch.int32, device=dev), torch.zeros(1, dtype=torch.int32, device=dev)
+    head = (t(rows), n_rows, vocab, t(uni), len(uni), t(np.asarray(roots, np.int32)), n_req)
+    tail = (ints[0], ints[1], vals[0], vals[1], ints[2], n_nodes)
+    call = (lambda **k: B.dyspec_build_tree_greedy_bounded(*head, m, *tail, **k)) if greedy else \
+           (lambda **k: B.dyspec_build_tree_threshold_bounded(*head, 1e-3, m, *tail, **k))
+    call(wait_limit_ns=1, status=status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == -6 and int(n_nodes.abs().max()) == 0
+    status.zero_()
+    call(status=status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    got = [x.cpu().numpy() for x in (ints[0], ints[1], vals[0], vals[1], ints[2], n_nodes)]
+    for r in {0, n_req - 1}:
+        ref = orc.build_tree_greedy(rows, uni, m, root_row=roots[r]) if greedy else orc.build_tree_threshold(rows, uni, 1e-3, m, root_row=roots[r])
+        compare(got, r, ref)
+    with pytest.raises(B.DyspecError):
+        call(wait_limit_ns=-1)
