@@ -142,6 +142,32 @@ struct DynSmemGrant {
   }
 };
 
+// How many clusters of C CTAs of a kernel that takes a whole SM per CTA the current device holds at once: the SMs of a
+// cluster come from one GPC, so fewer than SMs / C.  One of these per kernel asks once per device and size.
+struct ClusterRoom {
+  std::atomic<int> known[DynSmemGrant::kDevices][4];   // for C = 1, 2, 4, 8; 0: not asked yet, else the answer + 1
+  template <typename Kernel>
+  int ask(Kernel kernel, int threads, int C) {
+    int dev = -1, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) { cudaGetLastError(); return kDefaultSMs / C; }
+    std::atomic<int>* at = dev < DynSmemGrant::kDevices ? &known[dev][C == 8 ? 3 : C == 4 ? 2 : C == 2 ? 1 : 0] : nullptr;
+    if (const int have = at ? at->load() : 0; have > 0) return have - 1;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = unsigned(C);
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(unsigned(C));
+    cfg.blockDim = dim3(unsigned(threads));
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) { cudaGetLastError(); return kDefaultSMs / C; }
+    if (at) at->store(n + 1);
+    return n;
+  }
+};
+
 // Key tiles of a (request, query tile) group, host and device: the tiles in front of the first one that
 // needs the mask, and how far the tree's column 0 sits inside that one (0 unless the tree rows are
 // part of the paged sequence).

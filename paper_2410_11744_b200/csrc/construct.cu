@@ -48,9 +48,20 @@
 // nodes 2518 -> 300 us.  What bounds it: single warps' chains of dependent instructions, about four cycles
 // each -- the hot stream's 900 cycles a draw (chunk 240, sub-block 165, token 260, tables 210), the planner's
 // 500 a step, about 150 us for the first 127 nodes, whose draws are still cold (2600 cycles a draw in a stream).
+//
+// Batches of trees with too many rows for this split go to the one-CTA form (construct_rows.cu); launch_tree says when.
 #include "vocab_ops.cuh"
 
 namespace dyspec {
+
+cudaError_t launch_build_tree_greedy_rows(const float* draft_table, int n_rows, int vocab, const float* uniforms, int n_uniforms,
+                                          const int32_t* root_row, int n_req, int m, int32_t* parents, int32_t* tokens,
+                                          float* values, float* child_values, int32_t* rows, int32_t* n_nodes,
+                                          cudaStream_t stream);
+cudaError_t launch_build_tree_threshold_rows(const float* draft_table, int n_rows, int vocab, const float* uniforms,
+                                             int n_uniforms, const int32_t* root_row, int n_req, float threshold, int max_nodes,
+                                             int32_t* parents, int32_t* tokens, float* values, float* child_values,
+                                             int32_t* rows, int32_t* n_nodes, cudaStream_t stream);
 
 namespace {
 
@@ -72,6 +83,7 @@ constexpr int kHotAhead = 256;         // draws a hot CTA may have ready before 
 constexpr int kMaxHot = 3;
 constexpr int kSub = 8, kChunk = 1024, kChunks = 32;          // hot tables: tokens per sub-block, per chunk; chunks
 constexpr int kSubs = kChunk / kSub / 32;                     // sub-blocks of a chunk per lane
+constexpr int kShortTree = 96;         // nodes x CTAs of a cluster up to which no second wave of clusters pays
 constexpr int kMaxAhead = 8;           // draws of a row that may be ordered before they are used
 constexpr uint32_t kEmpty = 0xFFFFFFFFu;
 constexpr uint32_t kPatientNs = 1000000;     // waits with a limit below this look at the clock at every probe
@@ -1158,32 +1170,56 @@ cudaError_t launch_tree(const TreeArgs& a, int n_req, int C, cudaStream_t stream
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
+// The general form, one CTA a request (construct_rows.cu).
+template <bool kGreedy>
+cudaError_t launch_rows(const TreeArgs& a, int n_req, cudaStream_t stream) {
+  return kGreedy ? launch_build_tree_greedy_rows(a.table, a.n_rows, a.vocab, a.uniforms, a.n_uniforms, a.root_row, n_req, a.m,
+                                                 a.parents, a.tokens, a.values, a.child_values, a.rows, a.n_nodes, stream)
+                 : launch_build_tree_threshold_rows(a.table, a.n_rows, a.vocab, a.uniforms, a.n_uniforms, a.root_row, n_req,
+                                                    a.threshold, a.m, a.parents, a.tokens, a.values, a.child_values, a.rows,
+                                                    a.n_nodes, stream);
+}
+
 template <bool kGreedy>
 cudaError_t launch_tree(TreeArgs a, int n_req, cudaStream_t stream) {
-  // The largest cluster for which the SMs suffice, n_req C <= 148; where none does, the smallest that holds the tree.  (15 clusters of
-  // 8 run at once, an SM's neighbours being what they are, but 16 - 18 requests in two waves of them take 181 us for
-  // 127 nodes where clusters of 4 take 204; 35 requests take 243 us with clusters of 4 and 409 with 2.)
-  const int leaf_bytes = 512 * (a.vocab <= kLeaves * 128 ? 1 : a.vocab <= kLeaves * 256 ? 2 : 4);
-  int C = 8;
-  while (C > 1 && int64_t(n_req) * C > kDefaultSMs) C /= 2;
+  const int K = a.vocab <= kLeaves * 128 ? 1 : a.vocab <= kLeaves * 256 ? 2 : 4, leaf_bytes = 512 * K;
   auto fits = [&](int c) {
     for (int hot = c == 8 ? kMaxHot : c == 4 ? 1 : 0; hot >= 0; --hot)
       if ((hot == 0 || a.m > kHotLeast) && tree_layout(a.m, a.n_rows, leaf_bytes, c, hot, a.lay)) return true;
     return false;
   };
-  while (!fits(C)) {
-    if (C == 8) return cudaErrorInvalidConfiguration;          // not reached: 2047 nodes and rows fit
-    C *= 2;
+  // The largest cluster for which the SMs suffice, n_req C <= 148.  (15 clusters of 8 run at once and fewer than 36 of 4, an SM's
+  // neighbours being what they are, but 16 - 18 requests in two waves of 8 take 150 - 290 us for 127 nodes and with clusters of
+  // 4 120 - 290, 37 take 230 - 310 in two waves of 4 and 340 - 460 with clusters of 2.)
+  int C = 8;
+  while (C > 1 && int64_t(n_req) * C > kDefaultSMs) C /= 2;
+  // Short trees: all at once.  (18 trees of 8 nodes: 37 us with clusters of 4, 61 - 66 in two waves of 8; of 16 nodes 45 - 54
+  // and 48 - 68.  37 of 8: 43 with clusters of 2, 67 in two waves of 4; of 16 70 and 100; at 64 nodes two waves win.)
+  static ClusterRoom room;
+  while (C > 2 && a.m * C <= kShortTree && n_req > room.ask(build_tree_kernel<kGreedy, 4>, kTreeThreads, C)) C /= 2;
+  // Trees with too many rows for that: the next larger cluster that has room for a hot CTA, in as many waves as it takes.
+  // (24 trees of 768 distinct rows: 1.0 ms with clusters of 8, 2.3 with 4 and no hot CTA, 5.6 one CTA each; 148 of
+  // them: 4.5 - 5.4, 11 and 5.6; 148 of 300 rows: 1.3 - 1.7 with clusters of 4, 3.5 with 2, 2.1 one CTA each.)
+  if (!fits(C) || (C == 4 && a.m > kHotLeast && a.lay.n_hot == 0)) {
+    const bool four = C < 4 && fits(4) && a.lay.n_hot > 0;
+    C = four ? 4 : 8;
+    if (!fits(C)) return launch_rows<kGreedy>(a, n_req, stream);
   }
+  // How many requests clusters of 8 finish while 148 CTAs build one tree each depends on the hot CTAs that the rows leave room for.
+  // (Vocabulary 16000 - 32000.  Three or two, up to 1550 rows: 148 trees in 0.8 - 1.04 of the single CTAs' time.  One, up to some
+  // 1850: 75 in 0.5 - 0.8, 148 in 0.8 - 1.4, 300, three waves of CTAs, in 0.6 - 0.95.  None: 30 in 0.9, 38 in 1.3, 148 in 4.5.)
+  const int together = a.lay.n_hot >= 2 ? kDefaultSMs : a.lay.n_hot == 1 ? 105 : 30;
+  if (C == 8 && n_req > int64_t(together) * ((n_req + kDefaultSMs - 1) / kDefaultSMs)) return launch_rows<kGreedy>(a, n_req, stream);
   a.rows_inverse = uint32_t((1ull << 32) / uint64_t(a.n_rows) - (a.n_rows == 1 ? 1 : 0));
   for (;;) {
-    const cudaError_t e = a.vocab <= kLeaves * 128   ? launch_tree<kGreedy, 1>(a, n_req, C, stream)
-                          : a.vocab <= kLeaves * 256 ? launch_tree<kGreedy, 2>(a, n_req, C, stream)
-                                                     : launch_tree<kGreedy, 4>(a, n_req, C, stream);
+    const cudaError_t e = K == 1   ? launch_tree<kGreedy, 1>(a, n_req, C, stream)
+                          : K == 2 ? launch_tree<kGreedy, 2>(a, n_req, C, stream)
+                                   : launch_tree<kGreedy, 4>(a, n_req, C, stream);
     // a share of a device whose SMs hold no cluster of this size: a smaller one, if the tree fits there
-    if (e != cudaErrorInvalidClusterSize || C == 1 || !fits(C / 2)) return e;
+    if (e != cudaErrorInvalidClusterSize || C == 1) return e;
     (void)cudaGetLastError();
     C /= 2;
+    if (!fits(C)) return launch_rows<kGreedy>(a, n_req, stream);
   }
 }
 

@@ -133,6 +133,26 @@ def test_greedy_tree_at_the_edges_of_the_kernel(B, vocab, n_rows, m, n_req):
             assert vocab == 4                                        # (so few tokens that equal slot values occur)
 
 
+# short trees of more requests than run at once; trees with too many rows for the cluster that the requests leave them (the next with a
+# hot CTA, or one CTA each): at each of the kernel's three row formats
+@pytest.mark.parametrize("vocab,n_rows,m,n_req", [(4096, 40, 6, 18), (4096, 40, 24, 37), (9000, 40, 33, 74), (20000, 700, 400, 75),
+                                                  (8192, 800, 700, 38), (9000, 800, 730, 24), (20000, 800, 700, 20), (2048, 2500, 2000, 106),
+                                                  (9000, 2100, 2047, 31), (17000, 1900, 1850, 31), (17000, 1700, 1700, 19)])
+@pytest.mark.parametrize("greedy", [True, False])
+def test_trees_in_every_form(B, vocab, n_rows, m, n_req, greedy):
+    rng = np.random.default_rng(vocab + m)
+    rows = rng.random((n_rows, vocab), dtype=np.float32) ** 8                    # uneven enough for depth, and hundreds of children
+    rows /= rows.sum(axis=1, keepdims=True)
+    uni = rng.random(4099, dtype=np.float32)
+    roots = [(5 * r) % n_rows for r in range(n_req)]
+    threshold = 1e-7
+    got = run_gpu(B, rows, uni, roots, m=m) if greedy else run_gpu(B, rows, uni, roots, threshold=threshold, max_nodes=m)
+    for r in (0, n_req - 1):
+        ref = orc.build_tree_greedy(rows, uni, m, root_row=roots[r]) if greedy else orc.build_tree_threshold(rows, uni, threshold, m, root_row=roots[r])
+        assert not excused(ref)
+        compare(got, r, ref)
+
+
 @pytest.mark.parametrize("vocab,n_req,cap", [(2048, 1, 600), (9000, 20, 200), (20000, 1, 2047)])
 def test_threshold_stream_through_a_collapsing_residual(B, vocab, n_req, cap):
     """Sixty tokens of probability 2^-1, 2^-2, ... and a tail of 1e-21: after some fifty draws what is left of the row is far
