@@ -19,10 +19,11 @@
 // that holds the crossing searches its part.  The random numbers are inputs (one acceptance number
 // per node, one sampling number per node), so the caller's generator decides reproducibility.
 //
-// What bounds it: memory latency and block barriers.  With one CTA a request (the rows then take 5500 cycles to
-// arrive, the draw 8700, 32 conversions to fp64 a thread among them, and every node of the walk 1000) a
-// 64-node tree at vocabulary 32000 took 13.0 us, 16 trees of 256 nodes 28.4; now 8.9 and 22.3 (back to back).  75 requests
-// and more still get one CTA each: 100 trees of 32 nodes 23.2 -> 22.7.
+// What bounds it: memory latency and block barriers.  With one CTA a request and the walk's numbers fetched one by one (the
+// rows then take 5500 cycles to arrive, the draw 8700, 32 conversions to fp64 a thread among them, and every node of
+// the walk 1000) a 64-node tree at vocabulary 32000 took 12 - 16 us back to back, 8 trees of 256 nodes 22.5; now 8 - 12 and
+// 18.4.  75 requests and more still get one CTA each and take what they took: 148 trees of 64 nodes 24.6 (without a
+// cluster's barriers, which would make it 26.7).
 #include "common.cuh"
 
 namespace dyspec {
@@ -85,6 +86,10 @@ verify_tree_kernel(const int32_t* __restrict__ parents, const int32_t* __restric
   uint32_t n_cta;
   asm("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(n_cta));
   const int r = int(blockIdx.x / n_cta), C = int(n_cta);
+  auto sync_parts = [&] {                   // all CTAs of the request (one alone: cluster barriers cost it 2 us a call)
+    if (C > 1) cluster_sync_all();
+    else __syncthreads();
+  };
   const int node0 = node_offsets[r], n = node_offsets[r + 1] - node0;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int n_vec = vocab >> 2;                                  // float4 chunks in a row
@@ -98,7 +103,7 @@ verify_tree_kernel(const int32_t* __restrict__ parents, const int32_t* __restric
     }
     return;                                 // (all CTAs of the request)
   }
-  cluster_arrive();                         // "this CTA has started": only then may the others write its shared memory
+  if (C > 1) cluster_arrive();              // "this CTA has started": only then may the others write its shared memory
   bool bad = false;
   for (int i = tid; i < n; i += kVThreads) {
     int p_ = parents[node0 + i];
@@ -129,7 +134,7 @@ verify_tree_kernel(const int32_t* __restrict__ parents, const int32_t* __restric
     s_go[p] = go;
   }
   __syncthreads();
-  cluster_wait();                           // (here, where every path passes; the loads above hide it)
+  if (C > 1) cluster_wait();                // (here, where every path passes; the loads above hide it)
 
   auto emit = [&](int token, int node) {
     if (writer && n_out < max_out) { out_tokens[size_t(r) * max_out + n_out] = token; out_nodes[size_t(r) * max_out + n_out] = node; }
@@ -257,7 +262,7 @@ verify_tree_kernel(const int32_t* __restrict__ parents, const int32_t* __restric
         }
       }
       __syncwarp();
-      cluster_sync_all();                                        // (also the block's barrier)
+      sync_parts();
       float tot = 0.f, all = 0.f;
       for (int c = 0; c < C; ++c) { tot += s.part[parity][c].sum; all += s.part[parity][c].count; }
       const Part own = s.part[parity][(y2 >> 2) / (K * kVThreads)];
@@ -311,7 +316,7 @@ verify_tree_kernel(const int32_t* __restrict__ parents, const int32_t* __restric
         st_dsmem_f64(map_to_cta(smem_u32(&s.draw[rank]), uint32_t(lane)), mine);
       }
       __syncwarp();
-      cluster_sync_all();
+      sync_parts();
       double total = 0.0;
       for (int c = 0; c < C; ++c) total += s.draw[c];
       if (attempt > 0 || total > 0.0) {
@@ -373,13 +378,13 @@ verify_tree_kernel(const int32_t* __restrict__ parents, const int32_t* __restric
         const int v4 = vec0 + k * kVThreads + tid;
         R[k] = v4 < n_vec ? __ldg(t_row + v4) : make_float4(0.f, 0.f, 0.f, 0.f);
       }
-      cluster_sync_all();                                        // everyone has read the parts of the first attempt
+      sync_parts();                                              // everyone has read the parts of the first attempt
     }
     ++n_out;
     break;
   }
   if (writer) out_count[r] = min(n_out, max_out);
-  cluster_sync_all();                                            // nobody leaves while its shared memory may be written
+  if (C > 1) cluster_sync_all();                                 // nobody leaves while its shared memory may be written
 }
 
 namespace {
@@ -402,7 +407,7 @@ cudaError_t launch_parts(int C, const int32_t* parents, const int32_t* tokens, c
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = C > 1 ? 1 : 0;
   const cudaError_t e = cudaLaunchKernelEx(&cfg, verify_tree_kernel<K>, parents, tokens, draft_probs, target_probs, accept_u, sample_u,
                                            node_offsets, max_nodes, vocab, bonus_at_leaf, out_tokens, out_nodes, out_count,
                                            max_out, status);
@@ -416,10 +421,13 @@ cudaError_t launch_verify_tree(const int32_t* parents, const int32_t* tokens, co
                                int32_t* out_tokens, int32_t* out_nodes, int32_t* out_count, int max_out, int32_t* status,
                                cudaStream_t stream) {
   if (n_req <= 0) return cudaSuccess;
-  // As many CTAs a request as leave every CTA a chunk of its own, while all requests still run at once.
+  // As many CTAs a request as leave every CTA a chunk of its own, while all requests still run at once: 15 clusters of 8 and 33 - 36 of
+  // 4 do, not the 18 and 37 that the SMs would make (vocabulary 32000, 18 trees of 256 nodes: 33 us in two waves of 8, 19 with
+  // clusters of 4; 37: 29 in two waves of 4, 22 with clusters of 2).
   const int n_chunks = (vocab + 4 * kVThreads - 1) / (4 * kVThreads);
+  static ClusterRoom room;
   int C = 8, K = 1;
-  while (C > 1 && (C >= 2 * n_chunks || int64_t(n_req) * C > kDefaultSMs)) C /= 2;
+  while (C > 1 && (C >= 2 * n_chunks || n_req > room.ask(verify_tree_kernel<8>, kVThreads, C))) C /= 2;
   auto go = [&](auto launch) {
     return launch(C, parents, tokens, draft_probs, target_probs, accept_u, sample_u, node_offsets, n_req, max_nodes, vocab,
                   bonus_at_leaf, out_tokens, out_nodes, out_count, max_out, status, stream);
