@@ -48,3 +48,44 @@ def test_first_launch_of_a_process(program):
     env = dict(os.environ, PYTHONPATH=os.pathsep.join([os.path.dirname(HERE), HERE]))
     r = subprocess.run([sys.executable, "-c", program], env=env, capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, r.stderr[-2000:]
+
+CAPTURED = """
+import numpy as np, torch
+import cuda.bindings.runtime as rt
+from paper_2410_11744_b200 import binding as B, workloads as wl
+t = lambda a: torch.from_numpy(np.ascontiguousarray(a)).to("cuda:0")
+case = wl.make_verify_case(3, 32000, [wl.chain_tree(3)] * 4, sharpness=2.0, disagreement=1.5)
+par, tok, offs = t(np.concatenate(case.parents)), t(np.concatenate(case.tokens)), t(case.node_offsets)
+dp, tp, au, su = t(case.draft_probs), t(case.target_probs), t(case.accept_u), t(case.sample_u)
+rows, uni = wl.make_draft_table(5, 16, 4096, 2.0)
+rows, uni, root = t(rows), t(uni), t(np.arange(4, dtype=np.int32))
+outs = []
+def call(stream):
+    o = [torch.zeros((4, 64), dtype=torch.int32, device="cuda:0") for _ in range(5)] + [torch.zeros((4, 64), device="cuda:0") for _ in range(2)]
+    c = [torch.zeros(4, dtype=torch.int32, device="cuda:0") for _ in range(2)]
+    torch.cuda.synchronize()
+    outs.append(o + c)
+    return lambda: (B.dyspec_verify_tree(par, tok, dp, tp, au, su, offs, 4, 3, 32000, o[0], o[1], c[0], 64, bonus_at_leaf=True, stream=stream),
+                    B.dyspec_build_tree_greedy(rows, 16, 4096, uni, len(uni), root, 4, 63, o[2], o[3], o[5], o[6], o[4], c[1], stream=stream))
+s = torch.cuda.Stream()
+h = s.cuda_stream
+f = call(h)
+assert rt.cudaStreamBeginCapture(h, rt.cudaStreamCaptureMode.cudaStreamCaptureModeGlobal)[0] == 0
+f()
+err, graph = rt.cudaStreamEndCapture(h)
+assert err == 0, err
+err, run = rt.cudaGraphInstantiate(graph, 0)
+assert err == 0, err
+assert rt.cudaGraphLaunch(run, h)[0] == 0
+s.synchronize()
+call(h)()
+s.synchronize()
+assert all(torch.equal(a, b) for a, b in zip(*outs)) and int(outs[0][8].min()) == 64
+"""
+
+
+def test_first_launch_inside_a_capture():
+    pytest.importorskip("cuda.bindings.runtime")
+    env = dict(os.environ, PYTHONPATH=os.pathsep.join([os.path.dirname(HERE), HERE]))
+    r = subprocess.run([sys.executable, "-c", CAPTURED], env=env, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
