@@ -14,13 +14,14 @@
 //        enter(i) -> enter(first child of i), or exit(i) for a leaf
 //        exit(i)  -> enter(next sibling of i), or exit(parent of i), or the end of the list
 //   3. list ranking with weight 1 on enter elements: S(e) = number of enter elements from e to the
-//      end, so the pre-order index of node i is n - S(enter(i)).  Seven elements in 32 are splitters: those that a
+//      end, so the pre-order index of node i is n - S(enter(i)).  Up to 256 nodes by pointer jumping over all elements,
+//      ceil(log2(2 n)) rounds.  Larger trees: seven elements in 32 are splitters, those that a
 //      multiplication modulo a power of two (a bijection, so a splitter's number gives its element back) takes
 //      below a bound.  A thread walks from each splitter to the next one (5 steps on average, some 30 at
 //      most), the splitters alone are ranked by pointer jumping in eight warps, and every element adds its
-//      distance.  (Jumping over all 2 n elements takes ceil(log2(2 n)) rounds of four elements a thread; that, and
-//      a table that had to be cleared and searched, made this kernel take 3.3, 9.5 and 18.0 us for 64, 1024
-//      and 2048 random nodes, back to back; now 3.4, 8.9 and 13.6.)
+//      distance.
+// Measured back to back, us: random trees of 65, 128, 200 nodes 4.0, 3.9, 4.4 (with splitters 5.1, 4.4, 5.0); of 512, 1024 and
+// 2048 nodes 5.6, 8.3, 13.0 (without them 6.1, 9.8, 18.1).
 //
 // A parent outside {-1} U [0, i) makes that node a root and reports DYSPEC_ERR_BAD_TREE, as in the
 // mask builder.
@@ -31,8 +32,15 @@ namespace dyspec {
 
 namespace {
 constexpr uint32_t kNone = 0xFFFFu;
-constexpr int kJumpThreads = 256;
+constexpr int kJumpThreads = 256;                 // (a launch of more than kJumpAll nodes has more threads)
+
+__device__ __forceinline__ uint32_t jumped(const uint32_t* cur, int k) {
+  const uint32_t v = cur[k], to = v >> 16;
+  if (to == kNone) return v;
+  const uint32_t b = cur[to];
+  return (b & 0xFFFF0000u) | ((v & 0xFFFFu) + (b & 0xFFFFu));
 }
+}  // namespace
 
 __global__ void __launch_bounds__(1024, 1)
 dfs_reorder_kernel(const int32_t* __restrict__ parents, const ReqInfo* __restrict__ reqs, int single_n,
@@ -60,8 +68,8 @@ dfs_reorder_kernel(const int32_t* __restrict__ parents, const ReqInfo* __restric
   uint16_t* s_next = reinterpret_cast<uint16_t*>(ro_smem + l.next); // [E] the tour
   uint32_t* s_at = reinterpret_cast<uint32_t*>(ro_smem + l.at);     // [E] number of the segment's splitter << 16 | enter elements of the segment before it
   const Splitters sp(E);
-  uint32_t* cur = reinterpret_cast<uint32_t*>(ro_smem + l.jump);    // [sp.count] number of a splitter ahead << 16 | enter elements up to it
-  uint32_t* nxt = cur + sp.count;
+  uint32_t* cur = reinterpret_cast<uint32_t*>(ro_smem + l.jump);    // an element (n <= kJumpAll) or the number of a splitter ahead << 16 | enter elements up to it
+  uint32_t* nxt = cur + (n <= kJumpAll ? E : sp.count);
   bool bad = false;
 
 #pragma unroll 2
@@ -116,56 +124,55 @@ dfs_reorder_kernel(const int32_t* __restrict__ parents, const ReqInfo* __restric
   __syncthreads();
 
   // ---- 2. Euler tour
-  for (int e = tid; e < E; e += nthr) {
-    uint32_t nx;
-    if (e < n) {
-      nx = s_fc[e] != kNone ? uint32_t(s_fc[e]) : uint32_t(n + e);
-    } else {
-      const int i = e - n;
-      nx = s_ns[i] != kNone ? uint32_t(s_ns[i]) : (s_par[i] < n ? uint32_t(n + s_par[i]) : kNone);
-    }
-    s_next[e] = uint16_t(nx);
-  }
-  __syncthreads();
+  auto next_of = [&](int e) -> uint32_t {
+    if (e < n) return s_fc[e] != kNone ? uint32_t(s_fc[e]) : uint32_t(n + e);
+    const int i = e - n;
+    return s_ns[i] != kNone ? uint32_t(s_ns[i]) : s_par[i] < n ? uint32_t(n + s_par[i]) : kNone;
+  };
 
-  // ---- 3. list ranking.  A thread walks from each of its splitters to the next one (the tour starts at one: element 0) ...
-  for (int k = tid; k < sp.count; k += nthr) {
-    uint32_t e = sp.element(k), enters = 0;
-    if (e >= uint32_t(E)) continue;
-    int to;
-    do {                                                            // at most E steps: the tour has no cycle
-      s_at[e] = (uint32_t(k) << 16) | enters;
-      enters += e < uint32_t(n) ? 1u : 0u;
-      e = s_next[e];
-      to = sp.number(e);
-    } while (e != kNone && to >= sp.count);
-    cur[k] = ((e != kNone ? uint32_t(to) : kNone) << 16) | enters;
-  }
-  __syncthreads();
-  // ... and the splitters jump: after round r one points 2^r segments ahead (or to the end) and holds their enter elements.
-  // (Eight warps: with all 32 a round costs their barrier and four times the instruction issue.)
-  const int jumpers = min(nthr, kJumpThreads);
-  for (int span = 1; span < sp.count; span <<= 1) {
-    if (tid < jumpers) {
-      for (int k = tid; k < sp.count; k += jumpers) {
-        if (sp.element(k) >= uint32_t(E)) continue;
-        uint32_t v = cur[k];
-        const uint32_t to = v >> 16;
-        if (to != kNone) {
-          const uint32_t b = cur[to];
-          v = (b & 0xFFFF0000u) | ((v & 0xFFFFu) + (b & 0xFFFFu));
-        }
-        nxt[k] = v;
-      }
-      asm volatile("bar.sync 1, %0;" ::"r"(jumpers) : "memory");
+  // ---- 3. list ranking
+  if (n <= kJumpAll) {                                              // after round r an element points 2^r steps ahead
+    for (int e = tid; e < E; e += nthr) cur[e] = (next_of(e) << 16) | (e < n ? 1u : 0u);
+    __syncthreads();
+    for (int span = 1; span < E; span <<= 1) {
+      for (int e = tid; e < E; e += nthr) nxt[e] = jumped(cur, e);
+      __syncthreads();
+      uint32_t* t = cur; cur = nxt; nxt = t;
     }
-    uint32_t* t = cur; cur = nxt; nxt = t;
+  } else {
+    // A thread walks from each of its splitters to the next one (the tour starts at one: element 0) ...
+    for (int e = tid; e < E; e += nthr) s_next[e] = uint16_t(next_of(e));
+    __syncthreads();
+    for (int k = tid; k < sp.count; k += nthr) {
+      uint32_t e = sp.element(k), enters = 0;
+      if (e >= uint32_t(E)) continue;
+      int to;
+      do {                                                          // at most E steps: the tour has no cycle
+        s_at[e] = (uint32_t(k) << 16) | enters;
+        enters += e < uint32_t(n) ? 1u : 0u;
+        e = s_next[e];
+        to = sp.number(e);
+      } while (e != kNone && to >= sp.count);
+      cur[k] = ((e != kNone ? uint32_t(to) : kNone) << 16) | enters;
+    }
+    __syncthreads();
+    // ... and the splitters jump: after round r one points 2^r segments ahead (or to the end) and holds their enter elements.
+    // (Eight warps: with all 32 a round costs their barrier and four times the instruction issue.)
+    for (int span = 1; span < sp.exist; span <<= 1) {
+      if (tid < kJumpThreads) {
+        for (int k = tid; k < sp.count; k += kJumpThreads)
+          if (sp.element(k) < uint32_t(E)) nxt[k] = jumped(cur, k);
+        asm volatile("bar.sync 1, %0;" ::"n"(kJumpThreads) : "memory");
+      }
+      uint32_t* t = cur; cur = nxt; nxt = t;
+    }
+    __syncthreads();
   }
-  __syncthreads();
 
   grid_dependency_wait();     // outputs may still be in use by the kernel before this one in the stream
   if (bad && status) atomicCAS(status, 0, DYSPEC_ERR_BAD_TREE);
   auto preorder = [&](int i) {                                      // n - (enter elements from enter(i) to the end)
+    if (n <= kJumpAll) return n - int(cur[i] & 0xFFFFu);
     const uint32_t a = s_at[i];
     return n - int(cur[a >> 16] & 0xFFFFu) + int(a & 0xFFFFu);
   };

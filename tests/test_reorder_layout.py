@@ -16,12 +16,18 @@ int main() {
   for (int n = 1; n <= 2048; ++n) {
     const dyspec::DfsLayout l(n);
     const dyspec::Splitters sp(2 * n);
-    const int lists = l.jump + 8 * sp.count, tabled = l.table + (n + 1) * ((n + 31) / 32);
+    const bool all = n <= dyspec::kJumpAll;        // all elements jump, from the table's place on
+    const int lists = l.jump + 8 * (all ? 2 * n : sp.count), tabled = l.table + (n + 1) * ((n + 31) / 32);
+    if (!all && (l.next < l.table || l.at < l.next + 4 * n || l.jump < l.at + 8 * n)) { std::printf("n = %d: parts overlap\n", n); return 1; }
     if (l.bytes < lists || l.bytes < tabled) { std::printf("n = %d: %d bytes, %d and %d needed\n", n, l.bytes, lists, tabled); return 1; }
     if (l.bytes < worst) { std::printf("largest tree %d: %d bytes, %d needed by a smaller one\n", n, l.bytes, worst); return 1; }
     worst = l.bytes;
-    for (int e = 0; e < 2 * n; ++e)                // a splitter's number gives its element back
+    int exist = 0;
+    for (int e = 0; e < 2 * n; ++e) {              // a splitter's number gives its element back
       if (sp.element(sp.number(e)) != unsigned(e)) { std::printf("n = %d: element %d\n", n, e); return 1; }
+      exist += sp.number(e) < sp.count;
+    }
+    if (exist > sp.exist) { std::printf("n = %d: %d splitters, %d expected\n", n, exist, sp.exist); return 1; }   // rounds of jumping
   }
   return worst <= 227 * 1024 ? 0 : 1;
 }
