@@ -87,10 +87,11 @@ def _ptr(t) -> Optional[int]:
 
 def _stream(stream=None) -> int:
     if stream is None:
-        # The handle of torch.cuda.current_stream() without the Stream object around it: 0.4 us where that took 3.3 of the
-        # 8 - 11 us that a call cost the host, which is what a small call is bound by.
         import torch
-        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+        # The handle of torch.cuda.current_stream() without the Stream object around it: 0.4 us where that takes 3.3 of the
+        # 8 - 11 us that a call costs the host, which is what a small call is bound by.  It is not a public name of torch.
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        return raw(torch.cuda.current_device()) if raw is not None else torch.cuda.current_stream().cuda_stream
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream

@@ -86,3 +86,16 @@ def test_argument_errors_are_reported_before_any_launch(binding):
     assert lib.dyspec_set_default_shape(4, 4, 96, 4, 0.0) == -2
     assert lib.dyspec_set_tuning(7, 0, 1) == -1
     assert lib.dyspec_plan_destroy(None) == 0
+
+
+def test_current_stream_with_and_without_the_raw_handle(binding, monkeypatch):
+    """The raw handle's getter is not a public name of torch: without it the public one is asked."""
+    import types
+    import torch
+    monkeypatch.setattr(torch.cuda, "current_device", lambda: 3)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: types.SimpleNamespace(cuda_stream=77))
+    monkeypatch.setattr(torch._C, "_cuda_getCurrentRawStream", lambda device: 1000 + device, raising=False)
+    assert binding._stream() == 1003
+    monkeypatch.delattr(torch._C, "_cuda_getCurrentRawStream")
+    assert binding._stream() == 77
+    assert binding._stream(5) == 5 and binding._stream(types.SimpleNamespace(cuda_stream=6)) == 6
