@@ -987,7 +987,8 @@ __device__ __forceinline__ void run_hot(const TreeArgs& a, uint8_t* sm, const ui
     }
     __syncwarp();
     if (stop) return;
-    if (total.hi + total.lo < built * 0x1p-40) {               // (rare: what is left is small against the tables' rounding)
+    // rare: what is left is small against the tables' rounding, or no number (a token that was none may just have left)
+    if (!(total.hi + total.lo >= built * 0x1p-40)) {
       for (int k = 0; k < kChunks; ++k) build_chunk(s_row, s_sub, k, lane);
       __syncwarp();
       upto = scan(s_sub[(lane * kSubs + kSubs - 1) * 32 + 31], lane);

@@ -241,3 +241,30 @@ def test_a_wait_that_runs_out_is_reported(B, greedy, n_req):
         compare(got, r, ref)
     with pytest.raises(B.DyspecError):
         call(wait_limit_ns=-1)
+
+
+@pytest.mark.parametrize("what", ["nan last", "nan inside", "inf inside", "no mass"])
+@pytest.mark.parametrize("greedy", [True, False])
+def test_rows_that_are_no_distributions_whatever_the_cluster(B, what, greedy):
+    """Where a sum is no number the last token is drawn, with r = 0, and leaves the row; if it was the cause, the draws after it are
+    ordinary ones again.  The same in hot CTAs, in clusters without one and in a single CTA."""
+    rng = np.random.default_rng(3)
+    vocab, m = 1000, 60
+    rows = rng.random((12, vocab), dtype=np.float32) ** 4
+    rows /= rows.sum(axis=1, keepdims=True)
+    if what == "no mass":
+        rows[::2] = 0.0
+    else:
+        rows[::2, vocab - 1 if what == "nan last" else vocab // 2] = np.inf if what == "inf inside" else np.nan
+    uni = rng.random(4099, dtype=np.float32)
+    trees = []
+    for n_req in (1, 20, 40, 80):
+        got = run_gpu(B, rows, uni, [0] * n_req, m=m) if greedy else run_gpu(B, rows, uni, [0] * n_req, threshold=1e-6, max_nodes=m)
+        assert int(got[5].min()) == int(got[5].max()) == m + 1
+        trees.append([x[n_req - 1] for x in got[:5]])
+    assert trees[0][1][1] == vocab - 1
+    if what == "nan last":
+        assert len(set(trees[0][1][1:].tolist())) >= 4
+    for t in trees[1:]:
+        assert all(np.array_equal(t[i], trees[0][i]) for i in (0, 1, 4))
+        assert np.allclose(t[2], trees[0][2], rtol=1e-6, atol=0) and np.allclose(t[3], trees[0][3], rtol=1e-6, atol=0)
