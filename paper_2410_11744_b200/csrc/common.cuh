@@ -237,8 +237,8 @@ __device__ __forceinline__ bool mbar_test_wait(uint32_t bar, uint32_t parity) {
       : "memory");
   return done != 0;
 }
-// Three probes whose round trips overlap: the answers come back together, about one probe latency
-// after the first was issued (three mbar_test_wait calls in a row would take three latencies, since
+// Three (two) probes whose round trips overlap: the answers come back together, about one probe latency
+// after the first was issued (mbar_test_wait calls in a row would take a latency each, since
 // each consumes its predicate before the next is issued).  Bit k of the result = barrier k's phase done.
 __device__ __forceinline__ uint32_t mbar_test_wait3(uint32_t bar0, uint32_t parity0, uint32_t bar1, uint32_t parity1,
                                                     uint32_t bar2, uint32_t parity2) {
@@ -252,6 +252,18 @@ __device__ __forceinline__ uint32_t mbar_test_wait3(uint32_t bar0, uint32_t pari
       "or.b32 r0, r0, r1;\n\tor.b32 %0, r0, r2;\n\t}"
       : "=r"(done)
       : "r"(bar0), "r"(parity0), "r"(bar1), "r"(parity1), "r"(bar2), "r"(parity2)
+      : "memory");
+  return done;
+}
+__device__ __forceinline__ uint32_t mbar_test_wait2(uint32_t bar0, uint32_t parity0, uint32_t bar1, uint32_t parity1) {
+  uint32_t done;
+  asm volatile(
+      "{\n\t.reg .pred p0, p1;\n\t.reg .u32 r0, r1;\n\t"
+      "mbarrier.test_wait.parity.shared::cta.b64 p0, [%1], %2;\n\t"
+      "mbarrier.test_wait.parity.shared::cta.b64 p1, [%3], %4;\n\t"
+      "selp.u32 r0, 1, 0, p0;\n\tselp.u32 r1, 2, 0, p1;\n\tor.b32 %0, r0, r1;\n\t}"
+      : "=r"(done)
+      : "r"(bar0), "r"(parity0), "r"(bar1), "r"(parity1)
       : "memory");
   return done;
 }
@@ -486,6 +498,32 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
   uint32_t r;
   asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
   return r;
+}
+// Packed fp32 pairs (sm_100: one instruction works on two floats held in a 64-bit register pair)
+// and the three-input maximum: the softmax threads are bound by instruction issue, and these halve
+// the count of the scale, sum and max instructions.
+__device__ __forceinline__ uint64_t pack_f32x2(float lo, float hi) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void unpack_f32x2(uint64_t v, float& lo, float& hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ uint64_t fma_f32x2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ float max3_f32(float a, float b, float c) {
+  float d;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
 }
 #endif  // __CUDACC__
 
