@@ -7,7 +7,7 @@
 //   warp 9     issues S = Q K^T on the tensor cores (tcgen05.mma, M = 64, N = 64, both operands from
 //              shared memory) as soon as a tile's K has landed and one of four score buffers in tensor
 //              memory is free, so the scores run ahead of the softmax;
-//   warp 10    issues O += P V on the tensor cores (M = 64, one product per 64-column panel of V) when a
+//   warp 10    issues O += P V on the tensor cores (M = 64, N = D) when a
 //              warp set has put the tile's probabilities into shared memory (over the K tile, which the
 //              score product has finished with), into that set's accumulator in tensor memory; the
 //              commit behind it frees the ring stage;
@@ -104,15 +104,14 @@ __device__ __forceinline__ void tmem_ld_scores(uint32_t taddr, float (&s)[BN / 8
   }
 }
 
-// O += P V on the tensor cores as well: M = 64 rows, K = 64 keys in four 16-key steps, one product per
-// 64-column panel of V (N = 64).  P is a K-major operand (64 rows x 64 keys of bf16 = one 128-byte row each,
-// same layout as a Q or K panel); a V panel is an MN-major operand (keys x 64 columns, columns contiguous):
-// 8-key groups 1024 bytes apart.  (One N = D product whose operand hops from panel to panel through the
-// descriptor's leading-dimension offset gave wrong upper columns in every CTA but the first of a cluster;
-// per-panel products do not depend on that field.)
+// O += P V on the tensor cores as well: M = 64 rows, N = D columns, K = 64 keys in four 16-key steps.  P is a K-major
+// operand (64 rows x 64 keys of bf16 = one 128-byte row each, same layout as a Q or K panel); V is an MN-major operand (keys x
+// columns, columns contiguous) in panels of 64 columns: 8-key groups 1024 bytes apart, the next panel at the leading
+// offset.  (A product per panel reads P twice: eight layers of one 64-node tree over 1024 keys, 32 heads, 78.2 us against 76.7;
+// two of a ragged batch of 16 186.5 against 185.2.)
 template <int D>
 __host__ __device__ constexpr uint32_t idesc_pv() {
-  return (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | (uint32_t(64 >> 3) << 17) | (uint32_t(BM >> 4) << 24);   // N = 64 per panel
+  return (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | (uint32_t(D >> 3) << 17) | (uint32_t(BM >> 4) << 24);
 }
 constexpr int kSBufs = 4;                 // score buffers in tensor memory (64 columns each)
 constexpr float kRescaleThreshold = 8.f;  // log2 units: O is rescaled only when a row maximum grows by more
@@ -324,15 +323,11 @@ tree_attn_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
           mbar_wait(bar_pready + 8 * stage, ph, abort_flag, p.status);
           tc_fence_after();
           const uint32_t p_lo = desc_lo(s_kv + stage * L::kStageBytes);                        // P sits where the K tile was
-          const uint32_t v_lo = desc_lo(s_kv + stage * L::kStageBytes + L::kTileBytes);
-          // one product per 64-column panel of V (N = 64 each): no leading-dimension hop inside an operand
+          const uint32_t v_lo = desc_lo(s_kv + stage * L::kStageBytes + L::kTileBytes) - (1u << 16) + ((uint32_t(L::kPanelBytes) >> 4) << 16);
 #pragma unroll
-          for (int h = 0; h < L::kHalves; ++h)
-#pragma unroll
-            for (int kk = 0; kk < BN / 16; ++kk)
-              umma_ss(tmem_base + uint32_t(pv_set) * kOCols + uint32_t(h) * 64u, p_lo + uint32_t(kk) * (32u >> 4),
-                      v_lo + uint32_t(h) * (uint32_t(L::kPanelBytes) >> 4) + uint32_t(kk) * (2048u >> 4), kDescHi, kIdescPV,
-                      (m >= 2 || kk > 0) ? 1u : 0u);
+          for (int kk = 0; kk < BN / 16; ++kk)
+            umma_ss(tmem_base + uint32_t(pv_set) * kOCols, p_lo + uint32_t(kk) * (32u >> 4), v_lo + uint32_t(kk) * (2048u >> 4),
+                    kDescHi, kIdescPV, (m >= 2 || kk > 0) ? 1u : 0u);
           tc_commit(bar_empty + 8 * stage);
           tc_commit(bar_pvdone + 8 * pv_set);
           if (++stage == n_stages) { stage = 0; ph ^= 1u; }
