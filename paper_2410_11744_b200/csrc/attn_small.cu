@@ -86,8 +86,7 @@ constexpr uint32_t kIdescQK = (1u << 4) | (1u << 7) | (1u << 10) | (uint32_t(BN 
 // 16 w .. 16 w + 15 from its own lane quarter, and the 16x256b load shape hands them out in 16 x 8
 // fragments: registers 4j .. 4j+3 of lane (gid = lane / 4, tig = lane % 4) are (row gid, columns
 // 8j + 2 tig, +1) and (row gid + 8, same columns).
-__device__ __forceinline__ void tmem_ld_scores(uint32_t taddr, float (&s)[BN / 8][4]) {
-  uint32_t r[32];
+__device__ __forceinline__ void tmem_ld_request(uint32_t taddr, uint32_t (&r)[32]) {   // (the wait is the caller's)
   asm volatile(
       "tcgen05.ld.sync.aligned.16x256b.x8.b32 "
       "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
@@ -96,7 +95,12 @@ __device__ __forceinline__ void tmem_ld_scores(uint32_t taddr, float (&s)[BN / 8
         "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
         "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
       : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+__device__ __forceinline__ void tmem_ld_scores(uint32_t taddr, float (&s)[BN / 8][4]) {
+  uint32_t r[32];
+  tmem_ld_request(taddr, r);
+  tmem_wait_ld();
 #pragma unroll
   for (int j = 0; j < BN / 8; ++j) {
     s[j][0] = __uint_as_float(r[4 * j]); s[j][1] = __uint_as_float(r[4 * j + 1]);
@@ -611,17 +615,18 @@ tree_attn_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
       const float ka_lo = fast_exp2(m_lo - ref_lo), kb_lo = fast_exp2(ml.x - ref_lo);
       const float ka_hi = fast_exp2(m_hi - ref_hi), kb_hi = fast_exp2(ml.y - ref_hi);
       static_assert(HT == 8 || HT == 4, "half of the columns: 64 or 32");
-      float mine[8][4], theirs[8][4];
+      uint32_t mine[32], theirs[32];                       // (both halves asked for before either is waited for)
       // (D = 64: a half is 32 columns; the loads fetch 64 and the upper 32 are ignored -- they belong to the
       //  neighbouring buffer, which is mapped, so this is safe)
-      if (my_tiles > 0) tmem_ld_rows<8>(t_rows + uint32_t(set) * kOCols + uint32_t(cbase), mine);
-      if (other_tiles > 0) tmem_ld_rows<8>(t_rows + uint32_t(1 - set) * kOCols + uint32_t(cbase), theirs);
+      if (my_tiles > 0) tmem_ld_request(t_rows + uint32_t(set) * kOCols + uint32_t(cbase), mine);
+      if (other_tiles > 0) tmem_ld_request(t_rows + uint32_t(1 - set) * kOCols + uint32_t(cbase), theirs);
+      tmem_wait_ld();
 #pragma unroll
       for (int j = 0; j < HT; ++j) {
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-          const float a_ = my_tiles > 0 ? mine[j][e] * (e < 2 ? ka_lo : ka_hi) : 0.f;
-          const float b_ = other_tiles > 0 ? theirs[j][e] * (e < 2 ? kb_lo : kb_hi) : 0.f;
+          const float a_ = my_tiles > 0 ? __uint_as_float(mine[4 * j + e]) * (e < 2 ? ka_lo : ka_hi) : 0.f;
+          const float b_ = other_tiles > 0 ? __uint_as_float(theirs[4 * j + e]) * (e < 2 ? kb_lo : kb_hi) : 0.f;
           o[j][e] = a_ + b_;
         }
       }
