@@ -503,7 +503,7 @@ tree_attn_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
         const float y_lo = __shfl_xor_sync(0xffffffffu, mx_lo, 1), y_hi = __shfl_xor_sync(0xffffffffu, mx_hi, 1);
         mx_lo = fmaxf(mx_lo, y_lo); mx_hi = fmaxf(mx_hi, y_hi);
         const float z_lo = __shfl_xor_sync(0xffffffffu, mx_lo, 2), z_hi = __shfl_xor_sync(0xffffffffu, mx_hi, 2);
-        mx_lo = fmaxf(mx_lo, z_lo) * p.scale_log2e; mx_hi = fmaxf(mx_hi, z_hi) * p.scale_log2e;
+        mx_lo = scaled_maximum(fmaxf(mx_lo, z_lo), p.scale_log2e); mx_hi = scaled_maximum(fmaxf(mx_hi, z_hi), p.scale_log2e);
       }
       const float mn_lo = fmaxf(m_lo, mx_lo), mn_hi = fmaxf(m_hi, mx_hi);
       confirm_pv_done((got & 2u) != 0u);
@@ -529,15 +529,16 @@ tree_attn_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
       // exp2(-inf - 0) = 0 and no inf - inf appears.
       const float ref_lo = m_lo == -INFINITY ? 0.f : m_lo;
       const float ref_hi = m_hi == -INFINITY ? 0.f : m_hi;
-      const uint64_t scale2 = pack_f32x2(p.scale_log2e, p.scale_log2e);
+      const float scale_lo = scale_for_reference(m_lo, p.scale_log2e), scale_hi = scale_for_reference(m_hi, p.scale_log2e);
+      const uint64_t scale2_lo = pack_f32x2(scale_lo, scale_lo), scale2_hi = pack_f32x2(scale_hi, scale_hi);
       const uint64_t neg_lo = pack_f32x2(-ref_lo, -ref_lo), neg_hi = pack_f32x2(-ref_hi, -ref_hi);
       uint64_t sum2_lo = 0ull, sum2_hi = 0ull;
       uint32_t pf[BN / 8][2];
 #pragma unroll
       for (int j = 0; j < BN / 8; ++j) {
         float p0, p1, p2, p3;
-        unpack_f32x2(fma_f32x2(pack_f32x2(s[j][0], s[j][1]), scale2, neg_lo), p0, p1);
-        unpack_f32x2(fma_f32x2(pack_f32x2(s[j][2], s[j][3]), scale2, neg_hi), p2, p3);
+        unpack_f32x2(fma_f32x2(pack_f32x2(s[j][0], s[j][1]), scale2_lo, neg_lo), p0, p1);
+        unpack_f32x2(fma_f32x2(pack_f32x2(s[j][2], s[j][3]), scale2_hi, neg_hi), p2, p3);
         p0 = fast_exp2(p0); p1 = fast_exp2(p1); p2 = fast_exp2(p2); p3 = fast_exp2(p3);
         sum2_lo = add_f32x2(sum2_lo, pack_f32x2(p0, p1));
         sum2_hi = add_f32x2(sum2_hi, pack_f32x2(p2, p3));

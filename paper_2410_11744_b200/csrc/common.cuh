@@ -525,6 +525,24 @@ __device__ __forceinline__ float max3_f32(float a, float b, float c) {
   asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
   return d;
 }
+// A softmax weight is exp2(score * scale - m), m the row's maximum times scale, rounded.  Product and difference are ONE
+// multiply-add, which keeps what m was rounded by: up to 2^30 a factor of at most 2^32 on all of a row's weights, which
+// the division by their sum takes out again; from 2^31 on an overflow (NaN, or a sum of 0).  Beyond 2^30 two fp32 scores
+// are equal or at least 2^6 apart after scaling, so every scale that is no smaller gives the same weights, and with
+// the next power of two the product, and with it m, is exact.  Maxima on the two sides of the line keep their order.
+// (Free: selects in front of the loop over a tile's scores.  A branch that rounds the products first costs
+// the tensor-core kernel 2 - 4 %, 128 scores a thread.)
+constexpr float kCoarseReference = 1073741824.f;
+__device__ __forceinline__ float scale_rounded_up(float scale) {
+  return __uint_as_float((__float_as_uint(scale) + 0x7fffffu) & 0xff800000u);
+}
+__device__ __forceinline__ float scaled_maximum(float raw, float scale) {
+  const float x = raw * scale;
+  return fabsf(x) > kCoarseReference ? raw * scale_rounded_up(scale) : x;
+}
+__device__ __forceinline__ float scale_for_reference(float m, float scale) {
+  return fabsf(m) > kCoarseReference ? scale_rounded_up(scale) : scale;
+}
 #endif  // __CUDACC__
 
 }  // namespace dyspec
