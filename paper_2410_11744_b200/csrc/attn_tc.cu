@@ -750,7 +750,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
           mx4[2] = max3_f32(mx4[2], __uint_as_float(sv[i + 4]), __uint_as_float(sv[i + 5]));
           mx4[3] = max3_f32(mx4[3], __uint_as_float(sv[i + 6]), __uint_as_float(sv[i + 7]));
         }
-        const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3])) * p.scale_log2e;   // scale > 0
+        const float mx = scaled_maximum(fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3])), p.scale_log2e);   // scale > 0
         const float m_new = fmaxf(m_used, mx);
         if (r == 0) trace_event(tc_cur, DYSPEC_TAG(1 + h, 3, j));
         if (j > 0) {
@@ -779,7 +779,8 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
         const float neg_ref = m_used == -INFINITY ? 0.f : -m_used;
 
         // P = 2^(s * scale - ref) as bf16 pairs, written over the first 64 S columns (masked: 2^-inf = 0)
-        const uint64_t scale2 = pack_f32x2(p.scale_log2e, p.scale_log2e), ref2 = pack_f32x2(neg_ref, neg_ref);
+        const float scale = scale_for_reference(m_used, p.scale_log2e);
+        const uint64_t scale2 = pack_f32x2(scale, scale), ref2 = pack_f32x2(neg_ref, neg_ref);
         uint64_t sum2[2] = {0ull, 0ull};
 #pragma unroll
         for (int c = 0; c < 4; ++c) {

@@ -18,7 +18,7 @@ def _bits(x):
     return (u >> 16).astype(np.uint16)
 
 
-@pytest.mark.parametrize("regime", [0])
+@pytest.mark.parametrize("regime", [0, 1])
 @pytest.mark.parametrize("ctas, combine", [(0, 2), (3, 0)])
 @pytest.mark.parametrize("hq, hkv, d, n, L", [(4, 4, 64, 16, 128), (32, 32, 128, 64, 440), (8, 1, 128, 8, 300), (8, 8, 64, 33, 0)])
 def test_scores_far_from_zero(hq, hkv, d, n, L, ctas, combine, regime):
