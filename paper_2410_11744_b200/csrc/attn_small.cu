@@ -324,7 +324,11 @@ tree_attn_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
         for (int m = 0; m < T; ++m) {
           const int pv_set = m & 1;
           if (m < 2 && qit > 0) mbar_wait(bar_ofree, (qit - 1) & 1u, abort_flag, p.status);   // first product into this accumulator
-          mbar_wait(bar_pready + 8 * stage, ph, abort_flag, p.status);
+          // V is under the TMA's own barrier, and this warp waits for it itself: that P is ready says no more than that
+          // K has landed.  V came long before P, so the two probes go out together.
+          const uint32_t got = mbar_test_wait2(bar_full + 8 * stage, ph, bar_pready + 8 * stage, ph);
+          if (!(got & 1u)) mbar_wait(bar_full + 8 * stage, ph, abort_flag, p.status);
+          if (!(got & 2u)) mbar_wait(bar_pready + 8 * stage, ph, abort_flag, p.status);
           tc_fence_after();
           const uint32_t p_lo = desc_lo(s_kv + stage * L::kStageBytes);                        // P sits where the K tile was
           const uint32_t v_lo = desc_lo(s_kv + stage * L::kStageBytes + L::kTileBytes) - (1u << 16) + ((uint32_t(L::kPanelBytes) >> 4) << 16);
