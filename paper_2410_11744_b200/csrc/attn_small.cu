@@ -377,6 +377,7 @@ tree_attn_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
       if (!seen) mbar_wait(bar_pvdone + 8 * set, uint32_t(pv_seen) & 1u, abort_flag, p.status);
       ++pv_seen;
     }
+    __syncwarp();            // (what follows, tensor-memory accesses and barriers, is the whole warp's)
     tc_fence_after();
   };
   uint32_t qit = 0;
@@ -438,6 +439,7 @@ tree_attn_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
       const uint32_t sph = uint32_t(pos / kSBufs) & 1u;
       const uint32_t got = mbar_test_wait2(bar_sfull + 8 * sb, sph, bar_pvdone + 8 * set, uint32_t(pv_seen) & 1u);
       if (!(got & 1u)) mbar_wait(bar_sfull + 8 * sb, sph, abort_flag, p.status);
+      __syncwarp();          // (the lanes' probes may differ, and the load below is one of the whole warp)
       tc_fence_after();
       if (threadIdx.x == 0 && w == item_begin && t == item.tile_begin) stamp(3);
       float s[BN / 8][4];

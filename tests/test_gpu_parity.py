@@ -309,6 +309,23 @@ def test_growing_maxima_exercise_the_lazy_rescale(rt, hq, hkv, n, L):
     run_and_check(rt, w)
 
 
+@pytest.mark.parametrize("hq,hkv,n,L,ctas", [(4, 4, 40, 500, 0), (4, 4, 40, 500, 2), (8, 1, 8, 700, 0), (32, 32, 64, 1024, 0)])
+def test_growing_maxima_at_head_dimension_64(rt, hq, hkv, n, L, ctas):
+    """As above with D = 64 and the small-tile kernel: every few tiles the wait for a set's last product is
+    followed by the rescale of its accumulator in tensor memory."""
+    rng = np.random.default_rng(hq * 1000 + n + 64)
+    w = wl.make_custom(71 + n, hq, hkv, 64, [L], [wl.greedy_tree(rng, n, 6, 0.3)])
+    pattern = np.where(rng.random(64) < 0.5, -1.0, 1.0)
+    q = pattern * (1.0 + 0.1 * rng.standard_normal((n, hq, 1))) + 0.05 * rng.standard_normal((n, hq, 64))
+    rows = w.k.shape[0]
+    ramp = (0.02 + 3.0 * np.arange(rows) / rows)[:, None, None]           # |score| grows ~ 35 log2 units over the cache
+    k = pattern * ramp + 0.05 * rng.standard_normal((rows, hkv, 64))
+    for dst, x in ((w.q, q), (w.k, k)):
+        u = np.ascontiguousarray(x, dtype=np.float32).view(np.uint32)
+        dst[...] = ((u + 0x7FFF + ((u >> 16) & 1)) >> 16).astype(np.uint16)
+    run_and_check(rt, w, regime=0, ctas=ctas)
+
+
 @pytest.mark.parametrize("n_nodes,heads", [(64, (8, 8)), (48, (32, 4)), (1024, (2, 2))])
 def test_mask_of_this_step_is_the_one_used_when_the_tree_changes(rt, n_nodes, heads):
     """The attention kernels start on the prefix tiles before the mask builder of the same step has
