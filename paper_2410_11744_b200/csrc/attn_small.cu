@@ -291,9 +291,12 @@ tree_attn_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
         mbar_wait(bar_qfull, qit & 1, abort_flag, p.status);
         for (int i = 0; i < T; ++i, ++pos) {
           const int sb = pos & (kSBufs - 1), sb_use = pos / kSBufs;
-          // (the score buffer first: it is free long before the tile is here, and a probe costs some 180 cycles)
-          if (sb_use > 0) mbar_wait(bar_sfree + 8 * sb, uint32_t(sb_use - 1) & 1u, abort_flag, p.status);
-          mbar_wait(bar_full + 8 * stage, ph, abort_flag, p.status);
+          // Which of the two comes last depends on the side that is slower, loads or softmax, and a probe costs some 180
+          // cycles, so both go out together.  (A buffer's first use: the parity that a fresh barrier has behind it.)
+          const uint32_t sf_ph = uint32_t(sb_use - 1) & 1u;
+          const uint32_t got = mbar_test_wait2(bar_sfree + 8 * sb, sf_ph, bar_full + 8 * stage, ph);
+          if (!(got & 1u)) mbar_wait(bar_sfree + 8 * sb, sf_ph, abort_flag, p.status);
+          if (!(got & 2u)) mbar_wait(bar_full + 8 * stage, ph, abort_flag, p.status);
           tc_fence_after();
           const uint32_t k_lo = desc_lo(s_kv + stage * L::kStageBytes);
 #pragma unroll
