@@ -1305,15 +1305,11 @@ size_t attn_tc_cluster_workspace_per_cta(int head_dim, int cluster_size) {
 // cluster cannot be launched at all, e.g. on a reduced share of the SMs); -1 when that cannot be asked
 // (no device).  Asked once per (device, head dimension, cluster size).
 int attn_tc_max_clusters(int head_dim, int cluster_size) {
-  static std::atomic<int> cache[DynSmemGrant::kDevices][2][4];
-  static std::atomic<bool> init{false};
+  static std::atomic<int> known[DynSmemGrant::kDevices][2][4];      // 0: not asked yet, else the answer + 1
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= DynSmemGrant::kDevices) { cudaGetLastError(); return -1; }
-  if (!init.exchange(true))
-    for (auto& d : cache) for (auto& h : d) for (auto& c : h) c.store(-2);
   const int hi = head_dim == 128 ? 0 : 1, ci = cluster_size == 8 ? 3 : cluster_size == 4 ? 2 : cluster_size == 2 ? 1 : 0;
-  int have = cache[dev][hi][ci].load();
-  if (have != -2 && have != -3) return have;           // (-3: another thread is filling the table; ask again below, harmless)
+  if (const int have = known[dev][hi][ci].load(); have > 0) return have - 1;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = unsigned(cluster_size);
@@ -1338,7 +1334,7 @@ int attn_tc_max_clusters(int head_dim, int cluster_size) {
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n, tree_attn_tc_kernel<64, false, false>, &cfg);
   }
   if (e != cudaSuccess) { cudaGetLastError(); n = 0; }
-  cache[dev][hi][ci].store(n);
+  known[dev][hi][ci].store(n + 1);
   return n;
 }
 
