@@ -52,7 +52,7 @@ struct SmemLayout {
   static constexpr int kBarOffset = kQBytes + kStages * kStageBytes;
   static constexpr int kExchMlOffset = kBarOffset + 512;  // set 1 -> set 0: (m, l) of every thread's two rows
   static constexpr int kTotal = kExchMlOffset + kSets * kComputeWarps * 32 * 16;
-  static constexpr int kTmemCols = 512;                  // one 64-column score buffer per ring stage (power of two)
+  static constexpr int kTmemCols = 512;                  // a power of two: an accumulator of D columns per warp set, four score buffers of 64
 };
 
 // Byte offset of 16-byte chunk `chunk` (0 .. D/8-1) of row `row` inside a tile stored as 64-column
@@ -111,8 +111,7 @@ __device__ __forceinline__ void tmem_ld_scores(uint32_t taddr, float (&s)[BN / 8
 // O += P V on the tensor cores as well: M = 64 rows, N = D columns, K = 64 keys in four 16-key steps.  P is a K-major
 // operand (64 rows x 64 keys of bf16 = one 128-byte row each, same layout as a Q or K panel); V is an MN-major operand (keys x
 // columns, columns contiguous) in panels of 64 columns: 8-key groups 1024 bytes apart, the next panel at the leading
-// offset.  (A product per panel reads P twice: eight layers of one 64-node tree over 1024 keys, 32 heads, 78.2 us against 76.7;
-// two of a ragged batch of 16 186.5 against 185.2.)
+// offset.  (A product per panel reads P twice: 2 % slower on one 64-node tree over 1024 keys, 32 heads.)
 template <int D>
 __host__ __device__ constexpr uint32_t idesc_pv() {
   return (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | (uint32_t(D >> 3) << 17) | (uint32_t(BM >> 4) << 24);
@@ -120,7 +119,7 @@ __host__ __device__ constexpr uint32_t idesc_pv() {
 constexpr int kSBufs = 4;                 // score buffers in tensor memory (64 columns each)
 constexpr float kRescaleThreshold = 8.f;  // log2 units: O is rescaled only when a row maximum grows by more
 
-// NJ 8-column groups of this warp's 16 accumulator rows (see tmem_ld_scores for the register layout)
+// NJ 8-column groups of this warp's 16 accumulator rows (see tmem_ld_request for the register layout)
 template <int NJ>
 __device__ __forceinline__ void tmem_ld_rows(uint32_t taddr, float (&v)[NJ][4]) {
   static_assert(NJ == 8, "64 columns at a time");
@@ -162,7 +161,7 @@ tree_attn_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
   const uint32_t s_q = smem_u32(smem);
   const uint32_t s_kv = s_q + L::kQBytes;
   const uint32_t s_bar = s_q + L::kBarOffset;
-  // barriers: full[kStages], empty[kStages], q_full, q_empty, src[8] (one per cluster peer), s_full[kStages]
+  // barriers: full[kStages] (K and V of the stage's tile), empty[kStages], q_full, q_empty, src[8] (one per cluster peer)
   const uint32_t bar_full = s_bar, bar_empty = s_bar + 8 * kStages;
   const uint32_t bar_qfull = s_bar + 16 * kStages, bar_qempty = bar_qfull + 8, bar_src = bar_qempty + 8;
   // ... s_full[4] / s_free[4] (score buffers), p_ready[kStages] (P of the stage's tile is in shared memory),
@@ -199,11 +198,9 @@ tree_attn_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
   auto item_of = [&](int w) -> WorkItem { return (w == 0 && first_here) ? first.item[blockIdx.x] : my_items[w]; };
   const int item_begin = 0;
   const int item_end = first_here ? first.item[blockIdx.x].n_in_cta : my_items[0].n_in_cta;
-  // Ring depth.  The last stage is where warp set 1 hands its partial output to set 0 (without clusters
-  // the ring is busy with the next item's tiles by then).  In cluster mode a CTA that merges (an owner)
-  // keeps the last TWO stages free for the partial rows its peers push into them, possibly while it
-  // is still streaming K/V itself, and hands over through a ring stage once the ring is idle; a CTA
-  // that does not merge receives nothing (it is the one with the most tiles).
+  // Ring depth.  In cluster mode a CTA that merges (an owner) keeps the last TWO stages free for the partial rows its
+  // peers push into them, possibly while it is still streaming K/V itself; a CTA that does not merge receives nothing
+  // (it is the one with the most tiles) and uses them all, as every CTA does without clusters.
   const bool merge_owner = p.cluster_size > 1 && ((uint32_t(first_here ? first.item[blockIdx.x].merge_owners : my_items[0].merge_owners) >> cluster_ctarank()) & 1u);
   const int n_stages = merge_owner ? kStages - 2 : kStages;
   // tensor memory: O of set 0, O of set 1 (D columns each), then the score buffers
@@ -404,8 +401,7 @@ tree_attn_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
     bool first = true;
 
     // ring position of this set's next tile, counted on: the ring's depth is not known to the compiler, and a quotient
-    // and a remainder a tile and role (here and in the issuing warps) cost 4 - 5 % of a call (64-node tree over
-    // 1024 keys, 32 heads, eight layers: 81.4 us against 78.2; ragged batch of 16, two layers: 194.5 against 184.4)
+    // and a remainder a tile and role (here and in the issuing warps) cost 4 - 5 % of a call
     int next_stage = (n_base + set) % n_stages;
     uint32_t next_ph = uint32_t((n_base + set) / n_stages) & 1u;
     for (int i = set; i < T_item; i += kSets) {
@@ -478,12 +474,11 @@ tree_attn_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
       // ---- online softmax (exp2 domain) against a LAZY reference: the accumulator lives in tensor memory, so
       //      it is rescaled only when some row's maximum has grown by more than 2^8 since the reference was
       //      set (probabilities then stay below 2^8, harmless in bf16 and fp32; the final normalisation
-      //      uses the same reference).  The warp is bound by instruction issue, so a tile that every row sees in
-      //      full (all prefix tiles but the last) has no masking, the scale (positive) goes into the
-      //      exponent's one multiply-add, and pairs of values share an instruction where one exists.  (With every
-      //      tile masked, 64-bit shifts by the lane's column, scale and reference applied apart, P stored word by
-      //      word and a probe each for S, the stage and the previous product: eight layers of one 64-node
-      //      tree over 1024 keys, 32 heads, 84.6 us against 81.2; two of a ragged batch of 16 205 against 194.)
+      //      uses the same reference).  Where tiles are there in time (one request, K and V in L2) the loop is bound by the
+      //      instructions of this warp, so a tile that every row sees in full (all prefix tiles but the last) has no
+      //      masking, the scale (positive) goes into the exponent's one multiply-add, and pairs of values share
+      //      an instruction where one exists.  (Eight layers of one 64-node tree over 1024 keys, 32 heads: 76.7 us, 84.6
+      //      before; two of a ragged batch of 16, which HBM bounds: 172.7, 205 before.)
       if (!all_visible) {
         const uint64_t a_ = vis_lo >> (2 * tig), b_ = vis_hi >> (2 * tig);     // the thread's columns at bits 8 j, 8 j + 1
         const uint32_t a2[2] = {uint32_t(a_), uint32_t(a_ >> 32)}, b2[2] = {uint32_t(b_), uint32_t(b_ >> 32)};

@@ -530,8 +530,8 @@ __device__ __forceinline__ float max3_f32(float a, float b, float c) {
 // the division by their sum takes out again; from 2^31 on an overflow (NaN, or a sum of 0).  Beyond 2^30 two fp32 scores
 // are equal or at least 2^6 apart after scaling, so every scale that is no smaller gives the same weights, and with
 // the next power of two the product, and with it m, is exact.  Maxima on the two sides of the line keep their order.
-// (Free: selects in front of the loop over a tile's scores.  A branch that rounds the products first costs
-// the tensor-core kernel 2 - 4 %, 128 scores a thread.)
+// (A few selects in front of the loop over a tile's scores: at most 0.3 % of a call.  A branch that rounds the
+// products first costs the tensor-core kernel, with 128 scores a thread, 2 - 4 %.)
 constexpr float kCoarseReference = 1073741824.f;
 __device__ __forceinline__ float scale_rounded_up(float scale) {
   return __uint_as_float((__float_as_uint(scale) + 0x7fffffu) & 0xff800000u);
