@@ -399,6 +399,7 @@ tree_attn_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
     const uint32_t t_rows = tmem_base + (uint32_t(cw * 32) << 16);         // this warp's 16 accumulator rows
     const uint32_t t_o = t_rows + uint32_t(set) * kOCols;                    // this set's output accumulator
     bool first = true;
+    float most_lo = -INFINITY, most_hi = -INFINITY;     // row maxima up to here leave the reference as it is
 
     // ring position of this set's next tile, counted on: the ring's depth is not known to the compiler, and a quotient
     // and a remainder a tile and role (here and in the issuing warps) cost 4 - 5 % of a call
@@ -507,42 +508,59 @@ tree_attn_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
         const float y_lo = __shfl_xor_sync(0xffffffffu, mx_lo, 1), y_hi = __shfl_xor_sync(0xffffffffu, mx_hi, 1);
         mx_lo = fmaxf(mx_lo, y_lo); mx_hi = fmaxf(mx_hi, y_hi);
         const float z_lo = __shfl_xor_sync(0xffffffffu, mx_lo, 2), z_hi = __shfl_xor_sync(0xffffffffu, mx_hi, 2);
-        mx_lo = scaled_maximum(fmaxf(mx_lo, z_lo), p.scale_log2e); mx_hi = scaled_maximum(fmaxf(mx_hi, z_hi), p.scale_log2e);
+        mx_lo = fmaxf(mx_lo, z_lo) * p.scale_log2e; mx_hi = fmaxf(mx_hi, z_hi) * p.scale_log2e;
       }
       const float mn_lo = fmaxf(m_lo, mx_lo), mn_hi = fmaxf(m_hi, mx_hi);
       confirm_pv_done((got & 2u) != 0u);
-      if (first) {
-        m_lo = mn_lo; m_hi = mn_hi;
-      } else if (__any_sync(0xffffffffu, mn_lo > m_lo + kRescaleThreshold || mn_hi > m_hi + kRescaleThreshold)) {
-        // O *= 2^(m - mn) for this warp's rows (every product of this set issued so far has landed)
-        const float f_lo = fast_exp2(m_lo - (mn_lo == -INFINITY ? 0.f : mn_lo));
-        const float f_hi = fast_exp2(m_hi - (mn_hi == -INFINITY ? 0.f : mn_hi));
+      bool shifted = false;             // the scores are differences from the reference already
+      if (first || __any_sync(0xffffffffu, mn_lo > most_lo || mn_hi > most_hi)) {
+        if (!first) {
+          // O *= 2^(m - mn) for this warp's rows (every product of this set issued so far has landed)
+          const float f_lo = fast_exp2(m_lo - (mn_lo == -INFINITY ? 0.f : mn_lo));
+          const float f_hi = fast_exp2(m_hi - (mn_hi == -INFINITY ? 0.f : mn_hi));
 #pragma unroll 1
-        for (int c0 = 0; c0 < D; c0 += 64) {
-          float ov[8][4];
-          tmem_ld_rows<8>(t_o + uint32_t(c0), ov);
+          for (int c0 = 0; c0 < D; c0 += 64) {
+            float ov[8][4];
+            tmem_ld_rows<8>(t_o + uint32_t(c0), ov);
 #pragma unroll
-          for (int j = 0; j < 8; ++j) { ov[j][0] *= f_lo; ov[j][1] *= f_lo; ov[j][2] *= f_hi; ov[j][3] *= f_hi; }
-          tmem_st_rows<8>(t_o + uint32_t(c0), ov);
+            for (int j = 0; j < 8; ++j) { ov[j][0] *= f_lo; ov[j][1] *= f_lo; ov[j][2] *= f_hi; ov[j][3] *= f_hi; }
+            tmem_st_rows<8>(t_o + uint32_t(c0), ov);
+          }
+          asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+          l_lo *= f_lo; l_hi *= f_hi;
         }
-        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-        l_lo *= f_lo; l_hi *= f_hi;
         m_lo = mn_lo; m_hi = mn_hi;
+        // A coarse reference (see common.cuh) has its products rounded first, in here, where a tile that leaves the
+        // references as they are never comes: such a row comes back at every tile.
+        const bool coarse_lo = reference_is_coarse(m_lo), coarse_hi = reference_is_coarse(m_hi);
+        most_lo = coarse_lo ? -INFINITY : m_lo + kRescaleThreshold;
+        most_hi = coarse_hi ? -INFINITY : m_hi + kRescaleThreshold;
+        if (__any_sync(0xffffffffu, coarse_lo || coarse_hi)) {
+          const float inv = 1.f / p.scale_log2e;          // (taken back by the multiply-add below)
+          const float r_lo = m_lo == -INFINITY ? 0.f : m_lo, r_hi = m_hi == -INFINITY ? 0.f : m_hi;
+#pragma unroll
+          for (int j = 0; j < BN / 8; ++j) {
+            s[j][0] = __fsub_rn(__fmul_rn(s[j][0], p.scale_log2e), r_lo) * inv;
+            s[j][1] = __fsub_rn(__fmul_rn(s[j][1], p.scale_log2e), r_lo) * inv;
+            s[j][2] = __fsub_rn(__fmul_rn(s[j][2], p.scale_log2e), r_hi) * inv;
+            s[j][3] = __fsub_rn(__fmul_rn(s[j][3], p.scale_log2e), r_hi) * inv;
+          }
+          shifted = true;
+        }
       }
       // A row that has seen no visible key yet keeps m = -inf; use 0 as the reference so that
       // exp2(-inf - 0) = 0 and no inf - inf appears.
-      const float ref_lo = m_lo == -INFINITY ? 0.f : m_lo;
-      const float ref_hi = m_hi == -INFINITY ? 0.f : m_hi;
-      const float scale_lo = scale_for_reference(m_lo, p.scale_log2e), scale_hi = scale_for_reference(m_hi, p.scale_log2e);
-      const uint64_t scale2_lo = pack_f32x2(scale_lo, scale_lo), scale2_hi = pack_f32x2(scale_hi, scale_hi);
+      const float ref_lo = shifted || m_lo == -INFINITY ? 0.f : m_lo;
+      const float ref_hi = shifted || m_hi == -INFINITY ? 0.f : m_hi;
+      const uint64_t scale2 = pack_f32x2(p.scale_log2e, p.scale_log2e);
       const uint64_t neg_lo = pack_f32x2(-ref_lo, -ref_lo), neg_hi = pack_f32x2(-ref_hi, -ref_hi);
       uint64_t sum2_lo = 0ull, sum2_hi = 0ull;
       uint32_t pf[BN / 8][2];
 #pragma unroll
       for (int j = 0; j < BN / 8; ++j) {
         float p0, p1, p2, p3;
-        unpack_f32x2(fma_f32x2(pack_f32x2(s[j][0], s[j][1]), scale2_lo, neg_lo), p0, p1);
-        unpack_f32x2(fma_f32x2(pack_f32x2(s[j][2], s[j][3]), scale2_hi, neg_hi), p2, p3);
+        unpack_f32x2(fma_f32x2(pack_f32x2(s[j][0], s[j][1]), scale2, neg_lo), p0, p1);
+        unpack_f32x2(fma_f32x2(pack_f32x2(s[j][2], s[j][3]), scale2, neg_hi), p2, p3);
         p0 = fast_exp2(p0); p1 = fast_exp2(p1); p2 = fast_exp2(p2); p3 = fast_exp2(p3);
         sum2_lo = add_f32x2(sum2_lo, pack_f32x2(p0, p1));
         sum2_hi = add_f32x2(sum2_hi, pack_f32x2(p2, p3));

@@ -527,12 +527,15 @@ __device__ __forceinline__ float max3_f32(float a, float b, float c) {
 }
 // A softmax weight is exp2(score * scale - m), m the row's maximum times scale, rounded.  Product and difference are ONE
 // multiply-add, which keeps what m was rounded by: up to 2^30 a factor of at most 2^32 on all of a row's weights, which
-// the division by their sum takes out again; from 2^31 on an overflow (NaN, or a sum of 0).  Beyond 2^30 two fp32 scores
-// are equal or at least 2^6 apart after scaling, so every scale that is no smaller gives the same weights, and with
-// the next power of two the product, and with it m, is exact.  Maxima on the two sides of the line keep their order.
-// (A few selects in front of the loop over a tile's scores: at most 0.3 % of a call.  A branch that rounds the
-// products first costs the tensor-core kernel, with 128 scores a thread, 2 - 4 %.)
+// the division by their sum takes out again; from 2^31 on an overflow (NaN, or a sum of 0).  Two ways around, for a
+// reference that is coarse: the small-tile kernel rounds the products first, in the branch that also rescales the output
+// (no cost to other tiles); the tensor-core kernel, where such a branch costs every call 2 - 4 % (128 scores a thread), takes
+// the next power of two as the scale, so that product and m are exact (a few selects, at most 0.3 % of a call).
+// Beyond 2^30 two fp32 scores are equal or at least 2^6 apart after scaling, so every scale that is no smaller gives the
+// same weights, and maxima on the two sides of the line keep their order; what it lacks is the last factor
+// of 2 below fp32's end, where a given scale above 1 / log2(e) can take the raised product over it.
 constexpr float kCoarseReference = 1073741824.f;
+__device__ __forceinline__ bool reference_is_coarse(float m) { return fabsf(m) > kCoarseReference && m != -INFINITY; }
 __device__ __forceinline__ float scale_rounded_up(float scale) {
   return __uint_as_float((__float_as_uint(scale) + 0x7fffffu) & 0xff800000u);
 }

@@ -46,3 +46,37 @@ def test_scores_far_from_zero(hq, hkv, d, n, L, ctas, combine, regime):
             assert status == 0 and np.isfinite(got).all(), (log2_score, growing)
             err = np.abs(got - ref)
             assert err.max() <= MAX_ABS and err.mean() <= MEAN_ABS, (log2_score, growing, err.max(), err.mean())
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_scores_at_the_end_of_the_range(d):
+    """Small-tile kernel, a given scale above 1 / log2(e): scaled scores up to a tenth below 2^128, all of them finite."""
+    import torch
+    from paper_2410_11744_b200 import binding as B, build
+    build.build()
+    L, n, H, scale = 8, 5, 4, 40.0
+    rng = np.random.default_rng(d)
+    w = wl.make_custom(62, H, H, d, [L], [wl.greedy_tree(rng, n, 3, 0.3)])
+    sign = np.where(rng.random(d) < 0.5, -1.0, 1.0)
+    side = np.where(rng.random((n, H, 1)) < 0.5, -1.0, 1.0)
+    a = 1 + rng.permutation(L + n) / 128
+    w.k[...] = _bits(sign * a[:, None, None] * np.ones((1, H, 1)))
+    w.q[...] = _bits(sign * side * 2.0 ** 122 / d)              # scores 2^122 * a, times 40 log2(e) = 2^127.85 * a
+    assert 2.0 ** 122 * a.max() * scale * np.log2(np.e) < 2.0 ** 128
+    ref = orc.tree_attention_ragged(w.q, w.k, w.v, w.prefix_len, w.n_nodes, w.kv_row_offset, w.parents, scale=scale)
+    t = lambda x, kind=torch.bfloat16: torch.from_numpy(np.ascontiguousarray(x)).to("cuda:0").view(kind)
+    q, k, v = t(w.q.view(np.int16)), t(w.k.view(np.int16)), t(w.v.view(np.int16))
+    W = B.dyspec_words_per_row(n)
+    B.dyspec_set_tuning(0, 0, 2)
+    try:
+        plan = B.Plan(H, H, d, w.prefix_len, w.n_nodes, w.kv_row_offset, L + n, W, scale)
+    finally:
+        B.dyspec_set_tuning(-1, 0, 2)
+    bits, depths, status = (torch.zeros(s, dtype=torch.int32, device="cuda:0") for s in ((n, W), (n,), (1,)))
+    out = torch.zeros_like(q)
+    workspace = torch.zeros(max(256, plan.workspace_bytes()), dtype=torch.uint8, device="cuda:0")
+    B.dyspec_plan_build_tree_mask(plan, t(w.parents[0], torch.int32), bits, depths, status)
+    B.dyspec_tree_attention_ragged(plan, q, k, v, bits, out, workspace, None, status)
+    torch.cuda.synchronize()
+    err = np.abs(out.float().cpu().numpy() - ref)
+    assert int(status.item()) == 0 and err.max() <= MAX_ABS and err.mean() <= MEAN_ABS, (err.max(), err.mean())
