@@ -478,8 +478,8 @@ tree_attn_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
       //      uses the same reference).  Where tiles are there in time (one request, K and V in L2) the loop is bound by the
       //      instructions of this warp, so a tile that every row sees in full (all prefix tiles but the last) has no
       //      masking, the scale (positive) goes into the exponent's one multiply-add, and pairs of values share
-      //      an instruction where one exists.  (Eight layers of one 64-node tree over 1024 keys, 32 heads: 76.7 us, 84.6
-      //      before; two of a ragged batch of 16, which HBM bounds: 172.7, 205 before.)
+      //      an instruction where one exists.  (Eight layers of one 64-node tree over 1024 keys, 32 heads: 76.5 us, 84.6
+      //      before; two of a ragged batch of 16, which HBM bounds: 173 - 176, 205 before.)
       if (!all_visible) {
         const uint64_t a_ = vis_lo >> (2 * tig), b_ = vis_hi >> (2 * tig);     // the thread's columns at bits 8 j, 8 j + 1
         const uint32_t a2[2] = {uint32_t(a_), uint32_t(a_ >> 32)}, b2[2] = {uint32_t(b_), uint32_t(b_ >> 32)};
