@@ -530,7 +530,7 @@ __device__ __forceinline__ float max3_f32(float a, float b, float c) {
 // the division by their sum takes out again; from 2^31 on an overflow (NaN, or a sum of 0).  Two ways around, for a
 // reference that is coarse: the small-tile kernel rounds the products first, in the branch that also rescales the output
 // (no cost to other tiles); the tensor-core kernel, where such a branch costs every call 2 - 4 % (128 scores a thread), takes
-// the next power of two as the scale, so that product and m are exact (a few selects, at most 0.3 % of a call).
+// the next power of two as the scale, so that product and m are exact (a few selects, 0 - 0.8 % of a call).
 // Beyond 2^30 two fp32 scores are equal or at least 2^6 apart after scaling, so every scale that is no smaller gives the
 // same weights, and maxima on the two sides of the line keep their order; what it lacks is the last factor
 // of 2 below fp32's end, where a given scale above 1 / log2(e) can take the raised product over it.
